@@ -219,43 +219,53 @@ struct Acc<float> {
     lo += e + e2;
     hi = t;
   }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ df total() const {   // renormalised pair
+    const float h = hi + lo;
+    return df(h, lo - (h - hi));
+  }
 };
 
 template <>
 struct Acc<df> {
   df s = df(0.f, 0.f);
   __device__ __forceinline__ void add_prod(df a, df b) { s = s + a * b; }
-  __device__ __forceinline__ double value() const { return (double)s.hi + (double)s.lo; }
+  __device__ __forceinline__ df total() const { return s; }
 };
 
 template <>
 struct Acc<double> {
   double s = 0.0;
   __device__ __forceinline__ void add_prod(double a, double b) { s = fma(a, b, s); }
-  __device__ __forceinline__ double value() const { return s; }
+  __device__ __forceinline__ double total() const { return s; }
 };
 
-// Block-wide FP64 sum (all threads call; result valid in thread 0).
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // lanes present in this warp (the last warp may be partial)
-  const int nl = min(32, (int)blockDim.x - (wid << 5));
-  const unsigned mask = nl == 32 ? 0xffffffffu : ((1u << nl) - 1u);
-#pragma unroll
+// Partial sums in transit between threads: FP32 and double-float passes carry
+// pairs (hi, lo), FP64 passes doubles.
+__device__ __forceinline__ df shfl_down_sum(unsigned mask, df v, int o) {
+  return df(__shfl_down_sync(mask, v.hi, o), __shfl_down_sync(mask, v.lo, o));
+}
+__device__ __forceinline__ double shfl_down_sum(unsigned mask, double v, int o) {
+  return __shfl_down_sync(mask, v, o);
+}
+__device__ __forceinline__ double sum_value(df v) { return (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ double sum_value(double v) { return v; }
+// A pair whose high part is this large could overflow FP32 in the sum of a
+// CTA (at most 1024 threads); such sums go through FP64.
+__device__ __forceinline__ bool sum_large(df v) { return !(fabsf(v.hi) < 1e34f); }
+__device__ __forceinline__ bool sum_large(double) { return false; }
+
+// Sum over the segments of `len` consecutive lanes of a warp (len <= 32, any
+// value; nl lanes present): the first lane of each segment gets its segment's
+// sum, added pairwise in a fixed order.
+template <typename V>
+__device__ __forceinline__ V segment_sum(V v, unsigned mask, int lane, int nl, int len) {
+  const int in = lane % len;
   for (int o = 16; o > 0; o >>= 1) {
-    const double t = __shfl_down_sync(mask, v, o);
-    if (lane + o < nl) v += t;
+    if (o >= len) continue;
+    const V t = shfl_down_sum(mask, v, o);
+    if (in + o < len && lane + o < nl) v = v + t;
   }
-  __syncthreads();
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    for (int w = 0; w < nw; ++w) s += sh[w];
-  }
-  return s;
+  return v;
 }
 
 // CG coefficient record for the Lanczos estimate (Sect. 6.4): alpha_j when
@@ -287,6 +297,7 @@ __device__ __forceinline__ void scalar_update(int sop, CgState* st, double sum) 
       if (sop == SC_BB_RHO) {   // plain CG: z = r, rho = ||r||^2, p = r
         st->rho = sum;
         st->beta = 0.0;
+        st->beta_f = 0.f;
         st->first = 0;
       }
       break;
@@ -297,6 +308,7 @@ __device__ __forceinline__ void scalar_update(int sop, CgState* st, double sum) 
         st->done = 1;
       } else {
         st->alpha = st->rho / sum;
+        st->alpha_f = (float)st->alpha;
         record_alpha(st);
       }
       break;
@@ -315,6 +327,7 @@ __device__ __forceinline__ void scalar_update(int sop, CgState* st, double sum) 
         st->done = 1;
       } else if (sop == SC_RCHECK_BETA) {
         st->beta = sum / st->rho;
+        st->beta_f = (float)st->beta;
         st->rho = sum;
         record_beta(st);
       }
@@ -328,8 +341,10 @@ __device__ __forceinline__ void scalar_update(int sop, CgState* st, double sum) 
         st->first = 0;
         st->rho = sum;
         st->beta = 0.0;
+        st->beta_f = 0.f;
       } else {
         st->beta = sum / st->rho;
+        st->beta_f = (float)st->beta;
         st->rho = sum;
         record_beta(st);
       }
@@ -398,26 +413,99 @@ __device__ __forceinline__ bool skip_instance(int mode, const CgState* st) {
   return done != 0 || *(volatile const int*)&st->upd == 0;
 }
 
-// Writes this CTA's partial; the last CTA of the instance sums all partials in
-// order and runs the scalar update.  Called by all threads of the CTA.
-__device__ __forceinline__ void grid_reduce(double v, double* sh, double* partial,
-                                            CgState* st, int sop, int ncta, int cta) {
-  double s = block_sum(v, sh);
+// CG scalars in a pass's element type.  The FP32 copies are kept in the state:
+// a double -> float conversion runs on the FP64 pipe, where one warp
+// instruction takes 64 cycles (19 per SM with every scheduler queueing), and
+// every warp of a source pass needs one before its arithmetic.
+template <typename T>
+__device__ __forceinline__ T cg_alpha(const CgState* st) { return (T)st->alpha; }
+template <>
+__device__ __forceinline__ float cg_alpha<float>(const CgState* st) { return st->alpha_f; }
+template <typename T>
+__device__ __forceinline__ T cg_beta(const CgState* st) { return (T)st->beta; }
+template <>
+__device__ __forceinline__ float cg_beta<float>(const CgState* st) { return st->beta_f; }
+
+// Reduction of a pass: every `seg` consecutive threads of a CTA give one
+// partial sum (seg divides the CTA; fewer than 32 threads or whole warps), and
+// the last CTA of the instance adds all partials and runs the scalar update.
+// Called by all threads of the CTA.
+//
+// Every order is fixed and, for a given seg, independent of how many segments
+// a CTA holds, so results are reproducible and do not depend on the CTA shape.
+// What bounds it is the FP64 pipe (64 cycles per dependent instruction): the
+// sums inside a CTA are pairs of FP32 values added with TwoSum (about 2^-47
+// of the sum per addition, below the 2^-44 of a thread's own compensated
+// sum), only a segment's total becomes a double, and the last CTA adds the
+// partials on 32 lanes in parallel.  Measured against shuffles and sums in
+// FP64 with one thread adding the partials (1024 of them at 4096^2, 32 us):
+// 4096^2, one map, sink 104 -> 59 us, r-update 124 -> 76 us; an iteration of
+// 1024^2 94.5 -> 84 us; 600 x 7000 x 4, r-update 106 -> 93 us.
+template <typename V>
+__device__ __forceinline__ void grid_reduce(V v, double* sh, double* partial, CgState* st,
+                                            int sop, int ncta, int cta, int seg) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int nthr = blockDim.x, nseg = nthr / seg, nw = (nthr + 31) >> 5;
+  const int nl = min(32, nthr - (wid << 5));   // lanes of this warp
+  const unsigned mask = nl == 32 ? 0xffffffffu : ((1u << nl) - 1u);
+  double* out = partial + (long long)cta * nseg;
   __shared__ bool last;
-  if (threadIdx.x == 0) {
-    partial[cta] = s;
-    __threadfence();
-    unsigned int t = atomicAdd(&st->ticket, 1u);
+  if (seg <= 32) {
+    V w = segment_sum(v, mask, lane, nl, seg);
+    double s = sum_value(w);
+    if (__any_sync(mask, sum_large(w))) s = segment_sum(sum_value(v), mask, lane, nl, seg);
+    if (lane % seg == 0) out[tid / seg] = s;
+  } else {
+    V* shv = reinterpret_cast<V*>(sh);
+    __shared__ int large;
+    if (tid == 0) large = 0;
+    V w = segment_sum(v, mask, lane, nl, 32);
+    __syncthreads();   // (sh may still be read by the previous use)
+    if (lane == 0) {
+      shv[wid] = w;
+      if (sum_large(w)) large = 1;
+    }
+    __syncthreads();
+    const int wps = seg >> 5;   // warps per segment
+    if (large) {                // uniform over the CTA; out of the FP32 range: in FP64
+      const double d = segment_sum(sum_value(v), mask, lane, nl, 32);
+      __syncthreads();
+      if (lane == 0) sh[wid] = d;
+      __syncthreads();
+      if (wid == 0) {
+        const double t = segment_sum(lane < nw ? sh[lane] : 0.0, mask, lane, min(nw, nl), wps);
+        if (lane < nw && lane % wps == 0) out[lane / wps] = t;
+      }
+    } else if (wid == 0) {
+      const V t = segment_sum(lane < nw ? shv[lane] : V(0.0), mask, lane, min(nw, nl), wps);
+      if (lane < nw && lane % wps == 0) out[lane / wps] = sum_value(t);
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    __threadfence();   // the CTA's partials (ordered before it by the barrier)
+    const unsigned int t = atomicAdd(&st->ticket, 1u);
     last = (t == (unsigned int)(ncta - 1));
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
-    __threadfence();
-    double tot = 0.0;
-    volatile double* vp = partial;
-    for (int c = 0; c < ncta; ++c) tot += vp[c];
+  if (!last || wid > 0) return;
+  __threadfence();
+  // 32 fixed lanes (a CTA may have fewer threads), then their pairwise sum
+  const int np = ncta * nseg, nt = min(nthr, 32);
+  for (int l = lane; l < 32; l += nt) {
+    double a = 0.0;
+#pragma unroll 8
+    for (int c = l; c < np; c += 32) a += __ldcg(partial + c);
+    sh[l] = a;
+  }
+  __syncwarp(mask);
+  for (int o = 16; o > 0; o >>= 1) {
+    for (int l = lane; l < o; l += nt) sh[l] += sh[l + o];
+    __syncwarp(mask);
+  }
+  if (tid == 0) {
     st->ticket = 0u;
-    scalar_update(sop, st, tot);
+    scalar_update(sop, st, sh[0]);
   }
 }
 

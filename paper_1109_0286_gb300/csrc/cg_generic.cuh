@@ -462,7 +462,7 @@ __device__ __forceinline__ void sink_op(const InstDesc<T>& I, const Opnd& o, con
     st_map_pair<T>(I.out + pix, m0 ? (T)0 : x[0] - a0, m1 ? (T)0 : x[1] - a1);
     st_pair(I.y + pix, m0 ? x[0] : a0, m1 ? x[1] : a1);
   } else if constexpr (OP == OP_RELAX) {
-    const T step = (T)I.st->alpha;
+    const T step = cg_alpha<T>(I.st);
     a0 = m0 ? a0 : (T)0;
     a1 = m1 ? a1 : (T)0;
     st_pair(I.w + pix, x[0] - step * a0, x[1] - step * a1);
@@ -677,7 +677,8 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
       }
     }
   } else {
-    const T alpha = (T)I.st->alpha, beta = (T)I.st->beta;
+    const T alpha = a.op == OP_R_UPD ? cg_alpha<T>(I.st) : (T)0;
+    const T beta = a.op == OP_P_UPD_Z || a.op == OP_P_UPD_R ? cg_beta<T>(I.st) : (T)0;
 #define CGF_SRC(OPC) gen::src_rows<T, OPC, V>(I, pix0, a.nx, nv, Z, L, t, nt, alpha, beta, acc)
     switch (a.op) {
       case OP_R_UPD: CGF_SRC(OP_R_UPD); break;
@@ -704,7 +705,7 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
   }
 
   if (a.sop != SC_NONE)
-    grid_reduce(acc.value(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x);
+    grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, nt);
 }
 
 // ----------------------------------------------------------------- column pass

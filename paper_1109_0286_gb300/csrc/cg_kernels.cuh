@@ -18,6 +18,10 @@ namespace cgf {
 // of 64 per thread at two 512-thread CTAs per SM).
 constexpr int kSrcChunk = 4, kSrcChunkWide = 2, kSinkChunk = 4;
 
+// Rows per partial sum of a row pass (fewer if the CTA holds fewer), so that
+// the sums do not depend on the CTA height.
+constexpr int kRedRows = 4;
+
 template <typename T> struct KCfg;
 template <> struct KCfg<float> { static constexpr int kMaxThreads = 1024; };
 template <> struct KCfg<double> { static constexpr int kMaxThreads = 512; };
@@ -238,7 +242,7 @@ __device__ __forceinline__ void sink_fill(const InstDesc<T>& I, const uint2* mwr
         st_map_pair<T>(I.out + rowpix + 2 * j, m0 ? (T)0 : x0[e] - a0, m1 ? (T)0 : x1[e] - a1);
         st_pair(I.y + rowpix + 2 * j, m0 ? x0[e] : a0, m1 ? x1[e] : a1);
       } else if constexpr (OP == OP_RELAX) {
-        const T step = (T)I.st->alpha;
+        const T step = cg_alpha<T>(I.st);
         a0 = m0 ? a0 : (T)0;
         a1 = m1 ? a1 : (T)0;
         st_pair(I.w + rowpix + 2 * j, x0[e] - step * a0, x1[e] - step * a1);
@@ -400,7 +404,8 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
   } else {
     __syncthreads();   // mask words
     if (threadIdx.x == 0) prefetch_compact(I, a.op, mws, rows * TT);
-    const T alpha = (T)I.st->alpha, beta = (T)I.st->beta;
+    const T alpha = a.op == OP_R_UPD ? cg_alpha<T>(I.st) : (T)0;
+    const T beta = a.op == OP_P_UPD_Z || a.op == OP_P_UPD_R ? cg_beta<T>(I.st) : (T)0;
     switch (a.op) {
       case OP_R_UPD: src_fill<T, TT, OP_R_UPD>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
       case OP_P_UPD_Z:
@@ -460,7 +465,8 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
   }
 
   if (a.sop != SC_NONE)
-    grid_reduce(acc.value(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x);
+    grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x,
+                min(rows, kRedRows) * TT);
 }
 
 // ----------------------------------------------------------------- column pass
@@ -642,7 +648,7 @@ k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
   const long long gstride = (long long)gridDim.x * blockDim.x;
   if (a.op == VOP_UPDATE || a.op == VOP_ZERO_UP) {
     // compact CG vectors: one element per masked pixel
-    const T alpha = (T)I.st->alpha;
+    const T alpha = cg_alpha<T>(I.st);
     for (long long i = gid; i < I.nvec; i += gstride) {
       if (a.op == VOP_ZERO_UP) {
         I.u[i] = (T)0;
@@ -753,7 +759,7 @@ k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
     }
   }
   if (a.sop != SC_NONE)
-    grid_reduce(acc.value(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x);
+    grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, blockDim.x);
 }
 
 // ----------------------------------------------------------------- band products

@@ -28,6 +28,7 @@ struct CgState {
   double rho;      // r^T z of the current iterate
   double alpha;    // step length
   double beta;     // direction update
+  float alpha_f, beta_f;   // alpha, beta rounded to FP32 (the FP32 passes)
   double bb;       // ||b||^2
   double rr;       // ||r||^2 after the last update
   double tol2;     // tol^2 (stop when rr <= tol2 * bb)

@@ -259,6 +259,7 @@ __global__ void k_inner_reset(const InstDesc<float>* lo, const InstDesc<df>* hi,
   a.first = 1;
   a.ticket = 0;
   a.alpha = a.beta = 0.0;
+  a.alpha_f = a.beta_f = 0.f;
   a.max_iter = max_iter;
   if (g.done) {
     a.done = 1;
@@ -1601,7 +1602,10 @@ fill_status fill_ml(fill_plan* p, const void* d, long long d_stride, double tol,
 namespace {
 __global__ void k_set_step(CgState* const* sts, int n, double step) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) sts[i]->alpha = step;
+  if (i < n) {
+    sts[i]->alpha = step;
+    sts[i]->alpha_f = (float)step;
+  }
 }
 
 // Kernel relaxation (Sect. 5, eq. Algo): w_M <- (K * w)_M = w_M - (C^-1 w)_M / a,
