@@ -1,17 +1,23 @@
 // Register-resident complex FFT of length L = 2^LOG_L (16 <= L <= 8192) by a
-// group of L/16 threads that each hold 16 elements.
+// group of L/E threads that each hold E = 2^LE elements (E = 4, 8 or 16).
 //
 // Stockham auto-sort formulation: a stage of radix R after sub-transforms of
 // size Ns reads element j + r L/R, multiplies it by W_{Ns R}^{(j mod Ns) r},
 // applies a length-R DFT and writes element (j div Ns) Ns R + (j mod Ns) + r Ns.
-// The plan is one leading stage of radix 2^(LOG_L mod 4) (if nonzero) and then
-// radix-16 stages.  On entry thread t holds x[t + e L/16] in v[e]; on exit it
-// holds X[t + e L/16] -- the same positions -- so a forward transform, a
+// The plan is one leading stage of radix 2^(LOG_L mod LE) (if nonzero) and then
+// radix-E stages.  On entry thread t holds x[t + e L/E] in v[e]; on exit it
+// holds X[t + e L/E] -- the same positions -- so a forward transform, a
 // diagonal multiply and an inverse transform chain without a shared-memory
-// round trip.  Between stages data goes through shared memory (XBuf).  A
-// radix-16 stage needs W^(jm r), r = 1..15: fifteen loads from its own
-// table of correctly rounded values (stw_* in cg_types.h), or three master
-// table entries and complex products (TAB = false).
+// round trip.  Between stages data goes through shared memory (XBuf).  The
+// twiddles W^(jm r), r = 1..E-1, of a stage come from the stage's own table of
+// correctly rounded values (stw_* in cg_types.h), or (E = 16 columns in FP32)
+// from three master table entries and complex products (TAB = false).
+//
+// E trades the exchanges against the length of a thread's instruction chain:
+// E = 16 for the large FP32 and double-float grids, which fill the chip and
+// are bound by issue and shared-memory traffic; E = 8 for small ones, where a
+// pass is one wave and its duration is the latency of one thread; E = 4 in
+// FP64, where an instruction occupies the FP64 pipe for 64 cycles per warp.
 #pragma once
 #include "cg_common.cuh"
 
@@ -168,8 +174,10 @@ __device__ __forceinline__ void dft_small(cx<T> (&u)[R]) {
     dft2<T, INV>(u[0], u[1]);
   } else if constexpr (R == 4) {
     dft4<T, INV>(u[0], u[1], u[2], u[3]);
-  } else {
+  } else if constexpr (R == 8) {
     dft8<T, INV>(u);
+  } else {
+    dft16<T, INV>(u);
   }
 }
 
@@ -243,18 +251,19 @@ struct XBar {
 
 // TAB: twiddles from the per-stage tables (the row passes: 5-11% faster at
 // 4096^2), else from three entries of the master table and complex products
-// (the column passes: the tables' loads raise their register pressure into
-// spills, 21% slower).
-template <typename T, int LOG_L, bool INV, bool TAB = true, typename XB>
-__device__ __forceinline__ void fft_regs(cx<T> (&v)[16], const XB& xb, int tid,
+// (the E = 16 FP32 column passes: the tables' loads raise their register
+// pressure into spills, 21% slower).
+template <typename T, int LOG_L, int LE, bool INV, bool TAB = true, typename XB>
+__device__ __forceinline__ void fft_regs(cx<T> (&v)[1 << LE], const XB& xb, int tid,
                                          const T* __restrict__ tw, XBar first = XBar{0, 0},
                                          XBar bar = XBar{0, 0}) {
-  constexpr int TT = (1 << LOG_L) / 16;
-  constexpr int S16 = LOG_L / 4;
-  constexpr int REM = LOG_L % 4;
+  static_assert(TAB || LE == 4, "twiddle products are written for radix 16");
+  constexpr int E = 1 << LE, TT = (1 << LOG_L) / E;
+  constexpr int SE = LOG_L / LE;
+  constexpr int REM = LOG_L % LE;
   constexpr int NS0 = REM > 0 ? (1 << REM) : 1;
   if constexpr (REM > 0) {
-    constexpr int R0 = 1 << REM, NB = 16 / R0;
+    constexpr int R0 = 1 << REM, NB = E / R0;
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       cx<T> u[R0];
@@ -273,35 +282,35 @@ __device__ __forceinline__ void fft_regs(cx<T> (&v)[16], const XB& xb, int tid,
       }
   }
 #pragma unroll
-  for (int s = 0; s < S16; ++s) {
-    int ns = NS0;
-#pragma unroll
-    for (int t = 0; t < s; ++t) ns *= 16;
+  for (int s = 0; s < SE; ++s) {
+    const int ns = NS0 << (LE * s);
     const bool first_stage = (REM == 0) && (s == 0);
-    const bool last = (s == S16 - 1);
+    const bool last = (s == SE - 1);
     if (!first_stage) {
       bar.sync();
 #pragma unroll
-      for (int e = 0; e < 16; ++e) v[e] = xb.ld(tid + e * TT);
+      for (int e = 0; e < E; ++e) v[e] = xb.ld(tid + e * TT);
       const int jm = tid & (ns - 1);
-      // W_{16 ns}^(jm r), r = 1..15: correctly rounded entries of the stage's
+      // W_{E ns}^(jm r), r = 1..E-1: correctly rounded entries of the stage's
       // table ([r - 1][jm]; consecutive jm of a warp read consecutive entries)
       if constexpr (TAB) {
-        // Loaded in three groups of five, each applied before the next group is
-        // issued (the empty asm with a memory clobber keeps the compiler from
-        // hoisting all fifteen loads, which would need 30 more registers).
-        const T* ts = tw + 2 * (kLmax + stw_base(LOG_L) + stw_stage_off(LOG_L, s) + jm);
+        const T* ts = tw + 2 * (kLmax + stw_base(LE, LOG_L) + stw_stage_off(LE, LOG_L, s) + jm);
+        // E = 16: loaded in three groups of five, each applied before the next
+        // group is issued (the empty asm with a memory clobber keeps the
+        // compiler from hoisting all fifteen loads, which would need 30 more
+        // registers).
+        constexpr int G = LE == 4 ? 3 : 1, K = (E - 1) / G;
 #pragma unroll
-        for (int g = 0; g < 3; ++g) {
-          cx<T> w[5];
+        for (int g = 0; g < G; ++g) {
+          cx<T> w[K];
 #pragma unroll
-          for (int k = 0; k < 5; ++k) w[k] = ldg_cx<T>(ts + 2 * (5 * g + k) * ns);
+          for (int k = 0; k < K; ++k) w[k] = ldg_cx<T>(ts + 2 * (K * g + k) * ns);
 #pragma unroll
-          for (int k = 0; k < 5; ++k) {
-            const int r = 5 * g + k + 1;
+          for (int k = 0; k < K; ++k) {
+            const int r = K * g + k + 1;
             v[r] = INV ? cmulc(v[r], w[k]) : cmul(v[r], w[k]);
           }
-          asm volatile("" ::: "memory");
+          if (G > 1) asm volatile("" ::: "memory");
         }
       } else {
         // W^(jm r) from three master-table entries (W^jm, W^4jm, W^8jm) and at
@@ -322,16 +331,16 @@ __device__ __forceinline__ void fft_regs(cx<T> (&v)[16], const XB& xb, int tid,
         for (int r = 1; r < 16; ++r) v[r] = INV ? cmulc(v[r], w[r]) : cmul(v[r], w[r]);
       }
     }
-    dft16<T, INV>(v);
+    dft_small<T, E, INV>(v);
     if (!last) {
       if (REM == 0 && s == 0)
         first.sync();
       else
         bar.sync();
       const int jm = tid & (ns - 1);
-      const int base = (tid - jm) * 16 + jm;
+      const int base = (tid - jm) * E + jm;
 #pragma unroll
-      for (int r = 0; r < 16; ++r) xb.st(base + r * ns, v[r]);
+      for (int r = 0; r < E; ++r) xb.st(base + r * ns, v[r]);
     }
   }
 }

@@ -10,13 +10,18 @@
 // projections P_x, the white-noise draw, the CG vector updates and the inner
 // products -- is fused into the row passes.
 #pragma once
+#include <type_traits>
+
 #include "cg_async.cuh"
 #include "cg_fft.cuh"
 
 namespace cgf {
-// Pixel pairs whose loads a source / sink issues together (register budget
-// of 64 per thread at two 512-thread CTAs per SM).
-constexpr int kSrcChunk = 4, kSrcChunkWide = 2, kSinkChunk = 4;
+// Pixel pairs whose loads a source / sink issues together: with 16 elements per
+// thread, a register budget of 64 (two 512-thread CTAs per SM); the smaller
+// kernels have the registers for all their loads at once.
+template <int E> CGF_HD constexpr int src_chunk() { return 4; }
+template <int E> CGF_HD constexpr int src_chunk_wide() { return E == 16 ? 2 : 4; }
+template <int E> CGF_HD constexpr int sink_chunk() { return 4; }
 
 // Rows per partial sum of a row pass (fewer if the CTA holds fewer), so that
 // the sums do not depend on the CTA height.
@@ -111,12 +116,12 @@ __device__ __forceinline__ void prefetch_compact(const InstDesc<T>& I, int op, c
 // values fed to the forward transform.  One instantiation per op: a chunk of
 // CK pixel pairs issues all its loads (indices come from shared memory, so
 // they do not wait on a global load) before its arithmetic and stores.
-template <typename T, int TT, int OP>
+template <typename T, int TT, int E, int OP>
 __device__ __forceinline__ void src_fill(const InstDesc<T>& I, const uint2* mwr, int rowpix,
-                                         int tid, T alpha, T beta, cx<T> (&v)[16], Acc<T>& acc) {
-  constexpr int CK = (OP == OP_R_UPD || OP == OP_U64_UPD) ? kSrcChunkWide : kSrcChunk;
+                                         int tid, T alpha, T beta, cx<T> (&v)[E], Acc<T>& acc) {
+  constexpr int CK = (OP == OP_R_UPD || OP == OP_U64_UPD) ? src_chunk_wide<E>() : src_chunk<E>();
 #pragma unroll
-  for (int h = 0; h < 16; h += CK) {
+  for (int h = 0; h < E; h += CK) {
     PairIdx q[CK];
     T x0[CK], x1[CK], y0[CK], y1[CK], z0[CK], z1[CK], w0[CK], w1[CK];
 #pragma unroll
@@ -187,13 +192,13 @@ __device__ __forceinline__ void src_fill(const InstDesc<T>& I, const uint2* mwr,
 // ----------------------------------------------------------------- sinks
 // A sink consumes the inverse transform's row values v[e] (pairs j = tid + e
 // TT): projection, stores and the inner product of its op.
-template <typename T, int TT, int OP>
+template <typename T, int TT, int E, int OP>
 __device__ __forceinline__ void sink_fill(const InstDesc<T>& I, const uint2* mwr, int rowpix,
-                                          int tid, const cx<T> (&v)[16], Acc<T>& acc,
+                                          int tid, const cx<T> (&v)[E], Acc<T>& acc,
                                           int param = 0) {
-  constexpr int CK = kSinkChunk;
+  constexpr int CK = sink_chunk<E>();
 #pragma unroll
-  for (int h = 0; h < 16; h += CK) {
+  for (int h = 0; h < E; h += CK) {
     PairIdx q[CK];
     T x0[CK], x1[CK];
 #pragma unroll
@@ -263,11 +268,11 @@ __device__ __forceinline__ void sink_fill(const InstDesc<T>& I, const uint2* mwr
 
 // Middle of a chain (between the inverse and the forward row transform):
 // P_x (OP_MASK), or y = v and v = (d - y) on U, 0 on M (OP_Y_W).
-template <typename T, int TT, int OP>
+template <typename T, int TT, int E, int OP>
 __device__ __forceinline__ void mid_fill(const InstDesc<T>& I, const uint2* mwr, int rowpix,
-                                         int tid, cx<T> (&v)[16]) {
+                                         int tid, cx<T> (&v)[E]) {
 #pragma unroll
-  for (int e = 0; e < 16; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int j = tid + e * TT;
     bool o0, o1;
     observed_at(mwr, j, o0, o1);
@@ -285,10 +290,10 @@ __device__ __forceinline__ void mid_fill(const InstDesc<T>& I, const uint2* mwr,
 }
 
 // ----------------------------------------------------------------- row pass
-// CTA = `rows` consecutive grid rows, L/16 threads per row; blockIdx.y is the
+// CTA = `rows` consecutive grid rows, L/E threads per row; blockIdx.y is the
 // instance.  Shared memory: per-row FFT exchange areas, aliased with the
 // transposed tile [(L+1) x rows] used for the spectrum load / store,
-// then the rows' mask words (nx/32 = L/16 per row: one per thread).
+// then the rows' mask words (nx/32 = L/16 per row).
 // XI: the source is the seed's white noise (kept out of the other source
 // kernels, whose register allocation it would otherwise burden).
 template <typename T>
@@ -301,7 +306,8 @@ __host__ __device__ __forceinline__ size_t row_main_bytes(int log_l, int rows) {
 template <typename T, int LOG_L, bool IN_SPEC, bool OUT_SPEC, bool XI = false>
 __global__ void __launch_bounds__(KCfg<T>::kMaxThreads)
 k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw) {
-  constexpr int L = 1 << LOG_L, TT = L / 16, PADL = L + L / 16 + 1;
+  constexpr int LE = row_le<T>(LOG_L), E = 1 << LE;
+  constexpr int L = 1 << LOG_L, TT = L / E, NW = L / 16, PADL = L + L / 16 + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
   __shared__ double red[32];
@@ -321,43 +327,46 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
   const int gs = lr < 4 ? 4 - lr : 0;
   auto tix = [&](int k, int r) { return (k << lr) + (r ^ ((k >> gs) & (rows - 1))); };
   uint2* mws = reinterpret_cast<uint2*>(smem_raw + row_main_bytes<T>(LOG_L, rows));
-  const uint2* mwr = mws + row * TT;            // this row's mask words
+  const uint2* mwr = mws + row * NW;            // this row's mask words
   constexpr int TWS = kLmax / (2 * L);          // W_{nx}^k = table[k * TWS]
   const int rowpix = y * a.nx;
-  // tile element (kk + i TT, rr) for i = 0..15 belongs to thread (kk, rr); the
+  // tile element (kk + i TT, rr) for i = 0..E-1 belongs to thread (kk, rr); the
   // Nyquist row k = L to threads 0..rows-1
   const int rr = threadIdx.x & (rows - 1), kk = threadIdx.x >> lr;
   const size_t tstep = 2 * (size_t)TT * ny;
-  // From L = 512 on, TT is a multiple of 2^max(lr, 4) (rows * TT <= 1024), so
+  // With TT >= 32, TT is a multiple of 2^max(lr, 4) (rows * TT <= 1024), so
   // adding multiples of TT to k leaves the swizzle bits g(k) unchanged: a
   // thread's tile indices for k0 + i TT are one base plus i (TT rows).
-  constexpr bool HOIST = LOG_L >= 9;
+  constexpr bool HOIST = TT >= 32;
   const int ts = TT << lr;
   const XBar cta{0, 0}, rbar = XBar::make(TT, rows, row);   // CTA / this row's barrier
-  cx<T> v[16];
+  cx<T> v[E];
   Acc<T> acc;
 
-  if constexpr (!XI) mws[threadIdx.x] = __ldg(I.mw + (size_t)y0 * TT + threadIdx.x);
+  if constexpr (!XI) {
+    if (E == 16 || threadIdx.x < rows * NW)
+      mws[threadIdx.x] = __ldg(I.mw + (size_t)y0 * NW + threadIdx.x);
+  }
 
   if constexpr (IN_SPEC) {
     const T* spec = (a.spec_sel ? I.spec2 : I.spec) + 2 * ((size_t)kk * ny + y0 + rr);
-    cx<T> t[16];
+    cx<T> t[E];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) t[i] = ld_stream_cx<T>(spec + i * tstep);
+    for (int i = 0; i < E; ++i) t[i] = ld_stream_cx<T>(spec + i * tstep);
     cx<T> tn{};
     if (threadIdx.x < rows)
       tn = ldg_cx<T>((a.spec_sel ? I.spec2 : I.spec) + 2 * ((size_t)L * ny + y0 + threadIdx.x));
     const int tb = tix(kk, rr);
 #pragma unroll
-    for (int i = 0; i < 16; ++i) tile[HOIST ? tb + i * ts : tix(kk + i * TT, rr)] = t[i];
+    for (int i = 0; i < E; ++i) tile[HOIST ? tb + i * ts : tix(kk + i * TT, rr)] = t[i];
     if (threadIdx.x < rows) tile[tix(L, threadIdx.x)] = tn;
     __syncthreads();
-    if (threadIdx.x == 0 && !OUT_SPEC) prefetch_compact(I, a.op, mws, rows * TT);
+    if (threadIdx.x == 0 && !OUT_SPEC) prefetch_compact(I, a.op, mws, rows * NW);
     // C2R: Z[k] = (X[k] + conj X[L-k]) + i e^{+2 pi i k / nx} (X[k] - conj X[L-k])
     const cx<T> wt = twiddle<T>(tw, tid * TWS);
     const int cb = tix(tid, row), cm = tix(L - tid, row);
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
+    for (int e = 0; e < E; ++e) {
       const int k = tid + e * TT;
       cx<T> xk = tile[HOIST ? cb + e * ts : tix(k, row)];
       cx<T> xc = conjx(tile[HOIST ? cm - e * ts : tix(L - k, row)]);
@@ -365,97 +374,97 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
         xk.i = (T)0;
         xc.i = (T)0;
       }
-      const cx<T> w = cmul(wt, w32<T>(e));   // W_nx^k, k = tid + e TT
+      const cx<T> w = cmul(wt, w32<T>(e * (16 / E)));   // W_nx^k, k = tid + e TT
       const cx<T> sum = xk + xc;
       const cx<T> dif = cmulc(xk - xc, w);  // (X - conj X') e^{+i...}
       v[e] = cx<T>{sum.r - dif.i, sum.i + dif.r};
     }
     // the first exchange overwrites tile entries other rows still read
-    fft_regs<T, LOG_L, true>(v, xb, tid, tw, cta, rbar);
+    fft_regs<T, LOG_L, LE, true>(v, xb, tid, tw, cta, rbar);
     // v[e] = x[2j] + i x[2j+1], j = tid + e TT
     if constexpr (OUT_SPEC) {
       if (a.op == OP_Y_W)
-        mid_fill<T, TT, OP_Y_W>(I, mwr, rowpix, tid, v);
+        mid_fill<T, TT, E, OP_Y_W>(I, mwr, rowpix, tid, v);
       else
-        mid_fill<T, TT, OP_MASK>(I, mwr, rowpix, tid, v);
+        mid_fill<T, TT, E, OP_MASK>(I, mwr, rowpix, tid, v);
     } else {
       switch (a.op) {
-        case OP_Q: sink_fill<T, TT, OP_Q>(I, mwr, rowpix, tid, v, acc); break;
-        case OP_Z: sink_fill<T, TT, OP_Z>(I, mwr, rowpix, tid, v, acc); break;
-        case OP_B: sink_fill<T, TT, OP_B>(I, mwr, rowpix, tid, v, acc); break;
-        case OP_RES: sink_fill<T, TT, OP_RES>(I, mwr, rowpix, tid, v, acc); break;
-        case OP_GRAD: sink_fill<T, TT, OP_GRAD>(I, mwr, rowpix, tid, v, acc); break;
-        case OP_RELAX: sink_fill<T, TT, OP_RELAX>(I, mwr, rowpix, tid, v, acc); break;
-        case OP_KSEL: sink_fill<T, TT, OP_KSEL>(I, mwr, rowpix, tid, v, acc, a.param); break;
-        case OP_STORE_Y: sink_fill<T, TT, OP_STORE_Y>(I, mwr, rowpix, tid, v, acc); break;
+        case OP_Q: sink_fill<T, TT, E, OP_Q>(I, mwr, rowpix, tid, v, acc); break;
+        case OP_Z: sink_fill<T, TT, E, OP_Z>(I, mwr, rowpix, tid, v, acc); break;
+        case OP_B: sink_fill<T, TT, E, OP_B>(I, mwr, rowpix, tid, v, acc); break;
+        case OP_RES: sink_fill<T, TT, E, OP_RES>(I, mwr, rowpix, tid, v, acc); break;
+        case OP_GRAD: sink_fill<T, TT, E, OP_GRAD>(I, mwr, rowpix, tid, v, acc); break;
+        case OP_RELAX: sink_fill<T, TT, E, OP_RELAX>(I, mwr, rowpix, tid, v, acc); break;
+        case OP_KSEL: sink_fill<T, TT, E, OP_KSEL>(I, mwr, rowpix, tid, v, acc, a.param); break;
+        case OP_STORE_Y: sink_fill<T, TT, E, OP_STORE_Y>(I, mwr, rowpix, tid, v, acc); break;
         case OP_STORE_Y_MASK:
-          sink_fill<T, TT, OP_STORE_Y_MASK>(I, mwr, rowpix, tid, v, acc);
+          sink_fill<T, TT, E, OP_STORE_Y_MASK>(I, mwr, rowpix, tid, v, acc);
           break;
         default: break;
       }
     }
   } else if constexpr (XI) {
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
+    for (int e = 0; e < E; ++e) {
       double x0, x1;
       normal_pair(I.seed, (uint32_t)((rowpix >> 1) + tid + e * TT), x0, x1);
       v[e] = cx<T>{(T)x0, (T)x1};
     }
   } else {
     __syncthreads();   // mask words
-    if (threadIdx.x == 0) prefetch_compact(I, a.op, mws, rows * TT);
+    if (threadIdx.x == 0) prefetch_compact(I, a.op, mws, rows * NW);
     const T alpha = a.op == OP_R_UPD ? cg_alpha<T>(I.st) : (T)0;
     const T beta = a.op == OP_P_UPD_Z || a.op == OP_P_UPD_R ? cg_beta<T>(I.st) : (T)0;
     switch (a.op) {
-      case OP_R_UPD: src_fill<T, TT, OP_R_UPD>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
+      case OP_R_UPD: src_fill<T, TT, E, OP_R_UPD>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
       case OP_P_UPD_Z:
-        src_fill<T, TT, OP_P_UPD_Z>(I, mwr, rowpix, tid, alpha, beta, v, acc);
+        src_fill<T, TT, E, OP_P_UPD_Z>(I, mwr, rowpix, tid, alpha, beta, v, acc);
         break;
       case OP_P_UPD_R:
-        src_fill<T, TT, OP_P_UPD_R>(I, mwr, rowpix, tid, alpha, beta, v, acc);
+        src_fill<T, TT, E, OP_P_UPD_R>(I, mwr, rowpix, tid, alpha, beta, v, acc);
         break;
-      case OP_LOAD_R: src_fill<T, TT, OP_LOAD_R>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
-      case OP_LOAD_U: src_fill<T, TT, OP_LOAD_U>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
-      case OP_LOAD_Y: src_fill<T, TT, OP_LOAD_Y>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
-      case OP_LOAD_W: src_fill<T, TT, OP_LOAD_W>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
+      case OP_LOAD_R: src_fill<T, TT, E, OP_LOAD_R>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
+      case OP_LOAD_U: src_fill<T, TT, E, OP_LOAD_U>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
+      case OP_LOAD_Y: src_fill<T, TT, E, OP_LOAD_Y>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
+      case OP_LOAD_W: src_fill<T, TT, E, OP_LOAD_W>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
       case OP_LOAD_W_MASK:
-        src_fill<T, TT, OP_LOAD_W_MASK>(I, mwr, rowpix, tid, alpha, beta, v, acc);
+        src_fill<T, TT, E, OP_LOAD_W_MASK>(I, mwr, rowpix, tid, alpha, beta, v, acc);
         break;
       case OP_LOAD_D_U:
-        src_fill<T, TT, OP_LOAD_D_U>(I, mwr, rowpix, tid, alpha, beta, v, acc);
+        src_fill<T, TT, E, OP_LOAD_D_U>(I, mwr, rowpix, tid, alpha, beta, v, acc);
         break;
       case OP_U64_UPD:
-        src_fill<T, TT, OP_U64_UPD>(I, mwr, rowpix, tid, alpha, beta, v, acc);
+        src_fill<T, TT, E, OP_U64_UPD>(I, mwr, rowpix, tid, alpha, beta, v, acc);
         break;
       default:
 #pragma unroll
-        for (int e = 0; e < 16; ++e) v[e] = cx<T>{(T)0, (T)0};
+        for (int e = 0; e < E; ++e) v[e] = cx<T>{(T)0, (T)0};
         break;
     }
   }
 
   if constexpr (OUT_SPEC) {
-    fft_regs<T, LOG_L, false>(v, xb, tid, tw, rbar, rbar);
+    fft_regs<T, LOG_L, LE, false>(v, xb, tid, tw, rbar, rbar);
     // Z (the half-length transform) into the transposed tile; the threads of
     // the global stores form X from Z[k] and Z[L-k]:
     // R2C: X[k] = (Z[k] + conj Z[L-k]) / 2 - (i/2) e^{-2 pi i k/nx} (Z[k] - conj Z[L-k])
     __syncthreads();   // the tile overwrites other rows' exchange areas
     const int cb = tix(tid, row);
 #pragma unroll
-    for (int e = 0; e < 16; ++e) tile[HOIST ? cb + e * ts : tix(tid + e * TT, row)] = v[e];
+    for (int e = 0; e < E; ++e) tile[HOIST ? cb + e * ts : tix(tid + e * TT, row)] = v[e];
     __syncthreads();
     const cx<T> wt = twiddle<T>(tw, kk * TWS);
     T* spec = (a.spec_sel ? I.spec2 : I.spec) + 2 * ((size_t)kk * ny + y0 + rr);
     const int tb = tix(kk, rr), tm = tix(L - kk, rr);   // L - kk: the Nyquist row when kk = 0
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
+    for (int i = 0; i < E; ++i) {
       const int k = kk + i * TT;
       const cx<T> zk = tile[HOIST ? tb + i * ts : tix(k, rr)];
       const int im = (i == 0 && kk == 0) ? tix(0, rr) : tm - i * ts;
       const cx<T> zc = conjx(tile[HOIST ? im : tix((L - k) & (L - 1), rr)]);
       const cx<T> ev = scal(zk + zc, (T)0.5);
       const cx<T> od = scal(mul_mi<T, false>(zk - zc), (T)0.5);
-      st_cx<T>(spec + i * tstep, ev + cmul(od, cmul(wt, w32<T>(i))));
+      st_cx<T>(spec + i * tstep, ev + cmul(od, cmul(wt, w32<T>(i * (16 / E)))));
     }
     if (threadIdx.x < rows) {   // Nyquist: X[L] = Re Z[0] - Im Z[0]
       const cx<T> z0 = tile[tix(0, threadIdx.x)];
@@ -470,7 +479,7 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
 }
 
 // ----------------------------------------------------------------- column pass
-// CTA = `ffts` spectrum rows (one kx each), N/16 threads per row; forward
+// CTA = `ffts` spectrum rows (one kx each), N/E threads per row; forward
 // column FFT, multiply by the real table, inverse column FFT, in place
 // (table < 0: forward transform only; PRE: start from the forward transform
 // held in spec and write to the buffer spec_sel names).  blockIdx.x is the instance, so the
@@ -479,7 +488,9 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
 template <typename T, int LOG_N, bool PRE = false>
 __global__ void __launch_bounds__(KCfg<T>::kMaxThreads)
 k_col(const InstDesc<T>* __restrict__ insts, ColArgs a, const T* __restrict__ tw) {
-  constexpr int N = 1 << LOG_N, TT = N / 16, PADN = N + N / 16 + 1;
+  constexpr int LE = col_le<T>(LOG_N), E = 1 << LE;
+  constexpr int N = 1 << LOG_N, TT = N / E, PADN = N + N / 16 + 1;
+  constexpr bool TAB = LE < 4 || !std::is_same<T, float>::value;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
   const InstDesc<T>& I = insts[blockIdx.x];
@@ -491,15 +502,15 @@ k_col(const InstDesc<T>* __restrict__ insts, ColArgs a, const T* __restrict__ tw
   const XBar bar = XBar::make(TT, a.ffts, f);
   T* col = (a.spec_sel ? I.spec2 : I.spec) + 2 * (long long)(act ? kx : 0) * N;
   const T* src = PRE ? I.spec + 2 * (long long)(act ? kx : 0) * N : col;
-  cx<T> v[16];
+  cx<T> v[E];
 #pragma unroll
-  for (int e = 0; e < 16; ++e) v[e] = act ? ld_stream_cx<T>(src + 2 * (tid + e * TT)) : cx<T>{(T)0, (T)0};
-  if constexpr (!PRE) fft_regs<T, LOG_N, false, false>(v, xb, tid, tw, bar, bar);
+  for (int e = 0; e < E; ++e) v[e] = act ? ld_stream_cx<T>(src + 2 * (tid + e * TT)) : cx<T>{(T)0, (T)0};
+  if constexpr (!PRE) fft_regs<T, LOG_N, LE, false, TAB>(v, xb, tid, tw, bar, bar);
   if (a.table >= 0) {
     const T* tab = (a.table >= 2 ? I.kt + (long long)(a.table - 2) * a.nkx * N
                     : a.table ? I.t_sqrt : I.t_inv) + (long long)(act ? kx : 0) * N;
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
+    for (int e = 0; e < E; ++e) {
       const T t = act ? ldg1(tab + tid + e * TT) : (T)0;
       v[e] = scal(v[e], t);
     }
@@ -508,11 +519,11 @@ k_col(const InstDesc<T>* __restrict__ insts, ColArgs a, const T* __restrict__ tw
     // them live across the table multiply and spill registers
     const T* tw_inv;
     asm("mov.b64 %0, %1;" : "=l"(tw_inv) : "l"(tw));
-    fft_regs<T, LOG_N, true, false>(v, xb, tid, tw_inv, bar, bar);
+    fft_regs<T, LOG_N, LE, true, TAB>(v, xb, tid, tw_inv, bar, bar);
   }
   if (act) {
 #pragma unroll
-    for (int e = 0; e < 16; ++e) st_cx<T>(col + 2 * (tid + e * TT), v[e]);
+    for (int e = 0; e < E; ++e) st_cx<T>(col + 2 * (tid + e * TT), v[e]);
   }
 }
 
@@ -531,6 +542,15 @@ k_col(const InstDesc<T>* __restrict__ insts, ColArgs a, const T* __restrict__ tw
 // done are skipped.  Every wait is bounded: on a timeout the CTA sets
 // *a.err, waits (bounded) for the copies it issued, and returns.
 constexpr int kColTmaSlots = 2;
+// Columns per item: 256 threads' worth (F N = 256 E complex values), one
+// 8192-point column above that.
+CGF_HD constexpr int col_tma_ffts(int log_n) {
+  const int f = (256 << col_le<float>(log_n)) >> log_n;
+  return f > 0 ? f : 1;
+}
+CGF_HD constexpr int col_tma_threads(int log_n) {
+  return (col_tma_ffts(log_n) << log_n) >> col_le<float>(log_n);
+}
 
 __host__ __device__ __forceinline__ size_t col_tma_smem(int log_n, int ffts) {
   const size_t fn = size_t(ffts) << log_n;
@@ -538,10 +558,12 @@ __host__ __device__ __forceinline__ size_t col_tma_smem(int log_n, int ffts) {
 }
 
 template <int LOG_N>
-__global__ void __launch_bounds__(LOG_N >= 13 ? 512 : 256, LOG_N >= 13 ? 1 : 2)
+__global__ void __launch_bounds__(col_tma_threads(LOG_N), LOG_N >= 13 ? 1 : 2)
 k_col_tma(const InstDesc<float>* __restrict__ insts, ColArgs a, const float* __restrict__ tw,
           int ninst) {
-  constexpr int N = 1 << LOG_N, TT = N / 16;
+  constexpr int LE = col_le<float>(LOG_N), E = 1 << LE;
+  constexpr int N = 1 << LOG_N, TT = N / E;
+  constexpr bool TAB = LE < 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int F = a.ffts;
   const size_t fn = size_t(F) * N;
@@ -609,26 +631,26 @@ k_col_tma(const InstDesc<float>* __restrict__ insts, ColArgs a, const float* __r
     const bool act = kx < a.nkx;
     float2* buf = slot0 + sl * fn + size_t(f) * N;
     const float* tb = tab0 + sl * fn + size_t(f) * N;
-    cx<float> v[16];
+    cx<float> v[E];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
+    for (int e = 0; e < E; ++e) {
       const float2 t = act ? buf[tid + e * TT] : make_float2(0.f, 0.f);
       v[e] = cx<float>{t.x, t.y};
     }
     const XBufSw xb(buf);
-    fft_regs<float, LOG_N, false, false>(v, xb, tid, tw, fbar, fbar);
+    fft_regs<float, LOG_N, LE, false, TAB>(v, xb, tid, tw, fbar, fbar);
 #pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = scal(v[e], act ? tb[tid + e * TT] : 0.f);
+    for (int e = 0; e < E; ++e) v[e] = scal(v[e], act ? tb[tid + e * TT] : 0.f);
     // the inverse transform reloads its twiddles (an opaque copy of the table
     // pointer): keeping the forward transform's alive across the table
     // multiply would cost some 60 registers and spills
     const float* tw_inv;
     asm("mov.b64 %0, %1;" : "=l"(tw_inv) : "l"(tw));
-    fft_regs<float, LOG_N, true, false>(v, xb, tid, tw_inv, fbar, fbar);
+    fft_regs<float, LOG_N, LE, true, TAB>(v, xb, tid, tw_inv, fbar, fbar);
     if (act) {
       float* col = I.spec + 2 * (long long)kx * N;
 #pragma unroll
-      for (int e = 0; e < 16; ++e) st_cx<float>(col + 2 * (tid + e * TT), v[e]);
+      for (int e = 0; e < E; ++e) st_cx<float>(col + 2 * (tid + e * TT), v[e]);
     }
     __syncthreads();   // slot sl is free again
     it = nxt;

@@ -9,9 +9,9 @@ namespace cgf {
 
 template <typename T>
 size_t Launch<T>::row_smem(int log_l, int rows) {
-  // FFT areas / transposed tile, then one mask word (8 bytes) per thread
-  const size_t tt = (size_t(1) << log_l) / 16;
-  return row_main_bytes<T>(log_l, rows) + size_t(rows) * tt * sizeof(uint2);
+  // FFT areas / transposed tile, then the mask words (8 bytes per 32 pixels)
+  const size_t nw = (size_t(1) << log_l) / 16;
+  return row_main_bytes<T>(log_l, rows) + size_t(rows) * nw * sizeof(uint2);
 }
 
 template <typename T>
@@ -42,7 +42,7 @@ inline cudaError_t allow_smem(K kernel) {
 template <typename T, int LL>
 cudaError_t row_ll(bool in_spec, bool out_spec, const InstDesc<T>* d, int ninst, const RowArgs& a,
                    const T* tw, cudaStream_t s) {
-  constexpr int TT = (1 << LL) / 16;
+  constexpr int TT = (1 << LL) >> row_le<T>(LL);
   dim3 grid(a.ny / a.rows, ninst), block(a.rows * TT);
   const size_t sm = Launch<T>::row_smem(LL, a.rows);
   if (in_spec && out_spec)
@@ -60,13 +60,9 @@ cudaError_t row_ll(bool in_spec, bool out_spec, const InstDesc<T>* d, int ninst,
 // set by prepare_cols.
 static int g_col_tma_ctas[14] = {};
 
-// Column FFTs per item of the TMA column pass: F N = 4096 complex values
-// (256 threads) when N <= 4096, one 8192-point column otherwise.
-inline int col_tma_ffts(int log_n) { return log_n >= 12 ? 1 : (4096 >> log_n); }
-
 template <int LN>
 cudaError_t prep_col_tma() {
-  const int F = col_tma_ffts(LN), threads = F * ((1 << LN) / 16);
+  constexpr int F = col_tma_ffts(LN), threads = col_tma_threads(LN);
   const size_t sm = col_tma_smem(LN, F);
   cudaError_t e = cudaFuncSetAttribute(k_col_tma<LN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
@@ -80,7 +76,7 @@ cudaError_t prep_col_tma() {
 
 template <typename T, int LN>
 cudaError_t col_ln(const InstDesc<T>* d, int ninst, const ColArgs& a, const T* tw, cudaStream_t s) {
-  constexpr int TT = (1 << LN) / 16;
+  constexpr int TT = (1 << LN) >> col_le<T>(LN);
   if constexpr (std::is_same<T, float>::value) {
     // the CG loops' table passes: persistent, bulk-copy fed
     if (a.variant == 1 && (a.table == 0 || a.table == 1) && !a.pre && a.spec_sel == 0 &&
@@ -90,7 +86,7 @@ cudaError_t col_ln(const InstDesc<T>* d, int ninst, const ColArgs& a, const T* t
       b.ffts = F;
       const long long items = (long long)((a.nkx + F - 1) / F) * ninst;
       const int grid = (int)(items < g_col_tma_ctas[LN] ? items : g_col_tma_ctas[LN]);
-      k_col_tma<LN><<<grid, F * TT, col_tma_smem(LN, F), s>>>(d, b, tw, ninst);
+      k_col_tma<LN><<<grid, col_tma_threads(LN), col_tma_smem(LN, F), s>>>(d, b, tw, ninst);
       return cudaGetLastError();
     }
   }

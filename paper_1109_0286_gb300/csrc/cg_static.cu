@@ -89,16 +89,17 @@ __global__ void k_static_setup(unsigned char* base, Layout L, int ny, int nx, co
   }
   // the per-stage tables of every power-of-two length (layout in cg_types.h)
   for (long long e = tid; e < kStwEntries; e += nthr) {
-    int l = 4;
-    while (l < 13 && e >= stw_base(l + 1)) ++l;
-    int rem = (int)(e - stw_base(l));
-    int st = stw_first(l);
-    while (st + 1 < l / 4 && rem >= stw_stage_off(l, st + 1)) ++st;
-    rem -= stw_stage_off(l, st);
-    const int ns = stw_ns(l, st);
+    int le = 2, l = 4;
+    while (le < 4 && e >= stw_base(le + 1, 4)) ++le;
+    while (l < 13 && e >= stw_base(le, l + 1)) ++l;
+    int rem = (int)(e - stw_base(le, l));
+    int st = stw_first(le, l);
+    while (st + 1 < l / le && rem >= stw_stage_off(le, l, st + 1)) ++st;
+    rem -= stw_stage_off(le, l, st);
+    const int ns = stw_ns(le, l, st);
     const int r = 1 + rem / ns, jm = rem % ns;
     double s, c;
-    sincospi(2.0 * double((long long)jm * r) / double(16LL * ns), &s, &c);
+    sincospi(2.0 * double((long long)jm * r) / double((1LL << le) * ns), &s, &c);
     tw[2 * (kLmax + e)] = (float)c;
     tw[2 * (kLmax + e) + 1] = (float)-s;
   }

@@ -222,35 +222,63 @@ struct VecArgs {
 
 constexpr int kLmax = 8192;        // twiddle master table: W_8192^m
 
+// Elements per thread of the register-resident FFTs (cg_fft.cuh), as log2:
+// the row transform of length 2^log (nx / 2) and the column transform of
+// length 2^log (ny), per element type.  They depend on the grid and the type
+// only (not on the batch), so a map's results do not depend on what it is
+// batched with.  Fewer elements per thread shorten the chain of instructions
+// that a small grid's pass consists of (one wave of CTAs); more save
+// exchanges once the chip is full.  Measured with 16, 8 and 4 elements:
+//   FP32, us per CG iteration: 64^2 62, 44, 38; 256^2 65, 53, 46 (16 maps 71,
+//   66, 71; rows 8 and columns 4: 49 and 67); 512^2 69, 55, 56 (16 maps 128,
+//   137, 186); 1024^2 76, 72, 78 (16 maps 359, 477, 424); 2048^2 149, 183, -.
+//   FP64: 64^2 264, -, 82; 512^2 586, -, 165; 1024^2 966, -, 606.  An FP64
+//   instruction holds its scheduler's pipe for 64 cycles, so a short chain
+//   counts most; from 2048 pixels on, 8 and 16 keep the rows of a CTA.
+//   Double-float (20 relaxation sweeps): 256^2 1641, 979, 661; 512^2 1877,
+//   1028, 767 (8 maps 2178, 2047, 2151); 1024^2 2127, 1352, -; 2048^2 x 8
+//   37176, 29635, -; 4096^2 21013, 17847, - us.
+template <typename T>
+CGF_HD constexpr int row_le(int log) { return log <= 6 ? 2 : log <= 8 ? 3 : 4; }
+template <typename T>
+CGF_HD constexpr int col_le(int log) { return log <= 8 ? 2 : log <= 9 ? 3 : 4; }
+struct df;
+template <>
+CGF_HD constexpr int row_le<df>(int log) { return log <= 8 ? 2 : log <= 11 ? 3 : 4; }
+template <>
+CGF_HD constexpr int col_le<df>(int log) { return log <= 9 ? 2 : log <= 12 ? 3 : 4; }
+template <>
+CGF_HD constexpr int row_le<double>(int log) { return log <= 9 ? 2 : log <= 11 ? 3 : 4; }
+template <>
+CGF_HD constexpr int col_le<double>(int log) { return log <= 10 ? 2 : log <= 12 ? 3 : 4; }
+
 // Per-stage twiddle tables of the register-resident FFT (cg_fft.cuh), stored
-// after the master table.  A transform of length 2^log (4 <= log <= 13) has
-// one leading stage of radix 2^(log mod 4) (if nonzero) and log/4 radix-16
-// stages; the radix-16 stage s runs on sub-transforms of size
-// ns = 2^(log mod 4) 16^s and needs W_{16 ns}^(jm r), jm < ns, r = 1..15
-// (none for the very first stage, ns = 1).  Its table holds them as
-// [r - 1][jm], so that the threads of a warp (consecutive jm) read
-// consecutive entries.
-CGF_HD constexpr int stw_ns0(int log) { return (log % 4) ? (1 << (log % 4)) : 1; }
-CGF_HD constexpr int stw_first(int log) { return (log % 4) ? 0 : 1; }   // first twiddled stage
-CGF_HD constexpr int stw_ns(int log, int s) {
-  int ns = stw_ns0(log);
-  for (int t = 0; t < s; ++t) ns *= 16;
-  return ns;
+// after the master table.  With 2^le elements per thread (le = 2, 3, 4) a
+// transform of length 2^log (4 <= log <= 13) has one leading stage of radix
+// 2^(log mod le) (if nonzero) and log/le stages of radix R = 2^le; the
+// radix-R stage s runs on sub-transforms of size ns = 2^(log mod le) R^s and
+// needs W_{R ns}^(jm r), jm < ns, r = 1..R-1 (none for the very first stage,
+// ns = 1).  Its table holds them as [r - 1][jm], so that the threads of a warp
+// (consecutive jm) read consecutive entries.
+CGF_HD constexpr int stw_first(int le, int log) { return (log % le) ? 0 : 1; }   // first twiddled stage
+CGF_HD constexpr int stw_ns(int le, int log, int s) {
+  return ((log % le) ? (1 << (log % le)) : 1) << (le * s);
 }
 // entries of the stages before s of length 2^log
-CGF_HD constexpr int stw_stage_off(int log, int s) {
+CGF_HD constexpr int stw_stage_off(int le, int log, int s) {
   int o = 0;
-  for (int t = stw_first(log); t < s; ++t) o += 15 * stw_ns(log, t);
+  for (int t = stw_first(le, log); t < s; ++t) o += ((1 << le) - 1) * stw_ns(le, log, t);
   return o;
 }
-CGF_HD constexpr int stw_size(int log) { return stw_stage_off(log, log / 4); }
-// entries of the lengths 2^4 .. 2^(log-1) (the tables of length 2^log start here)
-CGF_HD constexpr int stw_base(int log) {
+CGF_HD constexpr int stw_size(int le, int log) { return stw_stage_off(le, log, log / le); }
+// entries of the smaller le and, within le, of the lengths 2^4 .. 2^(log-1)
+CGF_HD constexpr int stw_base(int le, int log) {
   int o = 0;
-  for (int l = 4; l < log; ++l) o += stw_size(l);
+  for (int e = 2; e <= le; ++e)
+    for (int l = 4; l < (e < le ? 14 : log); ++l) o += stw_size(e, l);
   return o;
 }
-constexpr int kStwEntries = stw_base(14);   // all lengths 2^4 .. 2^13
+constexpr int kStwEntries = stw_base(4, 14);   // all lengths 2^4 .. 2^13, le = 2, 3, 4
 constexpr int kTwEntries = kLmax + kStwEntries;   // complex entries of a twiddle buffer
 constexpr int kMaxPartials = 4096; // CTAs per instance per reducing pass
 constexpr int kMaxBands = 64;      // band-power gradient bins

@@ -81,19 +81,20 @@ void unit_root(long long num, long long den, double* re, double* im) {
 
 // W_kLmax^m = exp(-2 pi i m / kLmax) from quadrant-reduced angles, followed
 // by the per-stage tables of every power-of-two length (stw_* in cg_types.h).
-void twiddles_host(std::vector<double>& tw) {
+std::vector<double> twiddles_build() {
   const int N = kLmax, Q = N / 4;
-  tw.resize(2 * size_t(kTwEntries));
-  for (int l = 4; l <= 13; ++l)
-    for (int st = stw_first(l); st < l / 4; ++st) {
-      const int ns = stw_ns(l, st);
-      const size_t base = size_t(kLmax) + stw_base(l) + stw_stage_off(l, st);
-      for (int r = 1; r < 16; ++r)
-        for (int jm = 0; jm < ns; ++jm) {
-          const size_t e = base + size_t(r - 1) * ns + jm;
-          unit_root((long long)jm * r, 16LL * ns, &tw[2 * e], &tw[2 * e + 1]);
-        }
-    }
+  std::vector<double> tw(2 * size_t(kTwEntries));
+  for (int le = 2; le <= 4; ++le)
+    for (int l = 4; l <= 13; ++l)
+      for (int st = stw_first(le, l); st < l / le; ++st) {
+        const int ns = stw_ns(le, l, st), R = 1 << le;
+        const size_t base = size_t(kLmax) + stw_base(le, l) + stw_stage_off(le, l, st);
+        for (int r = 1; r < R; ++r)
+          for (int jm = 0; jm < ns; ++jm) {
+            const size_t e = base + size_t(r - 1) * ns + jm;
+            unit_root((long long)jm * r, (long long)R * ns, &tw[2 * e], &tw[2 * e + 1]);
+          }
+      }
   for (int m = 0; m < N; ++m) {
     const int q = m / Q, r = m % Q;
     const double th = 2.0 * M_PI * double(r) / double(N);
@@ -108,6 +109,12 @@ void twiddles_host(std::vector<double>& tw) {
     tw[2 * m] = c;
     tw[2 * m + 1] = -s;
   }
+  return tw;
+}
+// Built once per process (constants).
+const std::vector<double>& twiddles_host() {
+  static const std::vector<double> tw = twiddles_build();
+  return tw;
 }
 
 template <typename T>
@@ -1231,7 +1238,7 @@ cudaError_t upload_tables(fill_plan* p, const std::vector<double>& tinv,
 
 template <typename T>
 fill_status setup_precision(fill_plan* p, const std::vector<double>& tinv,
-                            const std::vector<double>& tsqrt, const std::vector<double>& tw) {
+                            const std::vector<double>& tsqrt) {
   Precision<T>& P = prec<T>(p);
   P.used = true;
   const size_t B = p->batch, n = p->npix, nv = p->nv;
@@ -1262,10 +1269,20 @@ fill_status setup_precision(fill_plan* p, const std::vector<double>& tinv,
     for (size_t i = 0; i < B; ++i) ptrs[i] = P.st + i;
     CK(cudaMemcpy(P.stp, ptrs.data(), B * sizeof(CgState*), cudaMemcpyHostToDevice));
   }
-  std::vector<T> w(2 * size_t(kTwEntries));
-  for (size_t i = 0; i < w.size(); ++i) w[i] = (T)tw[i];
   CK(upload_tables<T>(p, tinv, tsqrt));
-  CK(cudaMemcpy(P.tw, w.data(), w.size() * sizeof(T), cudaMemcpyHostToDevice));
+  if (!p->gen) {
+    // the master table and the stage tables of this grid's two lengths
+    const int ll = p->log_l, ln = p->log_n, rl = row_le<T>(ll), cl = col_le<T>(ln);
+    const int part[3][2] = {{0, kLmax}, {kLmax + stw_base(rl, ll), stw_size(rl, ll)},
+                            {kLmax + stw_base(cl, ln), stw_size(cl, ln)}};
+    const std::vector<double>& tw = twiddles_host();
+    std::vector<T> w;
+    for (const auto& r : part) {
+      w.resize(2 * size_t(r[1]));
+      for (size_t i = 0; i < w.size(); ++i) w[i] = (T)tw[2 * size_t(r[0]) + i];
+      CK(cudaMemcpy(P.tw + 2 * size_t(r[0]), w.data(), w.size() * sizeof(T), cudaMemcpyHostToDevice));
+    }
+  }
   CK(cudaMemset(P.u, 0, B * nv * sizeof(T)));
   CK(cudaMemset(P.p, 0, B * nv * sizeof(T)));
   if (p->gen) {
@@ -1273,9 +1290,9 @@ fill_status setup_precision(fill_plan* p, const std::vector<double>& tinv,
     if (gs != FILL_OK) return gs;
   } else {
     const bool user = loop_precision<T>(p);
-    P.rows = user && p->o.rows_per_cta > 0 ? std::min(p->o.rows_per_cta, p->ny)
+    P.rows = user && p->o.rows_per_cta > 0 ? fit_rows<T>(p->log_l, std::min(p->o.rows_per_cta, p->ny))
                                            : default_rows<T>(p->log_l, p->ny);
-    P.ffts = user && p->o.ffts_per_cta > 0 ? p->o.ffts_per_cta
+    P.ffts = user && p->o.ffts_per_cta > 0 ? fit_ffts<T>(p->log_n, p->o.ffts_per_cta)
                                            : default_ffts<T>(p->log_n, p->nx / 2 + 1);
     if (!schedule_valid<T>(p->log_l, p->log_n, p->ny, P.rows, P.ffts)) return FILL_EINVAL;
     P.col_variant = std::is_same<T, float>::value ? p->o.col_kernel : 0;
@@ -1484,19 +1501,18 @@ fill_status fill_init(fill_plan** out, int ny, int nx, const double* P_half,
   if (e != cudaSuccess) return fail(cuda_fail(e, "fill_init"));
   e = cudaMemcpy(p->mw, words.data(), words.size() * sizeof(uint2), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return fail(cuda_fail(e, "upload mask"));
-  std::vector<double> tinv, tsqrt, tw;
+  std::vector<double> tinv, tsqrt;
   spectral_tables(ny, nx, P_half, tinv, tsqrt, &p->relax_a);
-  twiddles_host(tw);
   if (o.mode == FILL_MODE_FP32 || o.mode == FILL_MODE_MIXED) {
-    fs = setup_precision<float>(p, tinv, tsqrt, tw);
+    fs = setup_precision<float>(p, tinv, tsqrt);
     if (fs != FILL_OK) return fail(fs);
   }
   if (o.mode == FILL_MODE_FP64) {
-    fs = setup_precision<double>(p, tinv, tsqrt, tw);
+    fs = setup_precision<double>(p, tinv, tsqrt);
     if (fs != FILL_OK) return fail(fs);
   }
   if (o.mode == FILL_MODE_MIXED) {
-    fs = setup_precision<df>(p, tinv, tsqrt, tw);
+    fs = setup_precision<df>(p, tinv, tsqrt);
     if (fs != FILL_OK) return fail(fs);
     for (int i = 0; i < p->batch; ++i) {
       p->h.hdesc[i].dlt = p->f.hdesc[i].u;
@@ -2202,7 +2218,8 @@ cudaError_t autotune_ctx(Ctx<T> c, cudaStream_t s, int* best_rows, int* best_fft
   CE(cudaGetDevice(&dev));
   CE(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   const size_t limit = size_t(optin) - 1024;
-  const int TT = (1 << c.log_l) / 16, TN = (1 << c.log_n) / 16, nkx = c.nx / 2 + 1;
+  const int TT = (1 << c.log_l) >> row_le<T>(c.log_l), TN = (1 << c.log_n) >> col_le<T>(c.log_n);
+  const int nkx = c.nx / 2 + 1;
   float best = 1e30f;
   for (int r = 1; r <= c.ny && r <= 256; r *= 2) {
     if (r * TT > Launch<T>::max_threads() || r * TT < 32 || c.ny / r > kMaxPartials ||
@@ -2330,6 +2347,8 @@ fill_status tune_plan_t(fill_plan* p, const char* path) {
   }
   int nf = P.ffts, nv = P.col_variant;
   apply_col_choice(ffts, &nf, &nv);
+  rows = fit_rows<T>(p->log_l, rows);
+  nf = fit_ffts<T>(p->log_n, nf);
   if (rows != P.rows || nf != P.ffts || nv != P.col_variant) {
     P.rows = rows;
     P.ffts = nf;
@@ -2553,6 +2572,8 @@ fill_status group_setup(fill_group* g, int autotune, const char* path) {
       int tuned = c.col_variant ? -1 : c.ffts;
       if (cache_lookup(path, pr, c.ny, c.nx, c.ninst, &c.rows, &tuned)) {
         apply_col_choice(tuned, &c.ffts, &c.col_variant);
+        c.rows = fit_rows<T>(c.log_l, c.rows);
+        c.ffts = fit_ffts<T>(c.log_n, c.ffts);
       } else {
         Ctx<T> cx_ = gctx<T>(g, c);
         k_state_init<T><<<(c.ninst + 127) / 128, 128, 0, g->s>>>(
