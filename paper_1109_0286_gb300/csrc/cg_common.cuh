@@ -32,6 +32,15 @@ __device__ __forceinline__ cx<T> conjx(cx<T> a) { return {a.r, -a.i}; }
 template <typename T>
 __device__ __forceinline__ cx<T> scal(cx<T> a, T s) { return {a.r * s, a.i * s}; }
 
+// a * s rounded on its own (not contracted into the additions that follow), so
+// that two kernels that spell the same steps agree bit for bit.
+template <typename T>
+__device__ __forceinline__ cx<T> scal_rn(cx<T> a, T s) { return {a.r * s, a.i * s}; }
+template <>
+__device__ __forceinline__ cx<float> scal_rn<float>(cx<float> a, float s) {
+  return {__fmul_rn(a.r, s), __fmul_rn(a.i, s)};
+}
+
 // Double-float arithmetic (error-free transformations: Knuth's TwoSum for
 // the high parts, FMA-exact products; Dekker's renormalisation).  Relative
 // error of an operation about 2^-46 of the operands' magnitude.
@@ -49,6 +58,19 @@ __device__ __forceinline__ df operator*(df a, df b) {
   const float e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(a.hi, b.hi, -p)));
   const float h = p + e;
   return df(h, e - (h - p));
+}
+
+// Programmatic dependent launch: a pass launched with the attribute
+// (RowArgs::pdl and so on) starts while the pass before it in the stream still
+// runs, does what does not depend on it (descriptor, mask words, twiddles),
+// and waits here for its end (all its writes visible).  Without the attribute
+// both are no-ops.  The trigger, before a CTA's last stores and sums, lets the
+// next pass start in turn.  (Triggered right after the wait, the CTAs of the
+// next pass crowd onto the SMs that hold none of this one: 512^2 FP64 186
+// against 162 us per iteration, 256^2 x 16 70 against 63.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Vector types for 8- / 16-byte global accesses.
@@ -126,6 +148,19 @@ __device__ __forceinline__ cx<df> ld_stream_cx<df>(const df* p) {
                : "=f"(a), "=f"(b), "=f"(c), "=f"(d)
                : "l"(p));
   return {df(a, b), df(c, d)};
+}
+
+// Loads from L2 of values that other CTAs of the same kernel, or the kernel
+// before, wrote (volatile: kept behind the waits and barriers they follow).
+__device__ __forceinline__ double ld_l2(const double* p) {
+  double v;
+  asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned long long ld_l2(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
 }
 
 // Asks the copy engine to bring elements [c0, c1) of a vector into L2 (one
@@ -270,114 +305,113 @@ __device__ __forceinline__ V segment_sum(V v, unsigned mask, int lane, int nl, i
 
 // CG coefficient record for the Lanczos estimate (Sect. 6.4): alpha_j when
 // computed (j = iterations completed so far), beta_j after iteration j.
-__device__ __forceinline__ void record_alpha(CgState* st) {
-  if (st->coef && st->iter < st->hist_cap) st->coef[2 * st->iter] = st->alpha;
+__device__ __forceinline__ void record_alpha(const CgState& c, double alpha) {
+  if (c.coef && c.iter < c.hist_cap) c.coef[2 * c.iter] = alpha;
 }
-__device__ __forceinline__ void record_beta(CgState* st) {
-  if (st->coef && st->iter >= 1 && st->iter - 1 < st->hist_cap)
-    st->coef[2 * (st->iter - 1) + 1] = st->beta;
+__device__ __forceinline__ void set_beta(CgState* st, const CgState& c, int iter, double sum) {
+  const double beta = sum / c.rho;
+  st->beta = beta;
+  st->beta_f = (float)beta;
+  st->rho = sum;
+  if (c.coef && iter >= 1 && iter - 1 < c.hist_cap) c.coef[2 * (iter - 1) + 1] = beta;
+}
+__device__ __forceinline__ void zero_beta(CgState* st, double rho) {
+  st->rho = rho;
+  st->beta = 0.0;
+  st->beta_f = 0.f;
+  st->first = 0;
+}
+__device__ __forceinline__ void stop(CgState* st, int status) {
+  if (status) st->status = status;
+  st->done = 1;
+}
+__device__ __forceinline__ void record_hist(const CgState& c, int k, double sum) {
+  if (c.hist && k < c.hist_cap) c.hist[k] = sqrt(sum / c.bb);
 }
 
 // Scalar update executed once per instance by the last CTA of a pass, with
 // the sum of all CTA partials (fixed order, so results are reproducible).
-__device__ __forceinline__ void scalar_update(int sop, CgState* st, double sum) {
+// c: the state as it was when the pass began, in shared memory (grid_reduce
+// brings it there with one load per lane while the sums are formed; reading
+// the fields one after another from L2 took about 1.5 us of each reducing
+// pass); st: where the new values go.
+__device__ __forceinline__ void scalar_update(int sop, CgState* st, const CgState& c, double sum) {
   switch (sop) {
     case SC_BB:
     case SC_BB_RHO:
       st->bb = sum;
       st->rr = sum;
       st->rrmax = sum;
-      if (st->hist && st->hist_cap > 0) st->hist[0] = sum > 0.0 ? 1.0 : 0.0;
+      if (c.hist && c.hist_cap > 0) c.hist[0] = sum > 0.0 ? 1.0 : 0.0;
       if (!isfinite(sum)) {
-        st->done = 1;
-        st->status = 1;  // FILL_EINVAL: NaN / Inf in the data (P is validated on the host)
+        stop(st, 1);    // FILL_EINVAL: NaN / Inf in the data (P is validated on the host)
       } else if (sum == 0.0) {
-        st->done = 1;    // nothing to solve: u = 0
+        stop(st, 0);    // nothing to solve: u = 0
       }
-      if (sop == SC_BB_RHO) {   // plain CG: z = r, rho = ||r||^2, p = r
-        st->rho = sum;
-        st->beta = 0.0;
-        st->beta_f = 0.f;
-        st->first = 0;
-      }
+      if (sop == SC_BB_RHO) zero_beta(st, sum);   // plain CG: z = r, rho = ||r||^2, p = r
       break;
     case SC_ALPHA:
       st->pq = sum;
       if (!(sum > 0.0) || !isfinite(sum)) {
-        st->status = 4;
-        st->done = 1;
+        stop(st, 4);
       } else {
-        st->alpha = st->rho / sum;
-        st->alpha_f = (float)st->alpha;
-        record_alpha(st);
+        const double alpha = c.rho / sum;
+        st->alpha = alpha;
+        st->alpha_f = (float)alpha;
+        record_alpha(c, alpha);
       }
       break;
     case SC_RCHECK:
     case SC_RCHECK_BETA: {
+      const int iter = c.iter + 1;
       st->rr = sum;
-      st->iter += 1;
-      if (st->hist && st->iter < st->hist_cap) st->hist[st->iter] = sqrt(sum / st->bb);
-      if (!isfinite(sum)) {
-        st->status = 4;
-        st->done = 1;
-      } else if (sum <= st->tol2 * st->bb) {
-        st->done = 1;
-      } else if (st->iter >= st->max_iter) {
-        st->status = 3;
-        st->done = 1;
-      } else if (sop == SC_RCHECK_BETA) {
-        st->beta = sum / st->rho;
-        st->beta_f = (float)st->beta;
-        st->rho = sum;
-        record_beta(st);
-      }
+      st->iter = iter;
+      record_hist(c, iter, sum);
+      if (!isfinite(sum))
+        stop(st, 4);
+      else if (sum <= c.tol2 * c.bb)
+        stop(st, 0);
+      else if (iter >= c.max_iter)
+        stop(st, 3);
+      else if (sop == SC_RCHECK_BETA)
+        set_beta(st, c, iter, sum);
       break;
     }
     case SC_BETA:
-      if (!(sum > 0.0) || !isfinite(sum)) {
-        st->status = 4;
-        st->done = 1;
-      } else if (st->first) {
-        st->first = 0;
-        st->rho = sum;
-        st->beta = 0.0;
-        st->beta_f = 0.f;
-      } else {
-        st->beta = sum / st->rho;
-        st->beta_f = (float)st->beta;
-        st->rho = sum;
-        record_beta(st);
-      }
+      if (!(sum > 0.0) || !isfinite(sum))
+        stop(st, 4);
+      else if (c.first)
+        zero_beta(st, sum);
+      else
+        set_beta(st, c, c.iter, sum);
       break;
     case SC_RCHECK_UPD: {
+      const int iter = c.iter + 1;
       st->rr = sum;
-      st->iter += 1;
-      if (st->hist && st->iter < st->hist_cap) st->hist[st->iter] = sqrt(sum / st->bb);
+      st->iter = iter;
+      record_hist(c, iter, sum);
       if (!isfinite(sum)) {
-        st->status = 4;
-        st->done = 1;
-        st->peer->upd = 1;   // fold what was gained and report the true residual
-      } else if (sum <= st->delta2 * st->rrmax || sum <= st->tol2 * st->bb) {
-        st->peer->upd = 1;
-      } else if (st->iter >= st->max_iter) {
-        st->status = 3;
-        st->done = 1;
-        st->peer->upd = 1;
+        stop(st, 4);
+        c.peer->upd = 1;   // fold what was gained and report the true residual
+      } else if (sum <= c.delta2 * c.rrmax || sum <= c.tol2 * c.bb) {
+        c.peer->upd = 1;
+      } else if (iter >= c.max_iter) {
+        stop(st, 3);
+        c.peer->upd = 1;
       }
       break;
     }
     case SC_RES_UPD: {
-      CgState* f = st->peer;
+      CgState* f = c.peer;
       st->rr = sum;
       st->upd = 0;
-      st->refine += 1;
-      if (st->hist && st->refine < st->hist_cap) st->hist[st->refine] = sqrt(sum / st->bb);
+      st->refine = c.refine + 1;
+      record_hist(c, c.refine + 1, sum);
       if (!isfinite(sum)) {
-        st->status = 4;
-        st->done = 1;
+        stop(st, 4);
         f->done = 1;
-      } else if (sum <= st->tol2 * st->bb) {
-        st->done = 1;
+      } else if (sum <= c.tol2 * c.bb) {
+        stop(st, 0);
         f->done = 1;
       } else if (!f->done) {
         f->rr = sum;
@@ -391,14 +425,12 @@ __device__ __forceinline__ void scalar_update(int sop, CgState* st, double sum) 
       break;
     case SC_RES:
       st->rr = sum;
-      st->refine += 1;
-      if (st->hist && st->refine < st->hist_cap) st->hist[st->refine] = sqrt(sum / st->bb);
-      if (!isfinite(sum)) {
-        st->status = 4;
-        st->done = 1;
-      } else if (sum <= st->tol2 * st->bb) {
-        st->done = 1;
-      }
+      st->refine = c.refine + 1;
+      record_hist(c, c.refine + 1, sum);
+      if (!isfinite(sum))
+        stop(st, 4);
+      else if (sum <= c.tol2 * c.bb)
+        stop(st, 0);
       break;
     default:
       break;
@@ -450,6 +482,13 @@ __device__ __forceinline__ void grid_reduce(V v, double* sh, double* partial, Cg
   const unsigned mask = nl == 32 ? 0xffffffffu : ((1u << nl) - 1u);
   double* out = partial + (long long)cta * nseg;
   __shared__ bool last;
+  __shared__ alignas(8) unsigned char shst[sizeof(CgState)];   // for scalar_update
+  static_assert(sizeof(CgState) % 8 == 0, "copied in 8-byte words");
+  if (wid == 0) {
+    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(st);
+    for (int i = lane; i < (int)(sizeof(CgState) / 8); i += nl)
+      reinterpret_cast<unsigned long long*>(shst)[i] = ld_l2(src + i);
+  }
   if (seg <= 32) {
     V w = segment_sum(v, mask, lane, nl, seg);
     double s = sum_value(w);
@@ -495,7 +534,7 @@ __device__ __forceinline__ void grid_reduce(V v, double* sh, double* partial, Cg
   for (int l = lane; l < 32; l += nt) {
     double a = 0.0;
 #pragma unroll 8
-    for (int c = l; c < np; c += 32) a += __ldcg(partial + c);
+    for (int c = l; c < np; c += 32) a += ld_l2(partial + c);
     sh[l] = a;
   }
   __syncwarp(mask);
@@ -505,7 +544,7 @@ __device__ __forceinline__ void grid_reduce(V v, double* sh, double* partial, Cg
   }
   if (tid == 0) {
     st->ticket = 0u;
-    scalar_update(sop, st, sh[0]);
+    scalar_update(sop, st, *reinterpret_cast<const CgState*>(shst), sh[0]);
   }
 }
 

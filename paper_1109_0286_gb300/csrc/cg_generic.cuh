@@ -259,7 +259,7 @@ __device__ __forceinline__ void ld_spec(const T* spec, size_t off, int nv, bool 
     if (vec && nv == V) {
 #pragma unroll
       for (int h = 0; h < V; h += 2) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(spec + 2 * (off + h)));
+        const float4 a = *reinterpret_cast<const float4*>(spec + 2 * (off + h));
         x[h] = cx<float>{a.x, a.y};
         x[h + 1] = cx<float>{a.z, a.w};
       }
@@ -267,7 +267,7 @@ __device__ __forceinline__ void ld_spec(const T* spec, size_t off, int nv, bool 
     }
   }
 #pragma unroll
-  for (int v = 0; v < V; ++v) x[v] = v < nv ? ldg_cx<T>(spec + 2 * (off + v)) : cx<T>{(T)0, (T)0};
+  for (int v = 0; v < V; ++v) x[v] = v < nv ? ld_cx<T>(spec + 2 * (off + v)) : cx<T>{(T)0, (T)0};
 }
 template <typename T, int V>
 __device__ __forceinline__ void st_spec(T* spec, size_t off, int nv, bool vec, const cx<T> (&x)[V]) {
@@ -631,6 +631,7 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
   const InstDesc<T>& I = insts[blockIdx.y];
+  pdl_wait();
   if (skip_instance(a.check_done, I.st)) return;
   const int L = g.n, nt = g.nt, ny = a.ny;
   const int grp = threadIdx.x / nt, t = threadIdx.x - grp * nt;
@@ -701,9 +702,11 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
   if constexpr (OUT_SPEC) {
     __syncthreads();
     gen::dif<T, V>(Z, g, wl, t, g.nst);
+    pdl_trigger();
     gen::r2c<T, V>(a.spec_sel ? I.spec2 : I.spec, ny, y0, g, wx, Z, t, nt);
   }
 
+  if constexpr (!OUT_SPEC) pdl_trigger();
   if (a.sop != SC_NONE)
     grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, nt);
 }
@@ -776,6 +779,7 @@ __global__ void __launch_bounds__(kGenThreads, gen_col_minb<T>())
 k_col_gen(const InstDesc<T>* __restrict__ insts, ColArgs a, GenLen g, const T* __restrict__ wn) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const InstDesc<T>& I = insts[blockIdx.x];
+  pdl_wait();
   if (skip_instance(a.check_done, I.st)) return;
   const int N = g.n, nt = g.nt;
   const int grp = threadIdx.x / nt, t = threadIdx.x - grp * nt;
@@ -821,6 +825,7 @@ k_col_gen(const InstDesc<T>* __restrict__ insts, ColArgs a, GenLen g, const T* _
   if (a.table < 0) return;
   __syncthreads();
   gen::dit<T, V>(Z, g, wn, t, S - 1);
+  pdl_trigger();
   for (int y0 = t; y0 < N; y0 += gen::kGenChunk * nt) {
 #pragma unroll
     for (int c = 0; c < gen::kGenChunk; ++c) {
@@ -856,15 +861,11 @@ cudaError_t GenLaunch<T>::row(bool in_spec, bool out_spec, const InstDesc<T>* d,
   constexpr int V = gen_vrow<T>();
   const dim3 grid((a.ny + a.rows - 1) / a.rows, ninst), block(a.rows / V * g.nt);
   const size_t sm = row_smem(g.n, a.rows);
-  if (in_spec && out_spec)
-    k_row_gen<T, V, true, true><<<grid, block, sm, s>>>(d, a, g, wl, wx);
-  else if (in_spec)
-    k_row_gen<T, V, true, false><<<grid, block, sm, s>>>(d, a, g, wl, wx);
-  else if (a.op == OP_XI)
-    k_row_gen<T, V, false, true, true><<<grid, block, sm, s>>>(d, a, g, wl, wx);
-  else
-    k_row_gen<T, V, false, true><<<grid, block, sm, s>>>(d, a, g, wl, wx);
-  return cudaGetLastError();
+  const Launcher l{grid, block, sm, s, a.pdl != 0};
+  if (in_spec && out_spec) return l(k_row_gen<T, V, true, true>, d, a, g, wl, wx);
+  if (in_spec) return l(k_row_gen<T, V, true, false>, d, a, g, wl, wx);
+  if (a.op == OP_XI) return l(k_row_gen<T, V, false, true, true>, d, a, g, wl, wx);
+  return l(k_row_gen<T, V, false, true>, d, a, g, wl, wx);
 }
 
 template <typename T>
@@ -873,11 +874,9 @@ cudaError_t GenLaunch<T>::col(const InstDesc<T>* d, int ninst, const ColArgs& a,
   constexpr int V = gen_v<T>();
   const dim3 grid(ninst, (a.nkx + a.ffts - 1) / a.ffts), block(a.ffts / V * g.nt);
   const size_t sm = col_smem(g.n, a.ffts);
-  if (a.pre)
-    k_col_gen<T, V, true><<<grid, block, sm, s>>>(d, a, g, wn);
-  else
-    k_col_gen<T, V><<<grid, block, sm, s>>>(d, a, g, wn);
-  return cudaGetLastError();
+  const Launcher l{grid, block, sm, s, a.pdl != 0};
+  if (a.pre) return l(k_col_gen<T, V, true>, d, a, g, wn);
+  return l(k_col_gen<T, V>, d, a, g, wn);
 }
 
 template <typename T>

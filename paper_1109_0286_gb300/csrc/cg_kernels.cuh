@@ -312,7 +312,7 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
   T* sm = reinterpret_cast<T*>(smem_raw);
   __shared__ double red[32];
   const InstDesc<T>& I = insts[blockIdx.y];
-  if (skip_instance(a.check_done, I.st)) return;
+  CgState* const st = I.st;
 
   const int rows = a.rows, lr = a.log_rows;
   const int row = threadIdx.x / TT, tid = threadIdx.x - row * TT;
@@ -347,15 +347,21 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
     if (E == 16 || threadIdx.x < rows * NW)
       mws[threadIdx.x] = __ldg(I.mw + (size_t)y0 * NW + threadIdx.x);
   }
+  T* const specp = a.spec_sel ? I.spec2 : I.spec;
+  cx<T> wc{}, wr{};   // W_nx^tid (C2R), W_nx^kk (R2C)
+  if constexpr (IN_SPEC) wc = twiddle<T>(tw, tid * TWS);
+  if constexpr (OUT_SPEC) wr = twiddle<T>(tw, kk * TWS);
+  pdl_wait();
+  if (skip_instance(a.check_done, st)) return;
 
   if constexpr (IN_SPEC) {
-    const T* spec = (a.spec_sel ? I.spec2 : I.spec) + 2 * ((size_t)kk * ny + y0 + rr);
+    const T* spec = specp + 2 * ((size_t)kk * ny + y0 + rr);
     cx<T> t[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) t[i] = ld_stream_cx<T>(spec + i * tstep);
     cx<T> tn{};
     if (threadIdx.x < rows)
-      tn = ldg_cx<T>((a.spec_sel ? I.spec2 : I.spec) + 2 * ((size_t)L * ny + y0 + threadIdx.x));
+      tn = ld_cx<T>(specp + 2 * ((size_t)L * ny + y0 + threadIdx.x));
     const int tb = tix(kk, rr);
 #pragma unroll
     for (int i = 0; i < E; ++i) tile[HOIST ? tb + i * ts : tix(kk + i * TT, rr)] = t[i];
@@ -363,7 +369,6 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
     __syncthreads();
     if (threadIdx.x == 0 && !OUT_SPEC) prefetch_compact(I, a.op, mws, rows * NW);
     // C2R: Z[k] = (X[k] + conj X[L-k]) + i e^{+2 pi i k / nx} (X[k] - conj X[L-k])
-    const cx<T> wt = twiddle<T>(tw, tid * TWS);
     const int cb = tix(tid, row), cm = tix(L - tid, row);
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -374,7 +379,7 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
         xk.i = (T)0;
         xc.i = (T)0;
       }
-      const cx<T> w = cmul(wt, w32<T>(e * (16 / E)));   // W_nx^k, k = tid + e TT
+      const cx<T> w = cmul(wc, w32<T>(e * (16 / E)));   // W_nx^k, k = tid + e TT
       const cx<T> sum = xk + xc;
       const cx<T> dif = cmulc(xk - xc, w);  // (X - conj X') e^{+i...}
       v[e] = cx<T>{sum.r - dif.i, sum.i + dif.r};
@@ -413,8 +418,8 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
   } else {
     __syncthreads();   // mask words
     if (threadIdx.x == 0) prefetch_compact(I, a.op, mws, rows * NW);
-    const T alpha = a.op == OP_R_UPD ? cg_alpha<T>(I.st) : (T)0;
-    const T beta = a.op == OP_P_UPD_Z || a.op == OP_P_UPD_R ? cg_beta<T>(I.st) : (T)0;
+    const T alpha = a.op == OP_R_UPD ? cg_alpha<T>(st) : (T)0;
+    const T beta = a.op == OP_P_UPD_Z || a.op == OP_P_UPD_R ? cg_beta<T>(st) : (T)0;
     switch (a.op) {
       case OP_R_UPD: src_fill<T, TT, E, OP_R_UPD>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
       case OP_P_UPD_Z:
@@ -453,9 +458,9 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
 #pragma unroll
     for (int e = 0; e < E; ++e) tile[HOIST ? cb + e * ts : tix(tid + e * TT, row)] = v[e];
     __syncthreads();
-    const cx<T> wt = twiddle<T>(tw, kk * TWS);
-    T* spec = (a.spec_sel ? I.spec2 : I.spec) + 2 * ((size_t)kk * ny + y0 + rr);
+    T* spec = specp + 2 * ((size_t)kk * ny + y0 + rr);
     const int tb = tix(kk, rr), tm = tix(L - kk, rr);   // L - kk: the Nyquist row when kk = 0
+    pdl_trigger();
 #pragma unroll
     for (int i = 0; i < E; ++i) {
       const int k = kk + i * TT;
@@ -464,17 +469,18 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
       const cx<T> zc = conjx(tile[HOIST ? im : tix((L - k) & (L - 1), rr)]);
       const cx<T> ev = scal(zk + zc, (T)0.5);
       const cx<T> od = scal(mul_mi<T, false>(zk - zc), (T)0.5);
-      st_cx<T>(spec + i * tstep, ev + cmul(od, cmul(wt, w32<T>(i * (16 / E)))));
+      st_cx<T>(spec + i * tstep, ev + cmul(od, cmul(wr, w32<T>(i * (16 / E)))));
     }
     if (threadIdx.x < rows) {   // Nyquist: X[L] = Re Z[0] - Im Z[0]
       const cx<T> z0 = tile[tix(0, threadIdx.x)];
-      st_cx<T>((a.spec_sel ? I.spec2 : I.spec) + 2 * ((size_t)L * ny + y0 + threadIdx.x),
+      st_cx<T>(specp + 2 * ((size_t)L * ny + y0 + threadIdx.x),
                cx<T>{z0.r - z0.i, (T)0});
     }
   }
 
+  if constexpr (!OUT_SPEC) pdl_trigger();
   if (a.sop != SC_NONE)
-    grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x,
+    grid_reduce(acc.total(), red, I.partial, st, a.sop, gridDim.x, blockIdx.x,
                 min(rows, kRedRows) * TT);
 }
 
@@ -494,7 +500,7 @@ k_col(const InstDesc<T>* __restrict__ insts, ColArgs a, const T* __restrict__ tw
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
   const InstDesc<T>& I = insts[blockIdx.x];
-  if (skip_instance(a.check_done, I.st)) return;
+  CgState* const st = I.st;
   const int f = threadIdx.x / TT, tid = threadIdx.x - f * TT;
   const int kx = blockIdx.y * a.ffts + f;
   const bool act = kx < a.nkx;
@@ -502,17 +508,30 @@ k_col(const InstDesc<T>* __restrict__ insts, ColArgs a, const T* __restrict__ tw
   const XBar bar = XBar::make(TT, a.ffts, f);
   T* col = (a.spec_sel ? I.spec2 : I.spec) + 2 * (long long)(act ? kx : 0) * N;
   const T* src = PRE ? I.spec + 2 * (long long)(act ? kx : 0) * N : col;
+  const T* tab = nullptr;
+  if (a.table >= 0)
+    tab = (a.table >= 2 ? I.kt + (long long)(a.table - 2) * a.nkx * N
+           : a.table ? I.t_sqrt : I.t_inv) + (long long)(act ? kx : 0) * N;
+  // fewer elements per thread: the table's values are fetched before the wait
+  constexpr bool PT = E < 16;
+  T tv[PT ? E : 1];
+  if constexpr (PT) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) tv[e] = act && tab ? ldg1(tab + tid + e * TT) : (T)0;
+  }
+  pdl_wait();
+  if (skip_instance(a.check_done, st)) return;
   cx<T> v[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) v[e] = act ? ld_stream_cx<T>(src + 2 * (tid + e * TT)) : cx<T>{(T)0, (T)0};
   if constexpr (!PRE) fft_regs<T, LOG_N, LE, false, TAB>(v, xb, tid, tw, bar, bar);
   if (a.table >= 0) {
-    const T* tab = (a.table >= 2 ? I.kt + (long long)(a.table - 2) * a.nkx * N
-                    : a.table ? I.t_sqrt : I.t_inv) + (long long)(act ? kx : 0) * N;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const T t = act ? ldg1(tab + tid + e * TT) : (T)0;
-      v[e] = scal(v[e], t);
+      if constexpr (PT)
+        v[e] = scal_rn(v[e], tv[e]);
+      else
+        v[e] = scal(v[e], act ? ldg1(tab + tid + e * TT) : (T)0);
     }
     // the inverse transform reloads its twiddles through an opaque copy of
     // the table pointer: sharing the forward transform's loads would keep
@@ -521,6 +540,7 @@ k_col(const InstDesc<T>* __restrict__ insts, ColArgs a, const T* __restrict__ tw
     asm("mov.b64 %0, %1;" : "=l"(tw_inv) : "l"(tw));
     fft_regs<T, LOG_N, LE, true, TAB>(v, xb, tid, tw_inv, bar, bar);
   }
+  pdl_trigger();
   if (act) {
 #pragma unroll
     for (int e = 0; e < E; ++e) st_cx<T>(col + 2 * (tid + e * TT), v[e]);
@@ -640,7 +660,10 @@ k_col_tma(const InstDesc<float>* __restrict__ insts, ColArgs a, const float* __r
     const XBufSw xb(buf);
     fft_regs<float, LOG_N, LE, false, TAB>(v, xb, tid, tw, fbar, fbar);
 #pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = scal(v[e], act ? tb[tid + e * TT] : 0.f);
+    for (int e = 0; e < E; ++e) {
+      const float t = act ? tb[tid + e * TT] : 0.f;
+      v[e] = E < 16 ? scal_rn(v[e], t) : scal(v[e], t);
+    }
     // the inverse transform reloads its twiddles (an opaque copy of the table
     // pointer): keeping the forward transform's alive across the table
     // multiply would cost some 60 registers and spills
@@ -664,6 +687,7 @@ __global__ void __launch_bounds__(256)
 k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
   __shared__ double red[32];
   const InstDesc<T>& I = insts[blockIdx.y];
+  pdl_wait();
   if (skip_instance(a.check_done, I.st)) return;
   Acc<T> acc;
   const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -780,6 +804,7 @@ k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
       }
     }
   }
+  pdl_trigger();
   if (a.sop != SC_NONE)
     grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, blockDim.x);
 }

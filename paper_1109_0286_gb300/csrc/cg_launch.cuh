@@ -7,6 +7,29 @@
 
 namespace cgf {
 
+// One kernel launch, as a programmatic dependent of the kernel before it in
+// the stream if `pdl`.
+struct Launcher {
+  dim3 grid, block;
+  size_t smem;
+  cudaStream_t s;
+  bool pdl;
+  template <typename... P, typename... A>
+  cudaError_t operator()(void (*kernel)(P...), A... args) const {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+  }
+};
+
 template <typename T>
 size_t Launch<T>::row_smem(int log_l, int rows) {
   // FFT areas / transposed tile, then the mask words (8 bytes per 32 pixels)
@@ -45,15 +68,11 @@ cudaError_t row_ll(bool in_spec, bool out_spec, const InstDesc<T>* d, int ninst,
   constexpr int TT = (1 << LL) >> row_le<T>(LL);
   dim3 grid(a.ny / a.rows, ninst), block(a.rows * TT);
   const size_t sm = Launch<T>::row_smem(LL, a.rows);
-  if (in_spec && out_spec)
-    k_row<T, LL, true, true><<<grid, block, sm, s>>>(d, a, tw);
-  else if (in_spec)
-    k_row<T, LL, true, false><<<grid, block, sm, s>>>(d, a, tw);
-  else if (a.op == OP_XI)
-    k_row<T, LL, false, true, true><<<grid, block, sm, s>>>(d, a, tw);
-  else
-    k_row<T, LL, false, true><<<grid, block, sm, s>>>(d, a, tw);
-  return cudaGetLastError();
+  const Launcher l{grid, block, sm, s, a.pdl != 0};
+  if (in_spec && out_spec) return l(k_row<T, LL, true, true>, d, a, tw);
+  if (in_spec) return l(k_row<T, LL, true, false>, d, a, tw);
+  if (a.op == OP_XI) return l(k_row<T, LL, false, true, true>, d, a, tw);
+  return l(k_row<T, LL, false, true>, d, a, tw);
 }
 
 // Persistent CTAs of the TMA column pass (SMs x resident CTAs), per log2 N;
@@ -86,17 +105,16 @@ cudaError_t col_ln(const InstDesc<T>* d, int ninst, const ColArgs& a, const T* t
       b.ffts = F;
       const long long items = (long long)((a.nkx + F - 1) / F) * ninst;
       const int grid = (int)(items < g_col_tma_ctas[LN] ? items : g_col_tma_ctas[LN]);
-      k_col_tma<LN><<<grid, col_tma_threads(LN), col_tma_smem(LN, F), s>>>(d, b, tw, ninst);
-      return cudaGetLastError();
+      // (no programmatic launch: its reads go through the async proxy)
+      return Launcher{dim3(grid), dim3(col_tma_threads(LN)), col_tma_smem(LN, F), s, false}(
+          k_col_tma<LN>, d, b, tw, ninst);
     }
   }
   dim3 grid(ninst, (a.nkx + a.ffts - 1) / a.ffts), block(a.ffts * TT);
   const size_t sm = Launch<T>::col_smem(LN, a.ffts);
-  if (a.pre)
-    k_col<T, LN, true><<<grid, block, sm, s>>>(d, a, tw);
-  else
-    k_col<T, LN><<<grid, block, sm, s>>>(d, a, tw);
-  return cudaGetLastError();
+  const Launcher l{grid, block, sm, s, a.pdl != 0};
+  if (a.pre) return l(k_col<T, LN, true>, d, a, tw);
+  return l(k_col<T, LN>, d, a, tw);
 }
 
 template <typename T, int LL>
@@ -138,8 +156,7 @@ cudaError_t Launch<T>::col(int log_n, const InstDesc<T>* d, int ninst, const Col
 
 template <typename T>
 cudaError_t Launch<T>::vec(const InstDesc<T>* d, int ninst, const VecArgs& a, int nblk, cudaStream_t s) {
-  k_vec<T><<<dim3(nblk, ninst), 256, 0, s>>>(d, a);
-  return cudaGetLastError();
+  return Launcher{dim3(nblk, ninst), dim3(256), 0, s, a.pdl != 0}(k_vec<T>, d, a);
 }
 
 template <typename T>

@@ -186,6 +186,7 @@ struct RowArgs {
   int check_done;   // skip instances whose CG state is done
   int spec_sel;     // 0: spec, 1: spec2
   int param;        // op parameter (OP_KSEL: the kernel class)
+  int pdl;          // launch as a programmatic dependent of the previous kernel
 };
 
 struct ColArgs {
@@ -200,6 +201,7 @@ struct ColArgs {
   int* err;         // device error flag (set to 1 when a bounded wait gave up), or null
   int variant;      // FP32 table passes: 0 register-fed kernel, 1 persistent bulk-copy-fed
                     // kernel (chosen per grid by the autotuner)
+  int pdl;          // as RowArgs::pdl
 };
 
 // Band-binned spectral products for the band-power gradient.
@@ -218,6 +220,7 @@ struct VecArgs {
   int check_done;
   double p0, p1;    // op parameters (VOP_ANNULUS: r_in^2, r_out^2)
   int nx;           // row length (VOP_ANNULUS)
+  int pdl;          // as RowArgs::pdl
 };
 
 constexpr int kLmax = 8192;        // twiddle master table: W_8192^m

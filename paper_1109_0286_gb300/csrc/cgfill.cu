@@ -338,7 +338,28 @@ struct Ctx {
   const T* gwl = nullptr;
   const T* gwx = nullptr;
   const T* gwn = nullptr;
+  // programmatic dependent launches: a pass may start while the kernel before
+  // it in the stream still runs.  Off for the first pass after something that
+  // is no kernel of the same stream (an event, a conditional node), and for
+  // FP64 beyond 2^17 pixels: those passes are long against the launch gap, and
+  // CTAs that start early share an SM's FP64 pipe unevenly (512^2 165 without,
+  // 185 us per iteration with; 64^2 75 and 73; FP32 256^2 x 16 61 and 57;
+  // relaxation of 1024^2, launched from the host, 34 and 26 us per sweep), nor
+  // for mixed-radix grids beyond 2^19 pixels, for the same reason (375 x 1050 x 3
+  // FP32 14.6 ms without, 15.5 with; one map 13.4 and 13.3; 63 x 90 2.81 and 2.63).
+  int pdl = 1;
 };
+template <typename T>
+int use_pdl(long long npix, int ninst, bool gen) {
+  const long long most = std::is_same<T, double>::value ? 1LL << 17 : gen ? 1LL << 19 : 1LL << 62;
+  return npix * ninst <= most;
+}
+
+template <typename T>
+Ctx<T> no_pdl(Ctx<T> c) {
+  c.pdl = 0;
+  return c;
+}
 
 template <typename T>
 Ctx<T> ctx(fill_plan* p, int ninst = -1) {
@@ -346,6 +367,7 @@ Ctx<T> ctx(fill_plan* p, int ninst = -1) {
   Ctx<T> c{p->ny, p->nx, p->log_l, p->log_n, P.rows, P.ffts,
            ninst < 0 ? p->batch : ninst, p->o.precond, P.col_variant, p->npix, P.desc, P.tw,
            &p->launches, p->dev_err};
+  c.pdl = use_pdl<T>(p->npix, c.ninst, p->gen);
   if (p->gen) {
     c.grow = &p->grow;
     c.gcol = &p->gcol;
@@ -360,7 +382,7 @@ template <typename T>
 cudaError_t row(const Ctx<T>& c, cudaStream_t s, int op, int sop, bool in_spec, bool out_spec,
                 int skip, int spec_sel = 0, int param = 0) {
   ++*c.launches;
-  RowArgs a{c.ny, c.nx, c.rows, ilog2(c.rows), op, sop, skip, spec_sel, param};
+  RowArgs a{c.ny, c.nx, c.rows, ilog2(c.rows), op, sop, skip, spec_sel, param, c.pdl};
   if (c.grow)
     return GenLaunch<T>::row(in_spec, out_spec, c.desc, c.ninst, a, *c.grow, c.gwl, c.gwx, s);
   return Launch<T>::row(c.log_l, in_spec, out_spec, c.desc, c.ninst, a, c.tw, s);
@@ -370,7 +392,7 @@ template <typename T>
 cudaError_t col(const Ctx<T>& c, cudaStream_t s, int table, int skip, int spec_sel = 0,
                 int pre = 0) {
   ++*c.launches;
-  ColArgs a{c.ny, c.nx / 2 + 1, c.ffts, table, skip, spec_sel, pre, c.err, c.col_variant};
+  ColArgs a{c.ny, c.nx / 2 + 1, c.ffts, table, skip, spec_sel, pre, c.err, c.col_variant, c.pdl};
   if (c.gcol) return GenLaunch<T>::col(c.desc, c.ninst, a, *c.gcol, c.gwn, s);
   return Launch<T>::col(c.log_n, c.desc, c.ninst, a, c.tw, s);
 }
@@ -379,7 +401,7 @@ template <typename T>
 cudaError_t vec(const Ctx<T>& c, cudaStream_t s, int op, int sop, int skip, double p0 = 0.0,
                 double p1 = 0.0) {
   ++*c.launches;
-  VecArgs a{c.npix, op, sop, skip, p0, p1, c.nx};
+  VecArgs a{c.npix, op, sop, skip, p0, p1, c.nx, c.pdl};
   const long long pairs = c.npix / 2;
   const int nblk = (int)std::min<long long>((pairs + 255) / 256, 1024);
   return Launch<T>::vec(c.desc, c.ninst, a, nblk, s);
@@ -408,6 +430,12 @@ cudaError_t vec(fill_plan* p, cudaStream_t s, int op, int sop, int skip) {
 
 // Unconstrained draw and right-hand side (Sects. 2.3, 2.1):
 //   y = F^-1 sqrt(P) F xi;  b = -P_x F^-1 (1/P) F [(d - y) on U].
+// Iterations per loop body.  A body costs 8 us of its own (the control kernel
+// and the WHILE node) next to iterations of 30-60 us on small grids (64^2
+// FP32 with 1, 2, 4 iterations per body: 36, 34, 32 us per iteration);
+// iterations past the last convergence only cost their kernels' early exits.
+constexpr int kLoopUnroll = 4;
+
 template <typename T>
 cudaError_t draw_and_rhs(const Ctx<T>& c, cudaStream_t s, bool plain_cg) {
   CE(row<T>(c, s, OP_XI, SC_NONE, false, true, false));
@@ -435,10 +463,12 @@ cudaError_t pcg_start(const Ctx<T>& c, cudaStream_t s, int load_sop) {
 // One CG iteration (Sect. 2.4).  Preconditioned form with B = S S:
 //   p = z + beta p; q = A p; alpha = rho / p^T q; u += alpha p; r -= alpha q;
 //   z = S S r; beta = r^T z / rho.
+// first: the first pass follows something that is no kernel on s.
 template <typename T>
-cudaError_t pcg_iter(const Ctx<T>& c, cudaStream_t s) {
+cudaError_t pcg_iter(const Ctx<T>& c, cudaStream_t s, bool first) {
+  const Ctx<T> c0 = first ? no_pdl(c) : c;
   if (c.precond) {
-    CE(row<T>(c, s, OP_P_UPD_Z, SC_NONE, false, true, true));
+    CE(row<T>(c0, s, OP_P_UPD_Z, SC_NONE, false, true, true));
     CE(col<T>(c, s, 0, true));
     CE(row<T>(c, s, OP_Q, SC_ALPHA, true, false, true));
     CE(row<T>(c, s, OP_R_UPD, SC_RCHECK, false, true, true));
@@ -447,10 +477,17 @@ cudaError_t pcg_iter(const Ctx<T>& c, cudaStream_t s) {
     CE(col<T>(c, s, 1, true));
     return row<T>(c, s, OP_Z, SC_BETA, true, false, true);
   }
-  CE(row<T>(c, s, OP_P_UPD_R, SC_NONE, false, true, true));
+  CE(row<T>(c0, s, OP_P_UPD_R, SC_NONE, false, true, true));
   CE(col<T>(c, s, 0, true));
   CE(row<T>(c, s, OP_Q, SC_ALPHA, true, false, true));
   return vec<T>(c, s, VOP_UPDATE, SC_RCHECK_BETA, true);
+}
+
+// One loop body of a plan's lane or a group's class: kLoopUnroll iterations.
+template <typename T>
+cudaError_t pcg_body(const Ctx<T>& c, cudaStream_t s) {
+  for (int k = 0; k < kLoopUnroll; ++k) CE(pcg_iter<T>(c, s, k == 0));
+  return cudaSuccess;
 }
 
 template <typename T>
@@ -505,17 +542,17 @@ int active_lanes(const fill_plan* p) {
 }
 
 template <typename T>
-cudaError_t pcg_iter(fill_plan* p, cudaStream_t s, bool capturing = false) {
+cudaError_t pcg_body(fill_plan* p, cudaStream_t s, bool capturing = false) {
   return on_lanes(p, s, capturing, [&](int first, int count, cudaStream_t ls) {
-    return pcg_iter<T>(lane_ctx<T>(p, first, count), ls);
+    return pcg_body<T>(lane_ctx<T>(p, first, count), ls);
   });
 }
 
 // ----------------------------------------------------------------- device-side CG loop
 // A CG loop is one graph launch: a reset node, then a conditional WHILE node
-// whose body is one iteration followed by k_loop_ctl, which keeps the loop
-// going while any instance is not done -- and stops it after `limit` bodies
-// whatever the states say, so the loop always ends.
+// whose body is kLoopUnroll iterations followed by k_loop_ctl, which keeps the
+// loop going while any instance is not done -- and stops it after `limit`
+// bodies whatever the states say, so the loop always ends.
 // counter[0]: loop bodies run; counter[1]: IF bodies run (update passes).
 __global__ void k_loop_reset(int* counter) {
   counter[0] = 0;
@@ -635,7 +672,7 @@ fill_status build_iter_graph(fill_plan* p) {
   Precision<T>& P = prec<T>(p);
   if (P.iter_graph) return FILL_OK;
   return build_loop_graph(
-      p->cap, [&](cudaStream_t s) { return pcg_iter<T>(p, s, true); }, P.stp, p->batch,
+      p->cap, [&](cudaStream_t s) { return pcg_body<T>(p, s, true); }, P.stp, p->batch,
       p->loop_counter, p->o.max_iter + 4, &p->launches, &P.iter_graph, &P.iter_graph_kernels);
 }
 
@@ -646,7 +683,7 @@ fill_status run_pcg(fill_plan* p) {
   Precision<T>& P = prec<T>(p);
   if (p->o.host_loops)
     return run_loop_host(
-        p->s, [&](cudaStream_t s) { return pcg_iter<T>(p, s); }, P.stp, p->batch,
+        p->s, [&](cudaStream_t s) { return pcg_body<T>(p, s); }, P.stp, p->batch,
         p->loop_counter, p->hloop, p->o.max_iter + 4, &p->launches);
   fill_status fs = build_iter_graph<T>(p);
   if (fs != FILL_OK) return fs;
@@ -762,7 +799,7 @@ struct MixedLoop {
 
 cudaError_t mixed_update_passes(const Ctx<float>& lo, const Ctx<df>& hi, cudaStream_t s,
                                 bool reload) {
-  CE(row<df>(hi, s, OP_U64_UPD, SC_NONE, false, true, SKIP_UNLESS_UPD));
+  CE(row<df>(no_pdl(hi), s, OP_U64_UPD, SC_NONE, false, true, SKIP_UNLESS_UPD));
   CE(col<df>(hi, s, 0, SKIP_UNLESS_UPD));
   CE(row<df>(hi, s, OP_RES, SC_RES_UPD, true, false, SKIP_UNLESS_UPD));
   if (!reload) return cudaSuccess;
@@ -791,25 +828,32 @@ cudaError_t update_if(const Ctx<float>& lo, const Ctx<df>& hi, cudaStream_t s, b
 }
 
 cudaError_t mixed_iter(const Ctx<float>& lo, const Ctx<df>& hi, cudaStream_t s,
-                       const MixedLoop& m) {
+                       const MixedLoop& m, bool first) {
+  const Ctx<float> lo0 = first ? no_pdl(lo) : lo;
   if (!lo.precond) {
-    CE(row<float>(lo, s, OP_P_UPD_R, SC_NONE, false, true, SKIP_DONE));
+    CE(row<float>(lo0, s, OP_P_UPD_R, SC_NONE, false, true, SKIP_DONE));
     CE(col<float>(lo, s, 0, SKIP_DONE));
     CE(row<float>(lo, s, OP_Q, SC_ALPHA, true, false, SKIP_DONE));
     CE(vec<float>(lo, s, VOP_UPDATE, SC_RCHECK_UPD, SKIP_DONE));
     CE(update_if(lo, hi, s, false, m));
     // plain CG: z = r, so beta = r^T r / rho (the reload pass also reduces ||r||^2)
-    return row<float>(lo, s, OP_LOAD_R, SC_BETA, false, true, SKIP_DONE);
+    return row<float>(no_pdl(lo), s, OP_LOAD_R, SC_BETA, false, true, SKIP_DONE);
   }
-  CE(row<float>(lo, s, OP_P_UPD_Z, SC_NONE, false, true, SKIP_DONE));
+  CE(row<float>(lo0, s, OP_P_UPD_Z, SC_NONE, false, true, SKIP_DONE));
   CE(col<float>(lo, s, 0, SKIP_DONE));
   CE(row<float>(lo, s, OP_Q, SC_ALPHA, true, false, SKIP_DONE));
   CE(row<float>(lo, s, OP_R_UPD, SC_RCHECK_UPD, false, true, SKIP_DONE));
   CE(update_if(lo, hi, s, true, m));
-  CE(col<float>(lo, s, 1, SKIP_DONE));
+  CE(col<float>(no_pdl(lo), s, 1, SKIP_DONE));
   CE(row<float>(lo, s, OP_MASK, SC_NONE, true, true, SKIP_DONE));
   CE(col<float>(lo, s, 1, SKIP_DONE));
   return row<float>(lo, s, OP_Z, SC_BETA, true, false, SKIP_DONE);
+}
+
+cudaError_t mixed_body(const Ctx<float>& lo, const Ctx<df>& hi, cudaStream_t s,
+                       const MixedLoop& m) {
+  for (int k = 0; k < kLoopUnroll; ++k) CE(mixed_iter(lo, hi, s, m, k == 0));
+  return cudaSuccess;
 }
 
 // Before a mixed loop (b, r and r32 set, the high-precision states holding
@@ -843,18 +887,18 @@ cudaError_t mixed_finish(const Ctx<float>& lo, const Ctx<df>& hi, cudaStream_t s
   return cudaGetLastError();
 }
 
-cudaError_t mixed_iter(fill_plan* p, cudaStream_t s, bool capturing) {
+cudaError_t mixed_body(fill_plan* p, cudaStream_t s, bool capturing) {
   return on_lanes(p, s, capturing, [&](int first, int count, cudaStream_t ls) {
     const MixedLoop m{p->h.stp + first, count, p->loop_counter, p->cap2, p->o.host_loops != 0,
                       &p->if_kernels};
-    return mixed_iter(lane_ctx<float>(p, first, count), lane_ctx<df>(p, first, count), ls, m);
+    return mixed_body(lane_ctx<float>(p, first, count), lane_ctx<df>(p, first, count), ls, m);
   });
 }
 
 fill_status build_mixed_graph(fill_plan* p) {
   if (p->mixed_graph) return FILL_OK;
   return build_loop_graph(
-      p->cap, [&](cudaStream_t s) { return mixed_iter(p, s, true); }, p->f.stp, p->batch,
+      p->cap, [&](cudaStream_t s) { return mixed_body(p, s, true); }, p->f.stp, p->batch,
       p->loop_counter, p->o.max_iter + 4, &p->launches, &p->mixed_graph, &p->mixed_graph_kernels);
 }
 
@@ -865,13 +909,13 @@ fill_status mixed_reliable(fill_plan* p, double tol) {
   fill_status fs;
   if (p->o.host_loops) {
     fs = run_loop_host(
-        p->s, [&](cudaStream_t s) { return mixed_iter(p, s, false); }, p->f.stp, p->batch,
+        p->s, [&](cudaStream_t s) { return mixed_body(p, s, false); }, p->f.stp, p->batch,
         p->loop_counter, p->hloop, p->o.max_iter + 4, &p->launches);
   } else {
     fs = build_mixed_graph(p);
     if (fs != FILL_OK) return fs;
     fs = run_loop_graph(p, p->mixed_graph, p->mixed_graph_kernels, p->if_kernels,
-                        active_lanes(p));
+                        active_lanes(p) * kLoopUnroll);
   }
   if (fs != FILL_OK) return fs;
   CK(mixed_finish(ctx<float>(p), ctx<df>(p), p->s));
@@ -2538,6 +2582,7 @@ Ctx<T> gctx(fill_group* g, GroupClass& c, bool hi = false) {
            c.ninst, g->precond, hi ? c.col_variant_hi : c.col_variant, c.npix,
            reinterpret_cast<const InstDesc<T>*>(hi ? c.desc_hi : c.desc), prec<T>(p0).tw,
            &g->launches, p0->dev_err};
+  x.pdl = use_pdl<T>(c.npix, c.ninst, p0->gen);
   if (p0->gen) {   // mixed-radix grid: the class shares the first plan's transforms
     x.grow = &p0->grow;
     x.gcol = &p0->gcol;
@@ -2630,13 +2675,13 @@ MixedLoop group_mixed_loop(fill_group* g, GroupClass& c, bool host_loops) {
   return MixedLoop{c.stp_hi, c.ninst, g->counter, g->cap2, host_loops, &g->if_kernels};
 }
 
-// One iteration of every class of a mixed group (class streams forked from
+// One loop body of every class of a mixed group (class streams forked from
 // and joined back to s).
-cudaError_t group_mixed_iter(fill_group* g, cudaStream_t s, cudaEvent_t fork, bool host_loops) {
+cudaError_t group_mixed_body(fill_group* g, cudaStream_t s, cudaEvent_t fork, bool host_loops) {
   CE(cudaEventRecord(fork, s));
   for (auto& c : g->cls) {
     CE(cudaStreamWaitEvent(c.cs, fork, 0));
-    CE(mixed_iter(gctx<float>(g, c), gctx<df>(g, c, true), c.cs, group_mixed_loop(g, c, host_loops)));
+    CE(mixed_body(gctx<float>(g, c), gctx<df>(g, c, true), c.cs, group_mixed_loop(g, c, host_loops)));
     CE(cudaEventRecord(c.join, c.cs));
     CE(cudaStreamWaitEvent(s, c.join, 0));
   }
@@ -2644,7 +2689,7 @@ cudaError_t group_mixed_iter(fill_group* g, cudaStream_t s, cudaEvent_t fork, bo
 }
 
 // The group's CG loop graph: every loop body forks the size classes onto
-// their streams (parallel branches), runs one iteration of each, and joins.
+// their streams (parallel branches), runs its iterations, and joins.
 template <typename T>
 fill_status group_build_graph(fill_group* g) {
   if (g->graph) return FILL_OK;
@@ -2654,7 +2699,7 @@ fill_status group_build_graph(fill_group* g) {
         CE(cudaEventRecord(g->fork_cap, cap));
         for (auto& c : g->cls) {
           CE(cudaStreamWaitEvent(c.cs, g->fork_cap, 0));
-          CE(pcg_iter<T>(gctx<T>(g, c), c.cs));
+          CE(pcg_body<T>(gctx<T>(g, c), c.cs));
           CE(cudaEventRecord(c.join, c.cs));
           CE(cudaStreamWaitEvent(cap, c.join, 0));
         }
@@ -2668,7 +2713,7 @@ fill_status group_build_graph(fill_group* g) {
 fill_status group_build_mixed_graph(fill_group* g) {
   if (g->graph) return FILL_OK;
   return build_loop_graph(
-      g->cap, [&](cudaStream_t cap) { return group_mixed_iter(g, cap, g->fork_cap, false); },
+      g->cap, [&](cudaStream_t cap) { return group_mixed_body(g, cap, g->fork_cap, false); },
       g->stp, g->ntot, g->counter, g->max_iter + 4, &g->launches, &g->graph, &g->graph_kernels);
 }
 
@@ -2722,7 +2767,7 @@ fill_status group_realize_t(fill_group* g, const void* const* d, const uint64_t*
           CE(cudaEventRecord(g->fork, s));
           for (auto& c : g->cls) {
             CE(cudaStreamWaitEvent(c.cs, g->fork, 0));
-            CE(pcg_iter<T>(gctx<T>(g, c), c.cs));
+            CE(pcg_body<T>(gctx<T>(g, c), c.cs));
             CE(cudaEventRecord(c.join, c.cs));
             CE(cudaStreamWaitEvent(s, c.join, 0));
           }
@@ -2814,7 +2859,7 @@ fill_status group_realize_mixed(fill_group* g, const void* const* d, const uint6
   if (fs != FILL_OK) return fs;
   if (g->host_loops) {
     fs = run_loop_host(
-        g->s, [&](cudaStream_t s) { return group_mixed_iter(g, s, g->fork, true); }, g->stp,
+        g->s, [&](cudaStream_t s) { return group_mixed_body(g, s, g->fork, true); }, g->stp,
         g->ntot, g->counter, g->hloop, g->max_iter + 4, &g->launches);
     if (fs != FILL_OK) return fs;
   } else {
@@ -2842,7 +2887,7 @@ fill_status group_realize_mixed(fill_group* g, const void* const* d, const uint6
   CK(queue_err_readback(p0));
   CK(cudaStreamSynchronize(g->s));
   if (!g->host_loops) {
-    const long long ifk = g->if_kernels, ncls = (long long)g->cls.size();
+    const long long ifk = g->if_kernels, ncls = (long long)g->cls.size() * kLoopUnroll;
     g->launches += 1 + (long long)g->hloop[0] * (g->graph_kernels - ncls * ifk) +
                    (long long)g->hloop[1] * ifk;
   }
