@@ -357,7 +357,7 @@ __device__ __forceinline__ void r2c(T* spec, int ny, int y0, const GenLen& g, co
 // words first, then every operand load, then the arithmetic and stores, so
 // the loads of a chunk are in flight together.
 
-struct Opnd {   // one pixel pair: mask flags, compact indices, pixel index
+struct Opnd {   // one pixel pair: mask flags, CG-vector index, pixel index
   PairIdx q;
   int pix;
   bool ok;
@@ -446,9 +446,9 @@ __device__ __forceinline__ void sink_op(const InstDesc<T>& I, const Opnd& o, con
   } else if constexpr (OP == OP_B) {
     a0 = m0 ? -a0 : (T)0;
     a1 = m1 ? -a1 : (T)0;
-    stc(I.r, q, a0, a1);
-    if (I.b) stc(I.b, q, a0, a1);
-    if (I.r32) stc(I.r32, q, a0, a1);
+    stc_act(I.r, q, a0, a1);
+    if (I.b) stc_act(I.b, q, a0, a1);
+    if (I.r32) stc_act(I.r32, q, a0, a1);
     acc.add_prod(a0, a0);
     acc.add_prod(a1, a1);
   } else if constexpr (OP == OP_RES) {
@@ -533,7 +533,7 @@ __device__ __forceinline__ void src_rows(const InstDesc<T>& I, int pix0, int nx,
     for (int c = 0; c < CH; ++c)
 #pragma unroll
       for (int v = 0; v < V; ++v)
-        if (C) o[c][v].ok = o[c][v].ok && (o[c][v].q.m0 || o[c][v].q.m1);
+        if (C) o[c][v].ok = o[c][v].ok && o[c][v].q.any();
     T x[CH][V][8];
 #pragma unroll
     for (int c = 0; c < CH; ++c)
@@ -568,7 +568,7 @@ __device__ __forceinline__ void sink_rows(const InstDesc<T>& I, int pix0, int nx
     for (int c = 0; c < CH; ++c)
 #pragma unroll
       for (int v = 0; v < V; ++v)
-        if (C) o[c][v].ok = o[c][v].ok && (o[c][v].q.m0 || o[c][v].q.m1);
+        if (C) o[c][v].ok = o[c][v].ok && (OP == OP_B ? o[c][v].q.act : o[c][v].q.any());
     T x[CH][V][2];
 #pragma unroll
     for (int c = 0; c < CH; ++c)

@@ -32,21 +32,27 @@ template <> struct KCfg<float> { static constexpr int kMaxThreads = 1024; };
 template <> struct KCfg<double> { static constexpr int kMaxThreads = 512; };
 template <> struct KCfg<df> { static constexpr int kMaxThreads = 512; };
 
-// Masked flags and compact CG-vector indices of the pixel pair (pix, pix+1)
-// (pix even) from the pair's mask word: a popcount.
+// Masked flags and CG-vector index of the pixel pair (pix, pix+1), pix even,
+// from the pair's mask word.  The CG vectors hold 32 values for every mask word
+// with a masked pixel, zero on its observed pixels, so a pair is one aligned
+// vector access at the word's offset plus the pair's place in the word.
+// (One value per masked pixel packed the vectors more tightly, but took a
+// popcount and two predicated 4-byte accesses per pair and vector.)
 struct PairIdx {
   bool m0, m1;   // pixel masked (to fill)
-  int i0, i1;    // compact indices (valid where masked)
+  bool act;      // the word has a masked pixel: the vectors hold the pair
+  int i;         // index of the pair's first value (valid where act)
+  __device__ __forceinline__ bool any() const { return m0 || m1; }
 };
 
 __device__ __forceinline__ PairIdx pair_from_word(uint2 w, int pix) {
-  const int b = (int)(pix & 31);
-  const uint32_t mb = ~w.x;
+  const int b = pix & 31;
+  const uint32_t t = ~w.x >> b;
   PairIdx q;
-  q.m0 = (mb >> b) & 1u;
-  q.m1 = (mb >> (b + 1)) & 1u;
-  q.i0 = (int)w.y + __popc(mb & ((1u << b) - 1u));
-  q.i1 = q.i0 + (q.m0 ? 1 : 0);
+  q.m0 = t & 1u;
+  q.m1 = t & 2u;
+  q.act = ~w.x != 0u;
+  q.i = (int)w.y + b;
   return q;
 }
 
@@ -66,21 +72,32 @@ __device__ __forceinline__ void observed_at(const uint2* mwr, int j, bool& o0, b
   o1 = (ob >> (b + 1)) & 1u;
 }
 
-// Compact loads / stores of a pixel pair (zero / nothing on observed pixels).
+// CG-vector loads / stores of a pixel pair (nothing for a pair without a
+// masked pixel, whose values are zero).  stc expects zeros on observed
+// pixels; stc_act also writes the zeros of an active word's other pairs.
 template <typename T, typename S>
 __device__ __forceinline__ void ldc(const S* v, const PairIdx& q, T& a0, T& a1) {
-  a0 = q.m0 ? (T)v[q.i0] : (T)0;
-  a1 = q.m1 ? (T)v[q.i1] : (T)0;
+  a0 = (T)0;
+  a1 = (T)0;
+  if (q.any()) {
+    S s0, s1;
+    ld_pair(v + q.i, s0, s1);
+    a0 = (T)s0;
+    a1 = (T)s1;
+  }
 }
 template <typename T, typename S>
 __device__ __forceinline__ void stc(S* v, const PairIdx& q, T a0, T a1) {
-  if (q.m0) v[q.i0] = (S)a0;
-  if (q.m1) v[q.i1] = (S)a1;
+  if (q.any()) st_pair(v + q.i, (S)a0, (S)a1);
+}
+template <typename T, typename S>
+__device__ __forceinline__ void stc_act(S* v, const PairIdx& q, T a0, T a1) {
+  if (q.act) st_pair(v + q.i, (S)a0, (S)a1);
 }
 
-// The compact CG-vector elements of a CTA's rows form one contiguous range
-// [c0, c1) (vectors are stored in row-major order of the masked pixels): its
-// first word's offset, and the last word's offset plus its masked count.
+// The CG-vector elements of a CTA's rows form one contiguous range [c0, c1)
+// (the words with masked pixels in row-major order): its first word's offset,
+// and the last word's offset plus its 32 values if it has a masked pixel.
 // One thread asks the copy engine to bring the ranges the op will read into
 // L2, so that the per-pixel-pair gathers later in the pass hit L2 instead of
 // waiting on HBM one chunk after another.
@@ -88,7 +105,7 @@ template <typename T>
 __device__ __forceinline__ void prefetch_compact(const InstDesc<T>& I, int op, const uint2* mws,
                                                  int nwords) {
   const uint2 w0 = mws[0], w1 = mws[nwords - 1];
-  const long long c0 = w0.y, c1 = (long long)w1.y + __popc(~w1.x);
+  const long long c0 = w0.y, c1 = (long long)w1.y + (~w1.x ? 32 : 0);
   switch (op) {
     case OP_R_UPD:
       prefetch_l2(I.r, c0, c1);
@@ -115,73 +132,91 @@ __device__ __forceinline__ void prefetch_compact(const InstDesc<T>& I, int op, c
 // A source fills v[e] = (x[2j], x[2j+1]), j = tid + e TT, with the real row
 // values fed to the forward transform.  One instantiation per op: a chunk of
 // CK pixel pairs issues all its loads (indices come from shared memory, so
-// they do not wait on a global load) before its arithmetic and stores.
+// they do not wait on a global load) before its arithmetic and stores.  The r
+// update skips the pairs of a warp (64 pixels of a row) without a masked pixel
+// by a branch that the whole warp takes: on the 4096^2 wide cut (a band and
+// 2000 discs) that is 63% of them (8 maps: 497 -> 453 us with it; the p
+// update, with half the work per pair, 331 -> 352, so it has none).
 template <typename T, int TT, int E, int OP>
 __device__ __forceinline__ void src_fill(const InstDesc<T>& I, const uint2* mwr, int rowpix,
                                          int tid, T alpha, T beta, cx<T> (&v)[E], Acc<T>& acc) {
   constexpr int CK = (OP == OP_R_UPD || OP == OP_U64_UPD) ? src_chunk_wide<E>() : src_chunk<E>();
+  constexpr bool C = OP == OP_R_UPD || OP == OP_P_UPD_Z || OP == OP_P_UPD_R || OP == OP_LOAD_R ||
+                     OP == OP_LOAD_U || OP == OP_U64_UPD;
+  constexpr bool SKIP = OP == OP_R_UPD || OP == OP_U64_UPD;
+  const unsigned warp = __activemask();
 #pragma unroll
   for (int h = 0; h < E; h += CK) {
     PairIdx q[CK];
+    bool on[CK];
     T x0[CK], x1[CK], y0[CK], y1[CK], z0[CK], z1[CK], w0[CK], w1[CK];
 #pragma unroll
     for (int e = 0; e < CK; ++e) {
       const int j = tid + (h + e) * TT;
+      on[e] = true;
       if constexpr (OP == OP_LOAD_W || OP == OP_LOAD_W_MASK || OP == OP_LOAD_Y) {
         ld_pair((OP == OP_LOAD_Y ? I.y : I.w) + rowpix + 2 * j, x0[e], x1[e]);
         if constexpr (OP == OP_LOAD_W_MASK) q[e] = pair_at(mwr, j);
       } else {
         q[e] = pair_at(mwr, j);
         if constexpr (OP == OP_LOAD_D_U) ld_map_pair<T>(I.d + rowpix + 2 * j, x0[e], x1[e]);
-        if constexpr (OP == OP_LOAD_R) ldc(I.r, q[e], x0[e], x1[e]);
-        if constexpr (OP == OP_LOAD_U) ldc(I.u, q[e], x0[e], x1[e]);
-        if constexpr (OP == OP_P_UPD_Z || OP == OP_P_UPD_R) {
-          ldc(OP == OP_P_UPD_Z ? I.z : I.r, q[e], x0[e], x1[e]);
-          ldc(I.p, q[e], y0[e], y1[e]);
-        }
-        if constexpr (OP == OP_R_UPD) {
-          ldc(I.r, q[e], x0[e], x1[e]);
-          ldc(I.q, q[e], y0[e], y1[e]);
-          ldc(I.u, q[e], z0[e], z1[e]);
-          ldc(I.p, q[e], w0[e], w1[e]);
-        }
-        if constexpr (OP == OP_U64_UPD) {
-          ldc(I.u, q[e], x0[e], x1[e]);
-          ldc(I.dlt, q[e], y0[e], y1[e]);
+        if constexpr (SKIP) on[e] = __any_sync(warp, q[e].any());
+        if (C && on[e]) {
+          if constexpr (OP == OP_LOAD_R) ldc(I.r, q[e], x0[e], x1[e]);
+          if constexpr (OP == OP_LOAD_U) ldc(I.u, q[e], x0[e], x1[e]);
+          if constexpr (OP == OP_P_UPD_Z || OP == OP_P_UPD_R) {
+            ldc(OP == OP_P_UPD_Z ? I.z : I.r, q[e], x0[e], x1[e]);
+            ldc(I.p, q[e], y0[e], y1[e]);
+          }
+          if constexpr (OP == OP_R_UPD) {
+            ldc(I.r, q[e], x0[e], x1[e]);
+            ldc(I.q, q[e], y0[e], y1[e]);
+            ldc(I.u, q[e], z0[e], z1[e]);
+            ldc(I.p, q[e], w0[e], w1[e]);
+          }
+          if constexpr (OP == OP_U64_UPD) {
+            ldc(I.u, q[e], x0[e], x1[e]);
+            ldc(I.dlt, q[e], y0[e], y1[e]);
+          }
         }
       }
     }
 #pragma unroll
     for (int e = 0; e < CK; ++e) {
-      T a0, a1;
+      T a0 = (T)0, a1 = (T)0;
       if constexpr (OP == OP_LOAD_W_MASK) {
         a0 = q[e].m0 ? x0[e] : (T)0;
         a1 = q[e].m1 ? x1[e] : (T)0;
       } else if constexpr (OP == OP_LOAD_D_U) {
         a0 = q[e].m0 ? (T)0 : x0[e];
         a1 = q[e].m1 ? (T)0 : x1[e];
-      } else if constexpr (OP == OP_P_UPD_Z || OP == OP_P_UPD_R) {
-        a0 = x0[e] + beta * y0[e];
-        a1 = x1[e] + beta * y1[e];
-        stc(I.p, q[e], a0, a1);
-      } else if constexpr (OP == OP_R_UPD) {
-        a0 = x0[e] - alpha * y0[e];
-        a1 = x1[e] - alpha * y1[e];
-        stc(I.r, q[e], a0, a1);
-        stc(I.u, q[e], z0[e] + alpha * w0[e], z1[e] + alpha * w1[e]);
-        acc.add_prod(a0, a0);
-        acc.add_prod(a1, a1);
-      } else if constexpr (OP == OP_U64_UPD) {
-        a0 = x0[e] + y0[e];
-        a1 = x1[e] + y1[e];
-        stc(I.u, q[e], a0, a1);
-        stc(I.dlt, q[e], 0.f, 0.f);   // folded
-      } else {
+      } else if constexpr (!C) {
         a0 = x0[e];
         a1 = x1[e];
-        if constexpr (OP == OP_LOAD_R) {
+      } else if (on[e]) {
+        if constexpr (OP == OP_P_UPD_Z || OP == OP_P_UPD_R) {
+          a0 = x0[e] + beta * y0[e];
+          a1 = x1[e] + beta * y1[e];
+          stc(I.p, q[e], a0, a1);
+        } else if constexpr (OP == OP_R_UPD) {
+          a0 = x0[e] - alpha * y0[e];
+          a1 = x1[e] - alpha * y1[e];
+          stc(I.r, q[e], a0, a1);
+          stc(I.u, q[e], z0[e] + alpha * w0[e], z1[e] + alpha * w1[e]);
           acc.add_prod(a0, a0);
           acc.add_prod(a1, a1);
+        } else if constexpr (OP == OP_U64_UPD) {
+          a0 = x0[e] + y0[e];
+          a1 = x1[e] + y1[e];
+          stc(I.u, q[e], a0, a1);
+          stc(I.dlt, q[e], 0.f, 0.f);   // folded
+        } else {
+          a0 = x0[e];
+          a1 = x1[e];
+          if constexpr (OP == OP_LOAD_R) {
+            acc.add_prod(a0, a0);
+            acc.add_prod(a1, a1);
+          }
         }
       }
       v[h + e] = cx<T>{a0, a1};
@@ -215,10 +250,10 @@ __device__ __forceinline__ void sink_fill(const InstDesc<T>& I, const uint2* mwr
     for (int e = 0; e < CK; ++e) {
       const int j = tid + (h + e) * TT;
       const bool m0 = q[e].m0, m1 = q[e].m1;   // masked = not observed
-      // compact-vector ops: nothing to store or add (exactly) for a pair
-      // without a masked pixel
+      // CG-vector ops: nothing to store or add (exactly) for a pair without a
+      // masked pixel (the right-hand side also sets the zeros of its words)
       constexpr bool C = OP == OP_Q || OP == OP_Z || OP == OP_B || OP == OP_RES || OP == OP_KSEL;
-      if (C && !(m0 || m1)) continue;
+      if (C && !(OP == OP_B ? q[e].act : q[e].any())) continue;
       T a0 = v[h + e].r, a1 = v[h + e].i;
       if constexpr (OP == OP_Q || OP == OP_Z) {
         a0 = m0 ? a0 : (T)0;
@@ -229,9 +264,9 @@ __device__ __forceinline__ void sink_fill(const InstDesc<T>& I, const uint2* mwr
       } else if constexpr (OP == OP_B) {
         a0 = m0 ? -a0 : (T)0;
         a1 = m1 ? -a1 : (T)0;
-        stc(I.r, q[e], a0, a1);
-        if (I.b) stc(I.b, q[e], a0, a1);
-        if (I.r32) stc(I.r32, q[e], a0, a1);
+        stc_act(I.r, q[e], a0, a1);
+        if (I.b) stc_act(I.b, q[e], a0, a1);
+        if (I.r32) stc_act(I.r32, q[e], a0, a1);
         acc.add_prod(a0, a0);
         acc.add_prod(a1, a1);
       } else if constexpr (OP == OP_RES) {
@@ -693,7 +728,7 @@ k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
   const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long gstride = (long long)gridDim.x * blockDim.x;
   if (a.op == VOP_UPDATE || a.op == VOP_ZERO_UP) {
-    // compact CG vectors: one element per masked pixel
+    // the CG vectors, elementwise (zero on observed pixels)
     const T alpha = cg_alpha<T>(I.st);
     for (long long i = gid; i < I.nvec; i += gstride) {
       if (a.op == VOP_ZERO_UP) {
@@ -792,9 +827,9 @@ k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
           ld_map_pair<T>(I.gx + pix, g0, g1);
           g0 = q.m0 ? g0 : (T)0;
           g1 = q.m1 ? g1 : (T)0;
-          stc(I.r, q, g0, g1);
-          stc(I.b, q, g0, g1);
-          if (I.r32) stc(I.r32, q, g0, g1);
+          stc_act(I.r, q, g0, g1);
+          stc_act(I.b, q, g0, g1);
+          if (I.r32) stc_act(I.r32, q, g0, g1);
           acc.add_prod(g0, g0);
           acc.add_prod(g1, g1);
           break;

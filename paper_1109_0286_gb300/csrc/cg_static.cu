@@ -114,7 +114,7 @@ __global__ void k_static_setup(unsigned char* base, Layout L, int ny, int nx, co
       const long long i = w * 32 + b;
       if (i < npix && (observed == nullptr || observed[i])) word |= 1u << b;
     }
-    bits[w] = make_uint2(word, 0u);   // compact offsets unused by these passes
+    bits[w] = make_uint2(word, 0u);   // CG-vector offsets unused by these passes
   }
   if (tid == 0) {
     CgState* st = reinterpret_cast<CgState*>(base + L.st);

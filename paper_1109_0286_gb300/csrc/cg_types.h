@@ -2,15 +2,17 @@
 //
 // Layout on the device, per realization ("instance"):
 //   * full maps (d, y, w, out, gx): row-major ny x nx;
-//   * CG vectors (r, p, q, z, u, b and the mixed-mode r32 / dlt): COMPACT,
-//     one value per masked pixel in row-major order (the masked system of
+//   * CG vectors (r, p, q, z, u, b and the mixed-mode r32 / dlt): COMPACT, 32
+//     values for every mask word with a masked pixel, in row-major order of
+//     the words, zero on the word's observed pixels (the masked system of
 //     Sect. 2.4 lives on M only; the vectors are zero on U);
 //   * half spectrum "spec": transposed, (nx/2+1) rows of ny complex values,
 //     spec[kx * ny + y]; the column pass runs along contiguous rows;
 //   * spectral tables [kx][ky] (same transposed layout), real, with the
 //     1/n of the inverse DFT folded in;
-//   * mask words: for each 32 pixels, the observed bits (1 = constraint) and
-//     the compact index of the word's first masked pixel.
+//   * mask words: for each 32 pixels, the observed bits (1 = constraint, also
+//     beyond the last pixel) and the index of the word's values in the CG
+//     vectors (the values of all words before it).
 #pragma once
 #include <cstdint>
 
@@ -82,7 +84,7 @@ struct MapOf<df> {
 // Per-instance pointers handed to every kernel (element type T of the pass).
 template <typename T>
 struct InstDesc {
-  const uint2* mw;         // mask words: x = observed bits, y = compact offset
+  const uint2* mw;         // mask words: x = observed bits, y = CG-vector offset
   const T* t_inv;          // 1 / (n P)     [kx][ky]
   const T* t_sqrt;         // sqrt(P) / n   [kx][ky]
   T* spec;                 // interleaved complex half spectrum, transposed
@@ -106,7 +108,7 @@ struct InstDesc {
   double* coef;            // CG coefficients (2 hist_cap entries), or null
   const T* kt;             // kernel tables [j][kx][ky] of the Sect. 6.3 solver, or null
   const uint8_t* cls;      // kernel class of every pixel (Sect. 6.3 solver), or null
-  long long nvec;          // compact CG-vector length: masked pixels of this instance
+  long long nvec;          // CG-vector length: 32 per word with a masked pixel
   unsigned long long seed;
 };
 

@@ -162,8 +162,9 @@ struct fill_plan {
   cudaStream_t lane_s[kMaxLanes] = {};
   cudaEvent_t lane_join[kMaxLanes] = {};
   cudaEvent_t lane_fork = nullptr, lane_fork_cap = nullptr;
-  uint2* mw = nullptr;           // mask words: observed bits, compact offset
-  long long nv = 0;              // compact vector stride per instance (>= nmasked)
+  uint2* mw = nullptr;           // mask words: observed bits, CG-vector offset
+  long long nvec = 0;            // CG-vector length: 32 per mask word with a masked pixel
+  long long nv = 0;              // CG-vector stride per instance (>= nvec)
   std::vector<double> P_half;    // host copy of the spectrum
   double* P_dev = nullptr;       // device copy (fill_set_spectrum builds the tables from it)
   double* sig_dev = nullptr;     // device copy of the band templates' S(k) (fill_set_bands)
@@ -1327,8 +1328,7 @@ fill_status setup_precision(fill_plan* p, const std::vector<double>& tinv,
       CK(cudaMemcpy(P.tw + 2 * size_t(r[0]), w.data(), w.size() * sizeof(T), cudaMemcpyHostToDevice));
     }
   }
-  CK(cudaMemset(P.u, 0, B * nv * sizeof(T)));
-  CK(cudaMemset(P.p, 0, B * nv * sizeof(T)));
+  for (T** v : cvecs) CK(cudaMemset(*v, 0, B * nv * sizeof(T)));
   if (p->gen) {
     fill_status gs = setup_generic<T>(p);
     if (gs != FILL_OK) return gs;
@@ -1345,7 +1345,7 @@ fill_status setup_precision(fill_plan* p, const std::vector<double>& tinv,
   for (size_t i = 0; i < B; ++i) {
     InstDesc<T> D{};
     D.mw = p->mw;
-    D.nvec = p->nmasked;
+    D.nvec = p->nvec;
     D.t_inv = P.t_inv;
     D.t_sqrt = P.t_sqrt;
     D.spec = P.spec + i * nspec;
@@ -1482,19 +1482,19 @@ fill_status fill_init(fill_plan** out, int ny, int nx, const double* P_half,
   const int nkx = nx / 2 + 1;
   if (!spectrum_valid(ny, nx, P_half)) return FILL_EINVAL;
   const long long npix = (long long)ny * nx;
-  long long nmasked = 0;
+  long long nmasked = 0, nvec = 0;
   std::vector<uint2> words((npix + 31) / 32, make_uint2(0u, 0u));
   for (long long w = 0; w < (long long)words.size(); ++w) {
-    words[w].y = (unsigned int)nmasked;   // compact index of the word's first masked pixel
+    words[w].y = (unsigned int)nvec;   // index of the word's values in the CG vectors
     for (int b = 0; b < 32; ++b) {
       const long long i = w * 32 + b;
-      if (i >= npix) break;
-      if (observed[i] > 1) return FILL_EINVAL;
-      if (observed[i])
+      if (i < npix && observed[i] > 1) return FILL_EINVAL;
+      if (i >= npix || observed[i])
         words[w].x |= 1u << b;
       else
         ++nmasked;
     }
+    if (~words[w].x) nvec += 32;
   }
   fill_plan* p = new (std::nothrow) fill_plan();
   if (!p) return FILL_ENOMEM;
@@ -1508,7 +1508,8 @@ fill_status fill_init(fill_plan** out, int ny, int nx, const double* P_half,
   p->batch = o.batch;
   p->npix = npix;
   p->nmasked = nmasked;
-  p->nv = std::max<long long>(64, (nmasked + 63) / 64 * 64);
+  p->nvec = nvec;
+  p->nv = std::max<long long>(64, (nvec + 63) / 64 * 64);
   p->o = o;
   p->s = reinterpret_cast<cudaStream_t>(stream);
   p->P_half.assign(P_half, P_half + (size_t)ny * nkx);
