@@ -11,7 +11,7 @@
 // round trip.  Between stages data goes through shared memory (XBuf).  The
 // twiddles W^(jm r), r = 1..E-1, of a stage come from the stage's own table of
 // correctly rounded values (stw_* in cg_types.h), or (E = 16 columns in FP32)
-// from three master table entries and complex products (TAB = false).
+// from three of the table's entries and complex products (TAB = false).
 //
 // E trades the exchanges against the length of a thread's instruction chain:
 // E = 16 for the large FP32 and double-float grids, which fill the chip and
@@ -249,8 +249,8 @@ struct XBar {
   }
 };
 
-// TAB: twiddles from the per-stage tables (the row passes: 5-11% faster at
-// 4096^2), else from three entries of the master table and complex products
+// TAB: every twiddle from the per-stage tables (the row passes: 5-11% faster at
+// 4096^2), else three of them and complex products
 // (the E = 16 FP32 column passes: the tables' loads raise their register
 // pressure into spills, 21% slower).
 template <typename T, int LOG_L, int LE, bool INV, bool TAB = true, typename XB>
@@ -313,13 +313,15 @@ __device__ __forceinline__ void fft_regs(cx<T> (&v)[1 << LE], const XB& xb, int 
           if (G > 1) asm volatile("" ::: "memory");
         }
       } else {
-        // W^(jm r) from three master-table entries (W^jm, W^4jm, W^8jm) and at
-        // most four complex products each (a few ulp)
-        const int stride = kLmax / (ns * 16);
+        // W^(jm r) from the stage table's rows r = 1, 4, 8 and at most four
+        // complex products each (a few ulp).  (The strided entries of the
+        // master table took up to 32 L1 wavefronts per load: 1600 of a
+        // 4096-point column's 4850, the L1 data pipe being its limit at 71%.)
+        const T* ts = tw + 2 * (kLmax + stw_base(LE, LOG_L) + stw_stage_off(LE, LOG_L, s) + jm);
         cx<T> w[16];
-        w[1] = twiddle<T>(tw, jm * stride);
-        w[4] = twiddle<T>(tw, 4 * jm * stride);
-        w[8] = twiddle<T>(tw, 8 * jm * stride);
+        w[1] = ldg_cx<T>(ts);
+        w[4] = ldg_cx<T>(ts + 2 * 3 * ns);
+        w[8] = ldg_cx<T>(ts + 2 * 7 * ns);
         w[2] = cmul(w[1], w[1]);
         w[3] = cmul(w[2], w[1]);
         w[5] = cmul(w[4], w[1]);
