@@ -326,16 +326,44 @@ __device__ __forceinline__ void mid_fill(const InstDesc<T>& I, const uint2* mwr,
 
 // ----------------------------------------------------------------- row pass
 // CTA = `rows` consecutive grid rows, L/E threads per row; blockIdx.y is the
-// instance.  Shared memory: per-row FFT exchange areas, aliased with the
-// transposed tile [(L+1) x rows] used for the spectrum load / store,
-// then the rows' mask words (nx/32 = L/16 per row).
+// instance.  Shared memory: per-row FFT exchange areas, which also hand the
+// row between its FFT threads (row, tid) and the threads (kk, rr) that load
+// and store the transposed half spectrum, then the rows' mask words (nx/32 =
+// L/16 per row).
+//
+// Half spectrum <-> half-length transform: thread (kk, rr) takes k = kk + i TT
+// (i < E/2, so k < L/2) together with L - k of row rr.  Z[k] and Z[L-k], and X[k]
+// and X[L-k], follow from one another, so each step is one write and one read
+// of the exchange area and one complex product per pair (two rows per thread
+// in 16-byte accesses measured 3% slower):
+//   s = X[k] + conj X[L-k], d = e^{+2 pi i k/nx} (X[k] - conj X[L-k]):
+//     Z[k] = s + i d, Z[L-k] = conj(s) + i conj(d);
+//   ev = (Z[k] + conj Z[L-k]) / 2, od = e^{-2 pi i k/nx} (-i/2)(Z[k] - conj Z[L-k]):
+//     X[k] = ev + od, X[L-k] = conj(ev - od);
+// k = 0 pairs with the Nyquist row L (Z[L] = Z[0]); k = L/2 is its own partner.
+// The passes are bound by the L1 data pipe (shared-memory and global
+// wavefronts; at 4096^2 77% of its peak in the middle pass, 72% in the p
+// update) and by the barriers.  Against a tile in shared memory, written once
+// and read twice with a CTA barrier on either side: FP32 passes at 8 x 4096^2
+// sink 377 -> 349, middle 511 -> 451, r update 454 -> 447 us; 1024^2 x 16 middle
+// 52 -> 47; 512^2 FP64 164 -> 152 us per iteration.
 // XI: the source is the seed's white noise (kept out of the other source
 // kernels, whose register allocation it would otherwise burden).
+
+// Exchange area of one row, in 8-byte words: XBuf's L + L/16 + 1 complex
+// elements, padded so that the areas of a CTA's rows start 16 / rows words
+// apart modulo the banks: 16 lanes of (kk, rr) -- 16 / rows consecutive k of
+// every row -- then touch 16 different 8-byte banks.
+template <typename T>
+__host__ __device__ __forceinline__ int row_area_words(int log_l, int rows) {
+  const int L = 1 << log_l, padl = L + L / 16 + 1;
+  const int words = sizeof(T) == 4 ? padl : 2 * padl;
+  const int want = rows < 16 ? 16 / rows : 1;
+  return words + ((want - words) & 15);
+}
 template <typename T>
 __host__ __device__ __forceinline__ size_t row_main_bytes(int log_l, int rows) {
-  const size_t L = size_t(1) << log_l, padl = L + L / 16 + 1;
-  const size_t fft = size_t(rows) * 2 * padl, tile = 2 * (L + 1) * size_t(rows);
-  return ((fft > tile ? fft : tile) * sizeof(T) + 15) & ~size_t(15);
+  return (size_t(rows) * row_area_words<T>(log_l, rows) * 8 + 15) & ~size_t(15);
 }
 
 template <typename T, int LOG_L, bool IN_SPEC, bool OUT_SPEC, bool XI = false>
@@ -353,28 +381,17 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
   const int row = threadIdx.x / TT, tid = threadIdx.x - row * TT;
   const int y0 = blockIdx.x * rows, y = y0 + row;
   const int ny = a.ny;
-  const XBuf<T> xb(sm + row * 2 * PADL, PADL);
-  // transposed tile [(L+1)][rows], aliases the FFT areas; column r of row k at
-  // k rows + (r ^ g(k)), g(k) = (k >> gs) & (rows - 1): both the
-  // consecutive-k accesses of one row and the (k, r) sweep of the global
-  // loads / stores are free of bank conflicts
-  cx<T>* tile = reinterpret_cast<cx<T>*>(sm);
-  const int gs = lr < 4 ? 4 - lr : 0;
-  auto tix = [&](int k, int r) { return (k << lr) + (r ^ ((k >> gs) & (rows - 1))); };
+  constexpr int W8 = 8 / sizeof(T);             // T values per 8-byte word
+  const int area = row_area_words<T>(LOG_L, rows) * W8;
+  const XBuf<T> xb(sm + row * area, PADL);      // this thread's row
   uint2* mws = reinterpret_cast<uint2*>(smem_raw + row_main_bytes<T>(LOG_L, rows));
   const uint2* mwr = mws + row * NW;            // this row's mask words
   constexpr int TWS = kLmax / (2 * L);          // W_{nx}^k = table[k * TWS]
   const int rowpix = y * a.nx;
-  // tile element (kk + i TT, rr) for i = 0..E-1 belongs to thread (kk, rr); the
-  // Nyquist row k = L to threads 0..rows-1
+  // half-spectrum side: pairs (k, L - k), k = kk + i TT, of row rr
   const int rr = threadIdx.x & (rows - 1), kk = threadIdx.x >> lr;
   const size_t tstep = 2 * (size_t)TT * ny;
-  // With TT >= 32, TT is a multiple of 2^max(lr, 4) (rows * TT <= 1024), so
-  // adding multiples of TT to k leaves the swizzle bits g(k) unchanged: a
-  // thread's tile indices for k0 + i TT are one base plus i (TT rows).
-  constexpr bool HOIST = TT >= 32;
-  const int ts = TT << lr;
-  const XBar cta{0, 0}, rbar = XBar::make(TT, rows, row);   // CTA / this row's barrier
+  const XBar rbar = XBar::make(TT, rows, row);   // this row's barrier
   cx<T> v[E];
   Acc<T> acc;
 
@@ -383,44 +400,42 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
       mws[threadIdx.x] = __ldg(I.mw + (size_t)y0 * NW + threadIdx.x);
   }
   T* const specp = a.spec_sel ? I.spec2 : I.spec;
-  cx<T> wc{}, wr{};   // W_nx^tid (C2R), W_nx^kk (R2C)
-  if constexpr (IN_SPEC) wc = twiddle<T>(tw, tid * TWS);
-  if constexpr (OUT_SPEC) wr = twiddle<T>(tw, kk * TWS);
+  cx<T> wk{};   // W_nx^kk
+  if constexpr (IN_SPEC || OUT_SPEC) wk = twiddle<T>(tw, kk * TWS);
   pdl_wait();
   if (skip_instance(a.check_done, st)) return;
 
   if constexpr (IN_SPEC) {
-    const T* spec = specp + 2 * ((size_t)kk * ny + y0 + rr);
-    cx<T> t[E];
+    // rows kk and L - kk of the half spectrum, stepping up and down by TT rows
+    const T* speck = specp + 2 * ((size_t)kk * ny + y0 + rr);
+    const T* specm = specp + 2 * ((size_t)(L - kk) * ny + y0 + rr);
+    const XBuf<T> xs(sm + rr * area, PADL);
+    cx<T> xk[E / 2], xm[E / 2], xh{};
 #pragma unroll
-    for (int i = 0; i < E; ++i) t[i] = ld_stream_cx<T>(spec + i * tstep);
-    cx<T> tn{};
-    if (threadIdx.x < rows)
-      tn = ld_cx<T>(specp + 2 * ((size_t)L * ny + y0 + threadIdx.x));
-    const int tb = tix(kk, rr);
+    for (int i = 0; i < E / 2; ++i) {
+      xk[i] = ld_stream_cx<T>(speck + i * tstep);
+      xm[i] = ld_stream_cx<T>(specm - i * tstep);
+    }
+    if (kk == 0) {
+      xh = ld_stream_cx<T>(specp + 2 * ((size_t)(L / 2) * ny + y0 + rr));
+      xk[0].i = (T)0;   // X[0] and X[L] are real
+      xm[0].i = (T)0;
+    }
 #pragma unroll
-    for (int i = 0; i < E; ++i) tile[HOIST ? tb + i * ts : tix(kk + i * TT, rr)] = t[i];
-    if (threadIdx.x < rows) tile[tix(L, threadIdx.x)] = tn;
+    for (int i = 0; i < E / 2; ++i) {
+      const int k = kk + i * TT;
+      const cx<T> w = cmul(wk, w32<T>(i * (16 / E)));   // W_nx^k
+      const cx<T> xc = conjx(xm[i]);
+      const cx<T> s = xk[i] + xc, d = cmulc(xk[i] - xc, w);
+      xs.st(k, cx<T>{s.r - d.i, s.i + d.r});
+      xs.st(L - k, cx<T>{s.r + d.i, d.r - s.i});   // (k = 0: the unused slot L)
+    }
+    if (kk == 0) xs.st(L / 2, cx<T>{xh.r + xh.r, -(xh.i + xh.i)});
     __syncthreads();
     if (threadIdx.x == 0 && !OUT_SPEC) prefetch_compact(I, a.op, mws, rows * NW);
-    // C2R: Z[k] = (X[k] + conj X[L-k]) + i e^{+2 pi i k / nx} (X[k] - conj X[L-k])
-    const int cb = tix(tid, row), cm = tix(L - tid, row);
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int k = tid + e * TT;
-      cx<T> xk = tile[HOIST ? cb + e * ts : tix(k, row)];
-      cx<T> xc = conjx(tile[HOIST ? cm - e * ts : tix(L - k, row)]);
-      if (k == 0) {
-        xk.i = (T)0;
-        xc.i = (T)0;
-      }
-      const cx<T> w = cmul(wc, w32<T>(e * (16 / E)));   // W_nx^k, k = tid + e TT
-      const cx<T> sum = xk + xc;
-      const cx<T> dif = cmulc(xk - xc, w);  // (X - conj X') e^{+i...}
-      v[e] = cx<T>{sum.r - dif.i, sum.i + dif.r};
-    }
-    // the first exchange overwrites tile entries other rows still read
-    fft_regs<T, LOG_L, LE, true>(v, xb, tid, tw, cta, rbar);
+    for (int e = 0; e < E; ++e) v[e] = xb.ld(tid + e * TT);
+    fft_regs<T, LOG_L, LE, true>(v, xb, tid, tw, rbar, rbar);
     // v[e] = x[2j] + i x[2j+1], j = tid + e TT
     if constexpr (OUT_SPEC) {
       if (a.op == OP_Y_W)
@@ -485,32 +500,37 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
 
   if constexpr (OUT_SPEC) {
     fft_regs<T, LOG_L, LE, false>(v, xb, tid, tw, rbar, rbar);
-    // Z (the half-length transform) into the transposed tile; the threads of
-    // the global stores form X from Z[k] and Z[L-k]:
-    // R2C: X[k] = (Z[k] + conj Z[L-k]) / 2 - (i/2) e^{-2 pi i k/nx} (Z[k] - conj Z[L-k])
-    __syncthreads();   // the tile overwrites other rows' exchange areas
-    const int cb = tix(tid, row);
+    rbar.sync();   // the row's last exchange has been read
 #pragma unroll
-    for (int e = 0; e < E; ++e) tile[HOIST ? cb + e * ts : tix(tid + e * TT, row)] = v[e];
+    for (int e = 0; e < E; ++e) xb.st(tid + e * TT, v[e]);
     __syncthreads();
-    T* spec = specp + 2 * ((size_t)kk * ny + y0 + rr);
-    const int tb = tix(kk, rr), tm = tix(L - kk, rr);   // L - kk: the Nyquist row when kk = 0
     pdl_trigger();
+    // (the middle pass recomputes what it would otherwise keep in registers
+    // through both transforms)
+    unsigned t2 = threadIdx.x;
+    const T* tw2 = tw;
+    if constexpr (IN_SPEC) {
+      asm volatile("" : "+r"(t2));
+      asm volatile("" : "+l"(tw2));
+    }
+    const int rr2 = t2 & (rows - 1), kk2 = t2 >> lr;
+    const XBuf<T> xs(sm + rr2 * area, PADL);
+    if constexpr (IN_SPEC) wk = twiddle<T>(tw2, kk2 * TWS);
+    T* speck = specp + 2 * ((size_t)kk2 * ny + y0 + rr2);
+    T* specm = specp + 2 * ((size_t)(L - kk2) * ny + y0 + rr2);
 #pragma unroll
-    for (int i = 0; i < E; ++i) {
-      const int k = kk + i * TT;
-      const cx<T> zk = tile[HOIST ? tb + i * ts : tix(k, rr)];
-      const int im = (i == 0 && kk == 0) ? tix(0, rr) : tm - i * ts;
-      const cx<T> zc = conjx(tile[HOIST ? im : tix((L - k) & (L - 1), rr)]);
+    for (int i = 0; i < E / 2; ++i) {
+      const int k = kk2 + i * TT;
+      const cx<T> zk = xs.ld(k);
+      const cx<T> zc = conjx(xs.ld(i == 0 && kk2 == 0 ? 0 : L - k));
+      const cx<T> w = cmul(wk, w32<T>(i * (16 / E)));   // W_nx^k
       const cx<T> ev = scal(zk + zc, (T)0.5);
-      const cx<T> od = scal(mul_mi<T, false>(zk - zc), (T)0.5);
-      st_cx<T>(spec + i * tstep, ev + cmul(od, cmul(wr, w32<T>(i * (16 / E)))));
+      const cx<T> od = cmul(scal(mul_mi<T, false>(zk - zc), (T)0.5), w);
+      st_cx<T>(speck + i * tstep, ev + od);
+      st_cx<T>(specm - i * tstep, conjx(ev - od));
     }
-    if (threadIdx.x < rows) {   // Nyquist: X[L] = Re Z[0] - Im Z[0]
-      const cx<T> z0 = tile[tix(0, threadIdx.x)];
-      st_cx<T>(specp + 2 * ((size_t)L * ny + y0 + threadIdx.x),
-               cx<T>{z0.r - z0.i, (T)0});
-    }
+    if (kk2 == 0)
+      st_cx<T>(specp + 2 * ((size_t)(L / 2) * ny + y0 + rr2), conjx(xs.ld(L / 2)));
   }
 
   if constexpr (!OUT_SPEC) pdl_trigger();
