@@ -1,8 +1,7 @@
 // Mixed-radix pass kernels (radix 2, 3, 4, 5, 7, 8, in-place DIF / DIT
 // transforms) and their launchers; see cg_generic.h.  The fused operations
-// are those of cg_kernels.cuh, applied per pixel pair; mask flags and compact
-// indices come from the global mask words (a row need not start on a word
-// boundary here).
+// are those of cg_kernels.cuh, applied per pixel pair; mask flags and CG-vector
+// indices come from the rows' mask words, staged in shared memory.
 #pragma once
 #include "cg_generic.h"
 #include "cg_launch.cuh"
@@ -138,7 +137,7 @@ __device__ __forceinline__ void stage(cx<T>* z, int ns, int h, int nb, const T* 
   const int dblk = nt / h, dj = nt - dblk * h;
   for (int b = t; b < nb; b += nt) {
     cx<T>* p = z + (blk * ns + j) * V;
-    const T* wj = tws + 2 * (j * (R - 1));
+    const T* wj = tws + 2 * j;
     cx<T> v[V][R];
 #pragma unroll
     for (int m = 0; m < R; ++m) {
@@ -151,7 +150,7 @@ __device__ __forceinline__ void stage(cx<T>* z, int ns, int h, int nb, const T* 
       if (twd) {
 #pragma unroll
         for (int m = 1; m < R; ++m) {
-          const cx<T> w = ldg_cx<T>(wj + 2 * (m - 1));
+          const cx<T> w = ldg_cx<T>(wj + 2 * (m - 1) * h);
 #pragma unroll
           for (int u = 0; u < V; ++u) v[u][m] = cmulc(v[u][m], w);
         }
@@ -163,7 +162,7 @@ __device__ __forceinline__ void stage(cx<T>* z, int ns, int h, int nb, const T* 
       if (twd) {
 #pragma unroll
         for (int m = 1; m < R; ++m) {
-          const cx<T> w = ldg_cx<T>(wj + 2 * (m - 1));
+          const cx<T> w = ldg_cx<T>(wj + 2 * (m - 1) * h);
 #pragma unroll
           for (int u = 0; u < V; ++u) v[u][m] = cmul(v[u][m], w);
         }
@@ -247,6 +246,9 @@ __device__ __forceinline__ cx<T> r2c_one(cx<T> zk, cx<T> zm, cx<T> w) {
 }
 
 constexpr int kGenChunk = 4;
+
+// Mask words that a row of nx pixels can touch.
+__host__ __device__ __forceinline__ int row_words(int nx) { return nx / 32 + 2; }
 
 // Rows y0 .. y0 + V - 1 of half-spectrum row k (element offset off = k ny + y0):
 // one 16-byte access per two FP32 rows when ny is even (off is then even) and
@@ -504,31 +506,51 @@ struct CompactOnly {
 // thread (one shared-memory slot), CH = kGenChunk / V pairs at a time: mask
 // words first, then every operand load, then the arithmetic and stores.
 // Operands of pairs j = j0 + c nt of the group's rows (row v starts at pixel
-// pix0 + v nx); rows at or beyond ny (v >= nv) are not ok and read the mask
-// word of pixel 0.
+// pix0 + v nx); rows at or beyond ny (v >= nv) are not ok and read the row's
+// first word.
 template <int V, int CH, bool WORD>
-__device__ __forceinline__ void chunk_words(const uint2* mw, int pix0, int nx, int nv, int j0,
+__device__ __forceinline__ void chunk_words(const uint2* mws, int pix0, int nx, int nv, int j0,
                                             int nt, int L, Opnd (&o)[CH][V]) {
 #pragma unroll
   for (int c = 0; c < CH; ++c)
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const int j = j0 + c * nt;
+      const int first = pix0 + v * nx;
       o[c][v].ok = j < L && v < nv;
-      o[c][v].pix = o[c][v].ok ? pix0 + v * nx + 2 * j : 0;   // pixel 0: a valid dummy
-      if (WORD) o[c][v].q = pair_index(mw, o[c][v].pix);
+      o[c][v].pix = o[c][v].ok ? first + 2 * j : 0;   // pixel 0: a valid dummy
+      if (WORD) {
+        const int w = o[c][v].ok ? (o[c][v].pix >> 5) - (first >> 5) : 0;
+        o[c][v].q = pair_from_word(mws[v * row_words(nx) + w], o[c][v].pix);
+      }
     }
 }
 
+// The mask words of the group's rows into shared memory (row v's from the word
+// of its first pixel on; a row need not start on a word boundary), so that the
+// elementwise loops do not wait for one global load after another.  Word 0 of
+// rows outside the grid is set too (read, not used).
+template <int V>
+__device__ __forceinline__ void stage_words(const uint2* mw, uint2* mws, int pix0, int nx, int nv,
+                                            int t, int nt) {
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const int first = pix0 + v * nx, w0 = first >> 5;
+    const int n = v < nv ? ((first + nx - 1) >> 5) - w0 + 1 : 0;
+    for (int i = t; i < max(n, 1); i += nt)
+      mws[v * row_words(nx) + i] = i < n ? __ldg(mw + w0 + i) : make_uint2(~0u, 0u);
+  }
+}
+
 template <typename T, int OP, int V>
-__device__ __forceinline__ void src_rows(const InstDesc<T>& I, int pix0, int nx, int nv, cx<T>* z,
+__device__ __forceinline__ void src_rows(const InstDesc<T>& I, const uint2* mws, int pix0, int nx, int nv, cx<T>* z,
                                          int L, int t, int nt, T alpha, T beta, Acc<T>& acc) {
   constexpr bool W = !(OP == OP_LOAD_W || OP == OP_LOAD_Y);
   constexpr bool C = CompactOnly<OP>::value;
   constexpr int CH = kGenChunk / V;
   for (int j0 = t; j0 < L; j0 += CH * nt) {
     Opnd o[CH][V];
-    chunk_words<V, CH, W>(I.mw, pix0, nx, nv, j0, nt, L, o);
+    chunk_words<V, CH, W>(mws, pix0, nx, nv, j0, nt, L, o);
 #pragma unroll
     for (int c = 0; c < CH; ++c)
 #pragma unroll
@@ -556,14 +578,14 @@ __device__ __forceinline__ void src_rows(const InstDesc<T>& I, int pix0, int nx,
 }
 
 template <typename T, int OP, int V>
-__device__ __forceinline__ void sink_rows(const InstDesc<T>& I, int pix0, int nx, int nv,
-                                          const cx<T>* z, int L, int t, int nt, Acc<T>& acc,
+__device__ __forceinline__ void sink_rows(const InstDesc<T>& I, const uint2* mws, int pix0,
+                                          int nx, int nv, const cx<T>* z, int L, int t, int nt, Acc<T>& acc,
                                           int param) {
   constexpr bool C = CompactOnly<OP>::value;
   constexpr int CH = kGenChunk / V;
   for (int j0 = t; j0 < L; j0 += CH * nt) {
     Opnd o[CH][V];
-    chunk_words<V, CH, true>(I.mw, pix0, nx, nv, j0, nt, L, o);
+    chunk_words<V, CH, true>(mws, pix0, nx, nv, j0, nt, L, o);
 #pragma unroll
     for (int c = 0; c < CH; ++c)
 #pragma unroll
@@ -591,12 +613,12 @@ __device__ __forceinline__ void sink_rows(const InstDesc<T>& I, int pix0, int nx
 }
 
 template <typename T, int OP, int V>
-__device__ __forceinline__ void mid_rows(const InstDesc<T>& I, int pix0, int nx, int nv, cx<T>* z,
+__device__ __forceinline__ void mid_rows(const InstDesc<T>& I, const uint2* mws, int pix0, int nx, int nv, cx<T>* z,
                                          int L, int t, int nt) {
   constexpr int CH = kGenChunk / V;
   for (int j0 = t; j0 < L; j0 += CH * nt) {
     Opnd o[CH][V];
-    chunk_words<V, CH, true>(I.mw, pix0, nx, nv, j0, nt, L, o);
+    chunk_words<V, CH, true>(mws, pix0, nx, nv, j0, nt, L, o);
     T d[CH][V][2];
 #pragma unroll
     for (int c = 0; c < CH; ++c)
@@ -619,11 +641,17 @@ __device__ __forceinline__ void mid_rows(const InstDesc<T>& I, int pix0, int nx,
 
 }  // namespace gen
 
+// Shared memory of the values of a CTA's rows (the mask words follow).
+template <typename T>
+__host__ __device__ __forceinline__ size_t gen_row_main(int L, int rows) {
+  return (size_t(rows) * L * sizeof(cx<T>) + 15) & ~size_t(15);
+}
+
 // ----------------------------------------------------------------- row pass
 // CTA = a.rows consecutive grid rows in groups of V (one group per g.nt
 // threads; blockIdx.y is the instance), rows at or beyond ny (odd ny) idle.
 // Shared memory: L complex values per row, interleaved [position][V] within a
-// group.
+// group, then the rows' mask words.
 template <typename T, int V, bool IN_SPEC, bool OUT_SPEC, bool XI = false>
 __global__ void __launch_bounds__(kGenThreads, gen_minb<T>())
 k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* __restrict__ wl,
@@ -631,27 +659,30 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
   const InstDesc<T>& I = insts[blockIdx.y];
-  pdl_wait();
-  if (skip_instance(a.check_done, I.st)) return;
   const int L = g.n, nt = g.nt, ny = a.ny;
   const int grp = threadIdx.x / nt, t = threadIdx.x - grp * nt;
   const int y0 = blockIdx.x * a.rows + grp * V;
   const int nv = min(V, ny - y0);   // rows of this group inside the grid
   cx<T>* Z = reinterpret_cast<cx<T>*>(smem_raw) + grp * L * V;
+  uint2* mws = reinterpret_cast<uint2*>(smem_raw + gen_row_main<T>(L, a.rows)) +
+               grp * V * gen::row_words(a.nx);
   Acc<T> acc;
 
   const int pix0 = y0 * a.nx;
+  if constexpr (!XI) gen::stage_words<V>(I.mw, mws, pix0, a.nx, nv, t, nt);
+  pdl_wait();
+  if (skip_instance(a.check_done, I.st)) return;
   if constexpr (IN_SPEC) {
     gen::c2r<T, V>(a.spec_sel ? I.spec2 : I.spec, ny, y0, g, wx, Z, t, nt);
     __syncthreads();
     gen::dit<T, V>(Z, g, wl, t, g.nst);   // Z[j] = x[2j] + i x[2j+1] (scaled)
 #define CGF_SINK(OPC, PARAM) \
-  gen::sink_rows<T, OPC, V>(I, pix0, a.nx, nv, Z, L, t, nt, acc, PARAM)
+  gen::sink_rows<T, OPC, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt, acc, PARAM)
     if constexpr (OUT_SPEC) {
       if (a.op == OP_Y_W)
-        gen::mid_rows<T, OP_Y_W, V>(I, pix0, a.nx, nv, Z, L, t, nt);
+        gen::mid_rows<T, OP_Y_W, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt);
       else
-        gen::mid_rows<T, OP_MASK, V>(I, pix0, a.nx, nv, Z, L, t, nt);
+        gen::mid_rows<T, OP_MASK, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt);
     } else {
       switch (a.op) {
         case OP_Q: CGF_SINK(OP_Q, 0); break;
@@ -678,9 +709,10 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
       }
     }
   } else {
+    __syncthreads();   // mask words
     const T alpha = a.op == OP_R_UPD ? cg_alpha<T>(I.st) : (T)0;
     const T beta = a.op == OP_P_UPD_Z || a.op == OP_P_UPD_R ? cg_beta<T>(I.st) : (T)0;
-#define CGF_SRC(OPC) gen::src_rows<T, OPC, V>(I, pix0, a.nx, nv, Z, L, t, nt, alpha, beta, acc)
+#define CGF_SRC(OPC) gen::src_rows<T, OPC, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt, alpha, beta, acc)
     switch (a.op) {
       case OP_R_UPD: CGF_SRC(OP_R_UPD); break;
       case OP_P_UPD_Z: CGF_SRC(OP_P_UPD_Z); break;
@@ -842,8 +874,11 @@ k_col_gen(const InstDesc<T>* __restrict__ insts, ColArgs a, GenLen g, const T* _
 
 // ----------------------------------------------------------------- launchers
 template <typename T>
+size_t GenLaunch<T>::row_main(int L, int rows) { return gen_row_main<T>(L, rows); }
+
+template <typename T>
 size_t GenLaunch<T>::row_smem(int L, int rows) {
-  return size_t(rows) * L * sizeof(cx<T>);
+  return gen_row_main<T>(L, rows) + size_t(rows) * gen::row_words(2 * L) * sizeof(uint2);
 }
 
 template <typename T>

@@ -49,8 +49,9 @@ struct GenLen {
   int code;   // radix schedule (gen_factor)
   int radix[kGenMaxStages];
   // Stage s < nst - 1: twiddles W_{n_s}^{q j} (j < h_s, q = 1 .. R_s - 1) at
-  // complex entry twoff[s] + j (R_s - 1) + q - 1 of the table.  The last stage
-  // (h = 1) has none.
+  // complex entry twoff[s] + (q - 1) h_s + j of the table, so that the threads
+  // of a warp (consecutive j) read consecutive entries.  The last stage (h = 1)
+  // has none.
   int twoff[kGenMaxStages];
   const unsigned short* rev;   // device, n entries: position -> frequency
   const unsigned short* pos;   // device, n entries: frequency -> position
@@ -107,7 +108,8 @@ struct GenLaunch {
                          cudaStream_t s);
   static cudaError_t col(const InstDesc<T>* d, int ninst, const ColArgs& a, const GenLen& g,
                          const T* wn, cudaStream_t s);
-  static size_t row_smem(int L, int rows);
+  static size_t row_smem(int L, int rows);   // row_main and the rows' mask words
+  static size_t row_main(int L, int rows);   // the rows' values
   static size_t col_smem(int ny, int ffts);
   static int max_threads();
   static cudaError_t prepare();

@@ -747,13 +747,16 @@ k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
   Acc<T> acc;
   const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long gstride = (long long)gridDim.x * blockDim.x;
-  if (a.op == VOP_UPDATE || a.op == VOP_ZERO_UP) {
+  if (a.op == VOP_UPDATE || a.op == VOP_ZERO_UP || a.op == VOP_NORM_R) {
     // the CG vectors, elementwise (zero on observed pixels)
     const T alpha = cg_alpha<T>(I.st);
     for (long long i = gid; i < I.nvec; i += gstride) {
       if (a.op == VOP_ZERO_UP) {
         I.u[i] = (T)0;
         I.p[i] = (T)0;
+      } else if (a.op == VOP_NORM_R) {
+        const T r = I.r[i];
+        acc.add_prod(r, r);
       } else {
         const T r = I.r[i] - alpha * I.q[i];
         I.r[i] = r;

@@ -176,6 +176,7 @@ enum VecOp : int {
   VOP_W_TO_OUT = 11,  // out = w (pass element type -> caller's map)
   VOP_ANNULUS = 12,   // w = 1 where r_in^2 < |offset|^2 <= r_out^2 (offset from pixel 0), else 0
   VOP_Y_TO_W_M = 13,  // w = y on M; acc ||y - w||^2 over M
+  VOP_NORM_R = 14,    // acc ||r||^2
 };
 
 // Launch arguments of the pass kernels.

@@ -452,7 +452,7 @@ cudaError_t pcg_start(const Ctx<T>& c, cudaStream_t s, int load_sop) {
   if (!c.precond) {
     if (load_sop == SC_NONE) return cudaSuccess;
     // plain CG inner solve: rho = bb = ||r||^2, beta = 0
-    return row<T>(c, s, OP_LOAD_R, SC_BB_RHO, false, true, true);
+    return vec<T>(c, s, VOP_NORM_R, SC_BB_RHO, true);
   }
   CE(row<T>(c, s, OP_LOAD_R, load_sop, false, true, true));
   CE(col<T>(c, s, 1, true));
@@ -837,8 +837,10 @@ cudaError_t mixed_iter(const Ctx<float>& lo, const Ctx<df>& hi, cudaStream_t s,
     CE(row<float>(lo, s, OP_Q, SC_ALPHA, true, false, SKIP_DONE));
     CE(vec<float>(lo, s, VOP_UPDATE, SC_RCHECK_UPD, SKIP_DONE));
     CE(update_if(lo, hi, s, false, m));
-    // plain CG: z = r, so beta = r^T r / rho (the reload pass also reduces ||r||^2)
-    return row<float>(no_pdl(lo), s, OP_LOAD_R, SC_BETA, false, true, SKIP_DONE);
+    // plain CG: z = r, so beta = r^T r / rho (r as the update left it; a norm of
+    // the masked pixels only, in place of a whole forward row pass whose
+    // spectrum nothing read: 80 of 425 us per iteration at 600 x 7000 x 4)
+    return vec<float>(no_pdl(lo), s, VOP_NORM_R, SC_BETA, SKIP_DONE);
   }
   CE(row<float>(lo0, s, OP_P_UPD_Z, SC_NONE, false, true, SKIP_DONE));
   CE(col<float>(lo, s, 0, SKIP_DONE));
@@ -1073,8 +1075,8 @@ void gen_tables(const GenLen& g, std::vector<double>& tw, std::vector<unsigned s
   int ns = n;
   for (int s = 0; s < S - 1; ++s) {
     const int R = g.radix[s], h = ns / R, step = n / ns;
-    for (int j = 0; j < h; ++j)
-      for (int q = 1; q < R; ++q) push(w, (int)(((long long)q * j * step) % n));
+    for (int q = 1; q < R; ++q)
+      for (int j = 0; j < h; ++j) push(w, (int)(((long long)q * j * step) % n));
     ns = h;
   }
   // position p = sum_s q_s h_s holds frequency k = sum_s q_s R_0 ... R_{s-1}
@@ -1136,12 +1138,12 @@ bool loop_precision(const fill_plan* p) {
 // Validity of a mixed-radix CTA shape for precision T: rows per CTA and
 // column FFTs per CTA are multiples of the group width V = gen_v<T>(), the
 // row groups a power of two, within kGenThreads threads, the partial-sum slots
-// and 200 KB of shared memory.
+// and 200 KB of shared memory (the mask words take up to 13 KB more).
 template <typename T>
 bool gen_row_ok(const fill_plan* p, int r) {
   constexpr int V = gen_vrow<T>();
   return r >= V && r % V == 0 && pow2(r / V) && (r / V) * p->grow.nt <= GenLaunch<T>::max_threads() &&
-         (p->ny + r - 1) / r <= kMaxPartials && GenLaunch<T>::row_smem(p->nx / 2, r) <= 200 * 1024;
+         (p->ny + r - 1) / r <= kMaxPartials && GenLaunch<T>::row_main(p->nx / 2, r) <= 200 * 1024;
 }
 template <typename T>
 bool gen_col_ok(const fill_plan* p, int f) {
@@ -1197,20 +1199,22 @@ fill_status gen_upload_maps(fill_plan* p) {
 }
 
 // Mixed-radix schedule and twiddle tables of one precision: rows per CTA
-// and column FFTs per CTA (one or two groups of g.nt threads, within 75 KB of
-// shared memory so that three CTAs share an SM), unless the options fix them;
-// the digit-reversal maps once per plan.
+// and column FFTs per CTA (groups of g.nt threads, within 75 KB of shared
+// memory so that three CTAs share an SM, and no more than leaves two CTAs per
+// SM), unless the options fix them; the digit-reversal maps once per plan.
 template <typename T>
 fill_status setup_generic(fill_plan* p) {
   Precision<T>& P = prec<T>(p);
   constexpr int V = gen_v<T>(), VR = gen_vrow<T>();
   const size_t third = 75 * 1024;
+  const int ctas = 2 * 152;
   const bool user = loop_precision<T>(p);
   if (user && p->o.rows_per_cta > 0) {
     P.rows = p->o.rows_per_cta;
   } else {
     P.rows = VR;
-    if (gen_row_ok<T>(p, 2 * VR) && GenLaunch<T>::row_smem(p->nx / 2, 2 * VR) <= third)
+    if (gen_row_ok<T>(p, 2 * VR) && GenLaunch<T>::row_smem(p->nx / 2, 2 * VR) <= third &&
+        (long long)p->ny * p->batch >= 2LL * VR * ctas)
       P.rows = 2 * VR;
   }
   if (user && p->o.ffts_per_cta > 0) {
@@ -1218,7 +1222,7 @@ fill_status setup_generic(fill_plan* p) {
   } else {
     P.ffts = V;
     while (gen_col_ok<T>(p, 2 * P.ffts) && GenLaunch<T>::col_smem(p->ny, 2 * P.ffts) <= third &&
-           2 * P.ffts <= 16)
+           2 * P.ffts <= 16 && (long long)(p->nx / 2 + 1) * p->batch >= 2LL * P.ffts * ctas)
       P.ffts *= 2;
   }
   if (!gen_row_ok<T>(p, P.rows) || !gen_col_ok<T>(p, P.ffts)) return FILL_EINVAL;
