@@ -369,7 +369,7 @@ template <typename T, int OP>
 __device__ __forceinline__ void src_load(const InstDesc<T>& I, const Opnd& o, T (&x)[8]) {
   if constexpr (OP == OP_LOAD_W || OP == OP_LOAD_Y || OP == OP_LOAD_W_MASK) {
     ld_pair((OP == OP_LOAD_Y ? I.y : I.w) + o.pix, x[0], x[1]);
-  } else if constexpr (OP == OP_LOAD_D_U) {
+  } else if constexpr (OP == OP_LOAD_D_U || OP == OP_LOAD_D || OP == OP_LOAD_D_M) {
     ld_map_pair<T>(I.d + o.pix, x[0], x[1]);
   } else if constexpr (OP == OP_LOAD_R || OP == OP_LOAD_U) {
     ldc(OP == OP_LOAD_R ? I.r : I.u, o.q, x[0], x[1]);
@@ -392,7 +392,7 @@ __device__ __forceinline__ cx<T> src_op(const InstDesc<T>& I, const Opnd& o, con
                                         T alpha, T beta, Acc<T>& acc) {
   const PairIdx& q = o.q;
   T a0 = x[0], a1 = x[1];
-  if constexpr (OP == OP_LOAD_W_MASK) {
+  if constexpr (OP == OP_LOAD_W_MASK || OP == OP_LOAD_D_M) {
     a0 = q.m0 ? a0 : (T)0;
     a1 = q.m1 ? a1 : (T)0;
   } else if constexpr (OP == OP_LOAD_D_U) {
@@ -478,6 +478,10 @@ __device__ __forceinline__ void sink_op(const InstDesc<T>& I, const Opnd& o, con
     st_pair(I.y + pix, a0, a1);
   } else if constexpr (OP == OP_STORE_Y_MASK) {
     st_pair(I.y + pix, m0 ? a0 : (T)0, m1 ? a1 : (T)0);
+  } else if constexpr (OP == OP_STORE_OUT) {
+    st_map_pair<T>(I.out + pix, a0, a1);
+  } else if constexpr (OP == OP_STORE_OUT_MASK) {
+    st_map_pair<T>(I.out + pix, m0 ? a0 : (T)0, m1 ? a1 : (T)0);
   }
 }
 
@@ -498,7 +502,7 @@ template <int OP>
 struct CompactOnly {
   static constexpr bool value = OP == OP_R_UPD || OP == OP_P_UPD_Z || OP == OP_P_UPD_R ||
                                 OP == OP_LOAD_R || OP == OP_LOAD_U || OP == OP_U64_UPD ||
-                                OP == OP_LOAD_W_MASK || OP == OP_Q || OP == OP_Z ||
+                                OP == OP_LOAD_W_MASK || OP == OP_LOAD_D_M || OP == OP_Q || OP == OP_Z ||
                                 OP == OP_B || OP == OP_RES || OP == OP_KSEL;
 };
 
@@ -542,10 +546,28 @@ __device__ __forceinline__ void stage_words(const uint2* mw, uint2* mws, int pix
   }
 }
 
+// Whether this thread's pixel pairs hold a pixel of class `param` (Sect. 6.3).
+template <int V>
+__device__ __forceinline__ bool class_in_rows(const uint2* mws, const uint8_t* cls, int pix0, int nx,
+                                              int nv, int L, int t, int nt, int param) {
+  bool any = false;
+  for (int j = t; j < L; j += nt) {
+    Opnd o[1][V];
+    chunk_words<V, 1, true>(mws, pix0, nx, nv, j, nt, L, o);
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      if (!o[0][v].ok || !o[0][v].q.any()) continue;
+      const uchar2 c = *reinterpret_cast<const uchar2*>(cls + o[0][v].pix);
+      any = any || (o[0][v].q.m0 && c.x == param) || (o[0][v].q.m1 && c.y == param);
+    }
+  }
+  return any;
+}
+
 template <typename T, int OP, int V>
 __device__ __forceinline__ void src_rows(const InstDesc<T>& I, const uint2* mws, int pix0, int nx, int nv, cx<T>* z,
                                          int L, int t, int nt, T alpha, T beta, Acc<T>& acc) {
-  constexpr bool W = !(OP == OP_LOAD_W || OP == OP_LOAD_Y);
+  constexpr bool W = !(OP == OP_LOAD_W || OP == OP_LOAD_Y || OP == OP_LOAD_D);
   constexpr bool C = CompactOnly<OP>::value;
   constexpr int CH = kGenChunk / V;
   for (int j0 = t; j0 < L; j0 += CH * nt) {
@@ -652,7 +674,7 @@ __host__ __device__ __forceinline__ size_t gen_row_main(int L, int rows) {
 // threads; blockIdx.y is the instance), rows at or beyond ny (odd ny) idle.
 // Shared memory: L complex values per row, interleaved [position][V] within a
 // group, then the rows' mask words.
-template <typename T, int V, bool IN_SPEC, bool OUT_SPEC, bool XI = false>
+template <typename T, int V, bool IN_SPEC, bool OUT_SPEC, bool AUX = false>
 __global__ void __launch_bounds__(kGenThreads, gen_minb<T>())
 k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* __restrict__ wl,
           const T* __restrict__ wx) {
@@ -669,11 +691,20 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
   Acc<T> acc;
 
   const int pix0 = y0 * a.nx;
+  constexpr bool XI = AUX && !IN_SPEC, KS = AUX && IN_SPEC;   // (as in k_row)
   if constexpr (!XI) gen::stage_words<V>(I.mw, mws, pix0, a.nx, nv, t, nt);
+  T* const specp = KS ? I.speck + 2 * (size_t)blockIdx.z * (L + 1) * ny
+                   : a.spec_sel ? I.spec2 : I.spec;
   pdl_wait();
   if (skip_instance(a.check_done, I.st)) return;
+  if constexpr (KS) {
+    __syncthreads();   // mask words
+    if (!__syncthreads_or(gen::class_in_rows<V>(mws, I.cls, pix0, a.nx, nv, L, t, nt,
+                                                a.param + blockIdx.z)))
+      return;
+  }
   if constexpr (IN_SPEC) {
-    gen::c2r<T, V>(a.spec_sel ? I.spec2 : I.spec, ny, y0, g, wx, Z, t, nt);
+    gen::c2r<T, V>(specp, ny, y0, g, wx, Z, t, nt);
     __syncthreads();
     gen::dit<T, V>(Z, g, wl, t, g.nst);   // Z[j] = x[2j] + i x[2j+1] (scaled)
 #define CGF_SINK(OPC, PARAM) \
@@ -683,6 +714,8 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
         gen::mid_rows<T, OP_Y_W, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt);
       else
         gen::mid_rows<T, OP_MASK, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt);
+    } else if constexpr (KS) {
+      CGF_SINK(OP_KSEL, a.param + blockIdx.z);
     } else {
       switch (a.op) {
         case OP_Q: CGF_SINK(OP_Q, 0); break;
@@ -691,9 +724,10 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
         case OP_RES: CGF_SINK(OP_RES, 0); break;
         case OP_GRAD: CGF_SINK(OP_GRAD, 0); break;
         case OP_RELAX: CGF_SINK(OP_RELAX, 0); break;
-        case OP_KSEL: CGF_SINK(OP_KSEL, a.param); break;
         case OP_STORE_Y: CGF_SINK(OP_STORE_Y, 0); break;
         case OP_STORE_Y_MASK: CGF_SINK(OP_STORE_Y_MASK, 0); break;
+        case OP_STORE_OUT: CGF_SINK(OP_STORE_OUT, 0); break;
+        case OP_STORE_OUT_MASK: CGF_SINK(OP_STORE_OUT_MASK, 0); break;
         default: break;
       }
     }
@@ -723,6 +757,8 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
       case OP_LOAD_W: CGF_SRC(OP_LOAD_W); break;
       case OP_LOAD_W_MASK: CGF_SRC(OP_LOAD_W_MASK); break;
       case OP_LOAD_D_U: CGF_SRC(OP_LOAD_D_U); break;
+      case OP_LOAD_D: CGF_SRC(OP_LOAD_D); break;
+      case OP_LOAD_D_M: CGF_SRC(OP_LOAD_D_M); break;
       case OP_U64_UPD: CGF_SRC(OP_U64_UPD); break;
       default:
         for (int j = t; j < L * V; j += nt) Z[j] = cx<T>{(T)0, (T)0};
@@ -735,7 +771,7 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
     __syncthreads();
     gen::dif<T, V>(Z, g, wl, t, g.nst);
     pdl_trigger();
-    gen::r2c<T, V>(a.spec_sel ? I.spec2 : I.spec, ny, y0, g, wx, Z, t, nt);
+    gen::r2c<T, V>(specp, ny, y0, g, wx, Z, t, nt);
   }
 
   if constexpr (!OUT_SPEC) pdl_trigger();
@@ -750,7 +786,8 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
 // then the remaining inverse stages and the store, in natural order
 // (table < 0: forward only, the last stage's outputs stored at their
 // frequencies; PRE: the input is spec, already transformed, gathered at the
-// same frequencies, and the output goes to spec_sel's buffer).  Shared
+// same frequencies, the table is kernel table - 2 + grid z, and the output goes
+// to speck's z-th spectrum).  Shared
 // memory: ny complex values per column.
 namespace gen {
 
@@ -820,7 +857,8 @@ k_col_gen(const InstDesc<T>* __restrict__ insts, ColArgs a, GenLen g, const T* _
   const int kxa = nv > 0 ? kx0 : 0;
   cx<T>* Z = reinterpret_cast<cx<T>*>(smem_raw) + grp * N * V;
   const long long cstride = 2LL * N;   // T elements between consecutive columns
-  T* col = (a.spec_sel ? I.spec2 : I.spec) + cstride * kxa;
+  const int kz = PRE ? blockIdx.z : 0;
+  T* col = (PRE ? I.speck + cstride * kz * a.nkx : a.spec_sel ? I.spec2 : I.spec) + cstride * kxa;
   const T* srcp = PRE ? I.spec + cstride * kxa : col;
   const int S = g.nst, R = g.radix[S - 1];
 
@@ -844,7 +882,7 @@ k_col_gen(const InstDesc<T>* __restrict__ insts, ColArgs a, GenLen g, const T* _
   const T* tab0 = nullptr;
   long long tstride = N;
   if (a.table >= 0)
-    tab0 = (a.table >= 2 ? I.kt + (long long)(a.table - 2) * a.nkx * N
+    tab0 = (PRE ? I.kt + (long long)(a.table - 2 + kz) * a.nkx * N
             : a.table ? I.t_sqrt : I.t_inv) + (long long)kxa * N;
   switch (R) {
     case 2: gen::col_middle<T, V, 2, PRE>(Z, g, tab0, tstride, srcp, col, cstride, nv, a.table, t, nt); break;
@@ -894,10 +932,12 @@ cudaError_t GenLaunch<T>::row(bool in_spec, bool out_spec, const InstDesc<T>* d,
                               const RowArgs& a, const GenLen& g, const T* wl, const T* wx,
                               cudaStream_t s) {
   constexpr int V = gen_vrow<T>();
-  const dim3 grid((a.ny + a.rows - 1) / a.rows, ninst), block(a.rows / V * g.nt);
+  const dim3 grid((a.ny + a.rows - 1) / a.rows, ninst, a.nz > 0 ? a.nz : 1);
+  const dim3 block(a.rows / V * g.nt);
   const size_t sm = row_smem(g.n, a.rows);
   const Launcher l{grid, block, sm, s, a.pdl != 0};
   if (in_spec && out_spec) return l(k_row_gen<T, V, true, true>, d, a, g, wl, wx);
+  if (in_spec && a.op == OP_KSEL) return l(k_row_gen<T, V, true, false, true>, d, a, g, wl, wx);
   if (in_spec) return l(k_row_gen<T, V, true, false>, d, a, g, wl, wx);
   if (a.op == OP_XI) return l(k_row_gen<T, V, false, true, true>, d, a, g, wl, wx);
   return l(k_row_gen<T, V, false, true>, d, a, g, wl, wx);
@@ -907,7 +947,8 @@ template <typename T>
 cudaError_t GenLaunch<T>::col(const InstDesc<T>* d, int ninst, const ColArgs& a, const GenLen& g,
                               const T* wn, cudaStream_t s) {
   constexpr int V = gen_v<T>();
-  const dim3 grid(ninst, (a.nkx + a.ffts - 1) / a.ffts), block(a.ffts / V * g.nt);
+  const dim3 grid(ninst, (a.nkx + a.ffts - 1) / a.ffts, a.nz > 0 ? a.nz : 1);
+  const dim3 block(a.ffts / V * g.nt);
   const size_t sm = col_smem(g.n, a.ffts);
   const Launcher l{grid, block, sm, s, a.pdl != 0};
   if (a.pre) return l(k_col_gen<T, V, true>, d, a, g, wn);
@@ -919,6 +960,7 @@ cudaError_t GenLaunch<T>::prepare() {
   constexpr int V = gen_v<T>(), VR = gen_vrow<T>();
   cudaError_t e = detail::allow_smem(k_row_gen<T, VR, true, true>);
   if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, true, false>);
+  if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, true, false, true>);
   if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, false, true>);
   if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, false, true, true>);
   if (e == cudaSuccess) e = detail::allow_smem(k_col_gen<T, V>);

@@ -159,7 +159,8 @@ __device__ __forceinline__ void src_fill(const InstDesc<T>& I, const uint2* mwr,
         if constexpr (OP == OP_LOAD_W_MASK) q[e] = pair_at(mwr, j);
       } else {
         q[e] = pair_at(mwr, j);
-        if constexpr (OP == OP_LOAD_D_U) ld_map_pair<T>(I.d + rowpix + 2 * j, x0[e], x1[e]);
+        if constexpr (OP == OP_LOAD_D_U || OP == OP_LOAD_D || OP == OP_LOAD_D_M)
+          ld_map_pair<T>(I.d + rowpix + 2 * j, x0[e], x1[e]);
         if constexpr (SKIP) on[e] = __any_sync(warp, q[e].any());
         if (C && on[e]) {
           if constexpr (OP == OP_LOAD_R) ldc(I.r, q[e], x0[e], x1[e]);
@@ -184,7 +185,7 @@ __device__ __forceinline__ void src_fill(const InstDesc<T>& I, const uint2* mwr,
 #pragma unroll
     for (int e = 0; e < CK; ++e) {
       T a0 = (T)0, a1 = (T)0;
-      if constexpr (OP == OP_LOAD_W_MASK) {
+      if constexpr (OP == OP_LOAD_W_MASK || OP == OP_LOAD_D_M) {
         a0 = q[e].m0 ? x0[e] : (T)0;
         a1 = q[e].m1 ? x1[e] : (T)0;
       } else if constexpr (OP == OP_LOAD_D_U) {
@@ -296,6 +297,10 @@ __device__ __forceinline__ void sink_fill(const InstDesc<T>& I, const uint2* mwr
         st_pair(I.y + rowpix + 2 * j, a0, a1);
       } else if constexpr (OP == OP_STORE_Y_MASK) {
         st_pair(I.y + rowpix + 2 * j, m0 ? a0 : (T)0, m1 ? a1 : (T)0);
+      } else if constexpr (OP == OP_STORE_OUT) {
+        st_map_pair<T>(I.out + rowpix + 2 * j, a0, a1);
+      } else if constexpr (OP == OP_STORE_OUT_MASK) {
+        st_map_pair<T>(I.out + rowpix + 2 * j, m0 ? a0 : (T)0, m1 ? a1 : (T)0);
       }
     }
   }
@@ -347,8 +352,10 @@ __device__ __forceinline__ void mid_fill(const InstDesc<T>& I, const uint2* mwr,
 // and read twice with a CTA barrier on either side: FP32 passes at 8 x 4096^2
 // sink 377 -> 349, middle 511 -> 451, r update 454 -> 447 us; 1024^2 x 16 middle
 // 52 -> 47; 512^2 FP64 164 -> 152 us per iteration.
-// XI: the source is the seed's white noise (kept out of the other source
-// kernels, whose register allocation it would otherwise burden).
+// AUX: the source is the seed's white noise, or the sink selects the pixels of
+// one kernel's class (Sect. 6.3; grid z = kernel), skipping the rows without
+// one.  Both are kept out of the other kernels, whose registers and barriers
+// they would burden (the row check in every sink: 349 -> 384 us at 8 x 4096^2).
 
 // Exchange area of one row, in 8-byte words: XBuf's L + L/16 + 1 complex
 // elements, padded so that the areas of a CTA's rows start 16 / rows words
@@ -366,7 +373,7 @@ __host__ __device__ __forceinline__ size_t row_main_bytes(int log_l, int rows) {
   return (size_t(rows) * row_area_words<T>(log_l, rows) * 8 + 15) & ~size_t(15);
 }
 
-template <typename T, int LOG_L, bool IN_SPEC, bool OUT_SPEC, bool XI = false>
+template <typename T, int LOG_L, bool IN_SPEC, bool OUT_SPEC, bool AUX = false>
 __global__ void __launch_bounds__(KCfg<T>::kMaxThreads)
 k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw) {
   constexpr int LE = row_le<T>(LOG_L), E = 1 << LE;
@@ -395,15 +402,31 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
   cx<T> v[E];
   Acc<T> acc;
 
+  constexpr bool XI = AUX && !IN_SPEC, KS = AUX && IN_SPEC;
   if constexpr (!XI) {
     if (E == 16 || threadIdx.x < rows * NW)
       mws[threadIdx.x] = __ldg(I.mw + (size_t)y0 * NW + threadIdx.x);
   }
-  T* const specp = a.spec_sel ? I.spec2 : I.spec;
+  T* const specp = KS ? I.speck + 2 * (size_t)blockIdx.z * (L + 1) * ny
+                   : a.spec_sel ? I.spec2 : I.spec;
   cx<T> wk{};   // W_nx^kk
   if constexpr (IN_SPEC || OUT_SPEC) wk = twiddle<T>(tw, kk * TWS);
   pdl_wait();
   if (skip_instance(a.check_done, st)) return;
+
+  if constexpr (KS) {
+    const int param = a.param + blockIdx.z;
+    __syncthreads();   // mask words
+    bool any = false;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const PairIdx q = pair_at(mwr, tid + e * TT);
+      if (!q.any()) continue;
+      const uchar2 c = *reinterpret_cast<const uchar2*>(I.cls + rowpix + 2 * (tid + e * TT));
+      any = any || (q.m0 && c.x == param) || (q.m1 && c.y == param);
+    }
+    if (!__syncthreads_or(any)) return;
+  }
 
   if constexpr (IN_SPEC) {
     // rows kk and L - kk of the half spectrum, stepping up and down by TT rows
@@ -432,7 +455,7 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
     }
     if (kk == 0) xs.st(L / 2, cx<T>{xh.r + xh.r, -(xh.i + xh.i)});
     __syncthreads();
-    if (threadIdx.x == 0 && !OUT_SPEC) prefetch_compact(I, a.op, mws, rows * NW);
+    if (threadIdx.x == 0 && !OUT_SPEC && !AUX) prefetch_compact(I, a.op, mws, rows * NW);
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = xb.ld(tid + e * TT);
     fft_regs<T, LOG_L, LE, true>(v, xb, tid, tw, rbar, rbar);
@@ -442,6 +465,8 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
         mid_fill<T, TT, E, OP_Y_W>(I, mwr, rowpix, tid, v);
       else
         mid_fill<T, TT, E, OP_MASK>(I, mwr, rowpix, tid, v);
+    } else if constexpr (KS) {
+      sink_fill<T, TT, E, OP_KSEL>(I, mwr, rowpix, tid, v, acc, a.param + blockIdx.z);
     } else {
       switch (a.op) {
         case OP_Q: sink_fill<T, TT, E, OP_Q>(I, mwr, rowpix, tid, v, acc); break;
@@ -450,10 +475,13 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
         case OP_RES: sink_fill<T, TT, E, OP_RES>(I, mwr, rowpix, tid, v, acc); break;
         case OP_GRAD: sink_fill<T, TT, E, OP_GRAD>(I, mwr, rowpix, tid, v, acc); break;
         case OP_RELAX: sink_fill<T, TT, E, OP_RELAX>(I, mwr, rowpix, tid, v, acc); break;
-        case OP_KSEL: sink_fill<T, TT, E, OP_KSEL>(I, mwr, rowpix, tid, v, acc, a.param); break;
         case OP_STORE_Y: sink_fill<T, TT, E, OP_STORE_Y>(I, mwr, rowpix, tid, v, acc); break;
         case OP_STORE_Y_MASK:
           sink_fill<T, TT, E, OP_STORE_Y_MASK>(I, mwr, rowpix, tid, v, acc);
+          break;
+        case OP_STORE_OUT: sink_fill<T, TT, E, OP_STORE_OUT>(I, mwr, rowpix, tid, v, acc); break;
+        case OP_STORE_OUT_MASK:
+          sink_fill<T, TT, E, OP_STORE_OUT_MASK>(I, mwr, rowpix, tid, v, acc);
           break;
         default: break;
       }
@@ -487,6 +515,10 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
         break;
       case OP_LOAD_D_U:
         src_fill<T, TT, E, OP_LOAD_D_U>(I, mwr, rowpix, tid, alpha, beta, v, acc);
+        break;
+      case OP_LOAD_D: src_fill<T, TT, E, OP_LOAD_D>(I, mwr, rowpix, tid, alpha, beta, v, acc); break;
+      case OP_LOAD_D_M:
+        src_fill<T, TT, E, OP_LOAD_D_M>(I, mwr, rowpix, tid, alpha, beta, v, acc);
         break;
       case OP_U64_UPD:
         src_fill<T, TT, E, OP_U64_UPD>(I, mwr, rowpix, tid, alpha, beta, v, acc);
@@ -542,8 +574,9 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
 // ----------------------------------------------------------------- column pass
 // CTA = `ffts` spectrum rows (one kx each), N/E threads per row; forward
 // column FFT, multiply by the real table, inverse column FFT, in place
-// (table < 0: forward transform only; PRE: start from the forward transform
-// held in spec and write to the buffer spec_sel names).  blockIdx.x is the instance, so the
+// (table < 0: forward transform only; PRE, Sect. 6.3: start from the forward
+// transform held in spec, times kernel table (table - 2 + grid z), into speck's
+// z-th spectrum).  blockIdx.x is the instance, so the
 // CTAs of all instances for the same kx run together and share the table
 // row through L2.
 template <typename T, int LOG_N, bool PRE = false>
@@ -561,12 +594,14 @@ k_col(const InstDesc<T>* __restrict__ insts, ColArgs a, const T* __restrict__ tw
   const bool act = kx < a.nkx;
   const XBuf<T> xb(sm + f * 2 * PADN, PADN);
   const XBar bar = XBar::make(TT, a.ffts, f);
-  T* col = (a.spec_sel ? I.spec2 : I.spec) + 2 * (long long)(act ? kx : 0) * N;
+  const int kz = PRE ? blockIdx.z : 0;
+  T* col = (PRE ? I.speck + 2 * (long long)kz * a.nkx * N : a.spec_sel ? I.spec2 : I.spec) +
+           2 * (long long)(act ? kx : 0) * N;
   const T* src = PRE ? I.spec + 2 * (long long)(act ? kx : 0) * N : col;
   const T* tab = nullptr;
   if (a.table >= 0)
-    tab = (a.table >= 2 ? I.kt + (long long)(a.table - 2) * a.nkx * N
-           : a.table ? I.t_sqrt : I.t_inv) + (long long)(act ? kx : 0) * N;
+    tab = (PRE ? I.kt + (long long)(a.table - 2 + kz) * a.nkx * N : a.table ? I.t_sqrt : I.t_inv) +
+          (long long)(act ? kx : 0) * N;
   // fewer elements per thread: the table's values are fetched before the wait
   constexpr bool PT = E < 16;
   T tv[PT ? E : 1];
@@ -793,18 +828,6 @@ k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
           ld_pair(I.y + pix, y0, y1);
           ldc(I.u, q, u0, u1);
           st_pair(I.w + pix, q.m0 ? u0 : d0 - y0, q.m1 ? u1 : d1 - y1);
-          break;
-        }
-        case VOP_MAP_IN: {
-          T a0, a1;
-          ld_map_pair<T>(I.d + pix, a0, a1);
-          st_pair(I.w + pix, a0, a1);
-          break;
-        }
-        case VOP_MAP_OUT: {
-          T a0, a1;
-          ld_pair(I.y + pix, a0, a1);
-          st_map_pair<T>(I.out + pix, a0, a1);
           break;
         }
         case VOP_ANNULUS: {   // offsets by minimum image from pixel 0

@@ -66,10 +66,11 @@ template <typename T, int LL>
 cudaError_t row_ll(bool in_spec, bool out_spec, const InstDesc<T>* d, int ninst, const RowArgs& a,
                    const T* tw, cudaStream_t s) {
   constexpr int TT = (1 << LL) >> row_le<T>(LL);
-  dim3 grid(a.ny / a.rows, ninst), block(a.rows * TT);
+  dim3 grid(a.ny / a.rows, ninst, a.nz > 0 ? a.nz : 1), block(a.rows * TT);
   const size_t sm = Launch<T>::row_smem(LL, a.rows);
   const Launcher l{grid, block, sm, s, a.pdl != 0};
   if (in_spec && out_spec) return l(k_row<T, LL, true, true>, d, a, tw);
+  if (in_spec && a.op == OP_KSEL) return l(k_row<T, LL, true, false, true>, d, a, tw);
   if (in_spec) return l(k_row<T, LL, true, false>, d, a, tw);
   if (a.op == OP_XI) return l(k_row<T, LL, false, true, true>, d, a, tw);
   return l(k_row<T, LL, false, true>, d, a, tw);
@@ -110,7 +111,7 @@ cudaError_t col_ln(const InstDesc<T>* d, int ninst, const ColArgs& a, const T* t
           k_col_tma<LN>, d, b, tw, ninst);
     }
   }
-  dim3 grid(ninst, (a.nkx + a.ffts - 1) / a.ffts), block(a.ffts * TT);
+  dim3 grid(ninst, (a.nkx + a.ffts - 1) / a.ffts, a.nz > 0 ? a.nz : 1), block(a.ffts * TT);
   const size_t sm = Launch<T>::col_smem(LN, a.ffts);
   const Launcher l{grid, block, sm, s, a.pdl != 0};
   if (a.pre) return l(k_col<T, LN, true>, d, a, tw);
@@ -121,6 +122,7 @@ template <typename T, int LL>
 cudaError_t prep_row() {
   cudaError_t e = allow_smem(k_row<T, LL, true, true>);
   if (e == cudaSuccess) e = allow_smem(k_row<T, LL, true, false>);
+  if (e == cudaSuccess) e = allow_smem(k_row<T, LL, true, false, true>);
   if (e == cudaSuccess) e = allow_smem(k_row<T, LL, false, true>);
   if (e == cudaSuccess) e = allow_smem(k_row<T, LL, false, true, true>);
   return e;

@@ -107,6 +107,7 @@ struct InstDesc {
   double* hist;            // residual history (hist_cap entries), or null
   double* coef;            // CG coefficients (2 hist_cap entries), or null
   const T* kt;             // kernel tables [j][kx][ky] of the Sect. 6.3 solver, or null
+  T* speck;                // spectra of that solver's kernels that run together, or null
   const uint8_t* cls;      // kernel class of every pixel (Sect. 6.3 solver), or null
   long long nvec;          // CG-vector length: 32 per word with a masked pixel
   unsigned long long seed;
@@ -125,6 +126,8 @@ enum RowOp : int {
   OP_LOAD_U = 8,    // v = u
   OP_LOAD_Y = 9,    // v = y
   OP_LOAD_D_U = 28, // v = d on U, 0 on M (maximum-likelihood right-hand side)
+  OP_LOAD_D = 31,   // v = d (operator applications on the caller's map)
+  OP_LOAD_D_M = 32, // v = P_x d
   // middles (input spectrum -> output spectrum)
   OP_MASK = 10,     // v = P_x v
   OP_Y_W = 11,      // store y = v; v = (d - y) on U, 0 on M
@@ -140,6 +143,8 @@ enum RowOp : int {
                     // acc ||v_M||^2
   OP_KSEL = 30,     // v = kernel j * w: y = v on the masked pixels of class j (Sect. 6.3)
   OP_LOAD_W = 26,   // (source) v = w
+  OP_STORE_OUT = 33,       // out = v (the caller's map)
+  OP_STORE_OUT_MASK = 34,  // out = P_x v
 };
 
 // Scalar updates run by the last CTA of a reducing pass.
@@ -170,8 +175,6 @@ enum VecOp : int {
   VOP_MAKE_W = 5,     // w = d - y on U, u on M
   VOP_LOAD_G = 6,     // r = b = P_x g (r32 = (float) r if set); acc ||r||^2
   VOP_ZERO_UP = 7,    // u = 0, p = 0
-  VOP_MAP_IN = 8,     // w = d (caller's map -> pass element type)
-  VOP_MAP_OUT = 9,    // out = y (pass element type -> caller's map)
   VOP_W_FROM_D = 10,  // w = d on U, 0 on M
   VOP_W_TO_OUT = 11,  // out = w (pass element type -> caller's map)
   VOP_ANNULUS = 12,   // w = 1 where r_in^2 < |offset|^2 <= r_out^2 (offset from pixel 0), else 0
@@ -187,9 +190,10 @@ struct RowArgs {
   int op;           // RowOp
   int sop;          // ScalarOp (SC_NONE: no reduction)
   int check_done;   // skip instances whose CG state is done
-  int spec_sel;     // 0: spec, 1: spec2
-  int param;        // op parameter (OP_KSEL: the kernel class)
+  int spec_sel;     // 0: spec, 1: spec2, 2: speck (grid z: one kernel's spectrum each)
+  int param;        // op parameter (OP_KSEL: the kernel class, plus grid z)
   int pdl;          // launch as a programmatic dependent of the previous kernel
+  int nz;           // grid z (spec_sel = 2), else 0
 };
 
 struct ColArgs {
@@ -199,12 +203,13 @@ struct ColArgs {
   int table;        // 0: 1/(nP), 1: sqrt(P)/n; j + 2: kernel table j; -1: forward only
   int check_done;
   int spec_sel;     // 0: spec, 1: spec2
-  int pre;          // 1: the input is spec, already column-transformed (table >= 0; the
-                    // forward FFT is skipped and the result goes to spec_sel's buffer)
+  int pre;          // 1: the input is spec, already column-transformed (table >= 2; the
+                    // forward FFT is skipped; grid z takes table + z into speck's z-th spectrum)
   int* err;         // device error flag (set to 1 when a bounded wait gave up), or null
   int variant;      // FP32 table passes: 0 register-fed kernel, 1 persistent bulk-copy-fed
                     // kernel (chosen per grid by the autotuner)
   int pdl;          // as RowArgs::pdl
+  int nz;           // grid z (pre), else 0
 };
 
 // Band-binned spectral products for the band-power gradient.

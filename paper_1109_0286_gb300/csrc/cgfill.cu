@@ -133,7 +133,8 @@ struct Precision {
   double* hist = nullptr;
   double* coef = nullptr;       // CG coefficients, 2 history_cap per instance
   T* kt = nullptr;              // kernel tables of the Sect. 6.3 solver
-  int nk = 0, nk_cap = 0;
+  T* speck = nullptr;           // its spectra: kz per instance
+  int nk = 0, nk_cap = 0, kz = 0;
   T* gwl = nullptr; T* gwx = nullptr; T* gwn = nullptr;   // mixed-radix twiddles
   InstDesc<T>* desc = nullptr;  // device, batch
   InstDesc<T>* hdesc = nullptr; // pinned
@@ -381,9 +382,9 @@ Ctx<T> ctx(fill_plan* p, int ninst = -1) {
 
 template <typename T>
 cudaError_t row(const Ctx<T>& c, cudaStream_t s, int op, int sop, bool in_spec, bool out_spec,
-                int skip, int spec_sel = 0, int param = 0) {
+                int skip, int spec_sel = 0, int param = 0, int nz = 0) {
   ++*c.launches;
-  RowArgs a{c.ny, c.nx, c.rows, ilog2(c.rows), op, sop, skip, spec_sel, param, c.pdl};
+  RowArgs a{c.ny, c.nx, c.rows, ilog2(c.rows), op, sop, skip, spec_sel, param, c.pdl, nz};
   if (c.grow)
     return GenLaunch<T>::row(in_spec, out_spec, c.desc, c.ninst, a, *c.grow, c.gwl, c.gwx, s);
   return Launch<T>::row(c.log_l, in_spec, out_spec, c.desc, c.ninst, a, c.tw, s);
@@ -391,9 +392,9 @@ cudaError_t row(const Ctx<T>& c, cudaStream_t s, int op, int sop, bool in_spec, 
 
 template <typename T>
 cudaError_t col(const Ctx<T>& c, cudaStream_t s, int table, int skip, int spec_sel = 0,
-                int pre = 0) {
+                int pre = 0, int nz = 0) {
   ++*c.launches;
-  ColArgs a{c.ny, c.nx / 2 + 1, c.ffts, table, skip, spec_sel, pre, c.err, c.col_variant, c.pdl};
+  ColArgs a{c.ny, c.nx / 2 + 1, c.ffts, table, skip, spec_sel, pre, c.err, c.col_variant, c.pdl, nz};
   if (c.gcol) return GenLaunch<T>::col(c.desc, c.ninst, a, *c.gcol, c.gwn, s);
   return Launch<T>::col(c.log_n, c.desc, c.ninst, a, c.tw, s);
 }
@@ -1760,12 +1761,22 @@ fill_status set_annuli_t(fill_plan* p, int nk, const double* r_in, const double*
     P.nk_cap = nk;
   }
   const size_t nspec = 2 * ntab;
-  if (!P.spec2 && p->dalloc(&P.spec2, size_t(p->batch) * nspec) != cudaSuccess)
-    return FILL_ENOMEM;
+  // spectra for all kernels at once (within 4 GB, or as many as there is room
+  // for: the solver then takes the kernels in turns of kz)
+  if (P.kz < nk) {
+    const size_t one = size_t(p->batch) * nspec * sizeof(T);
+    int kz = (int)std::max<size_t>(1, std::min<size_t>(nk, (size_t(4) << 30) / one));
+    while (kz > P.kz && p->dalloc(&P.speck, size_t(kz) * p->batch * nspec) != cudaSuccess) {
+      cudaGetLastError();
+      if (kz == 1) return FILL_ENOMEM;
+      kz /= 2;
+    }
+    P.kz = std::max(P.kz, kz);
+  }
   P.nk = nk;
   for (int i = 0; i < p->batch; ++i) {
     P.hdesc[i].kt = P.kt;
-    P.hdesc[i].spec2 = P.spec2 + size_t(i) * nspec;
+    P.hdesc[i].speck = P.speck + size_t(i) * P.kz * nspec;
   }
   fill_desc<T>(p, nullptr, 0, nullptr, nullptr, nullptr);
   CK(upload_desc<T>(p));
@@ -1788,9 +1799,11 @@ fill_status set_annuli_t(fill_plan* p, int nk, const double* r_in, const double*
 // Multi-scale kernel Laplace solver (Sect. 6.3): every sweep averages the map
 // over each masked pixel's annulus (class map `cls`), all from the same map.
 // One forward transform per sweep (row pass, then the column pass in forward
-// mode, into spec); per annulus the column pass multiplies by its table and
-// inverts into spec2, from which the inverse row pass writes the pixels of
-// that class.
+// mode, into spec); then one column pass multiplies by every annulus's table
+// and inverts (grid z = annulus, into its own spectrum), and one inverse row
+// pass writes the pixels of every class, skipping the rows without one.
+// (A launch per annulus and pass made a sweep 20 launches of 6 us each at
+// 1024^2 with 9 annuli.)
 template <typename T>
 fill_status laplace_ms_t(fill_plan* p, const void* d, long long d_stride, int iters,
                          const uint8_t* cls, void* out, fill_stats* stats) {
@@ -1811,9 +1824,10 @@ fill_status laplace_ms_t(fill_plan* p, const void* d, long long d_stride, int it
   for (int k = 0; k < iters; ++k) {
     CK(row<T>(c, p->s, OP_LOAD_W, SC_NONE, false, true, SKIP_NEVER));
     CK(col<T>(c, p->s, -1, SKIP_NEVER));
-    for (int j = 0; j < P.nk; ++j) {
-      CK(col<T>(c, p->s, 2 + j, SKIP_NEVER, 1, 1));
-      CK(row<T>(c, p->s, OP_KSEL, SC_NONE, true, false, SKIP_NEVER, 1, j));
+    for (int j = 0; j < P.nk; j += P.kz) {
+      const int n = std::min(P.kz, P.nk - j);
+      CK(col<T>(c, p->s, 2 + j, SKIP_NEVER, 0, 1, n));
+      CK(row<T>(c, p->s, OP_KSEL, SC_NONE, true, false, SKIP_NEVER, 2, j, n));
     }
     CK(vec<T>(c, p->s, VOP_Y_TO_W_M, k == 0 ? SC_BB : SC_RES, SKIP_NEVER));
   }
@@ -1860,68 +1874,69 @@ fill_status fill_laplace_ms(fill_plan* p, const void* d, long long d_stride, int
                                        : laplace_ms_t<df>(p, d, d_stride, iters, cls, out, stats);
 }
 
-fill_status fill_draw(fill_plan* p, const uint64_t* seeds, void* out) {
-  if (!p || !seeds || !out) return FILL_EINVAL;
-  const size_t n = p->npix;
-  if (p->o.mode == FILL_MODE_FP32) {
-    fill_desc<float>(p, nullptr, 0, seeds, nullptr, nullptr);
-    CK(upload_desc<float>(p));
-    CK(init_states<float>(p, 0.0));
-    CK(row<float>(p, p->s, OP_XI, SC_NONE, false, true, false));
-    CK(col<float>(p, p->s, 1, false));
-    CK(row<float>(p, p->s, OP_STORE_Y, SC_NONE, true, false, false));
-    CK(cudaMemcpyAsync(out, p->f.y, p->batch * n * sizeof(float), cudaMemcpyDeviceToDevice, p->s));
-  } else if (p->o.mode == FILL_MODE_FP64) {
-    fill_desc<double>(p, nullptr, 0, seeds, nullptr, nullptr);
-    CK(upload_desc<double>(p));
-    CK(init_states<double>(p, 0.0));
-    CK(row<double>(p, p->s, OP_XI, SC_NONE, false, true, false));
-    CK(col<double>(p, p->s, 1, false));
-    CK(row<double>(p, p->s, OP_STORE_Y, SC_NONE, true, false, false));
-    CK(cudaMemcpyAsync(out, p->g.y, p->batch * n * sizeof(double), cudaMemcpyDeviceToDevice, p->s));
-  } else {
-    fill_desc<df>(p, nullptr, 0, seeds, out, nullptr);
-    CK(upload_desc<df>(p));
-    CK(init_states<df>(p, 0.0));
-    CK(row<df>(p, p->s, OP_XI, SC_NONE, false, true, false));
-    CK(col<df>(p, p->s, 1, false));
-    CK(row<df>(p, p->s, OP_STORE_Y, SC_NONE, true, false, false));
-    CK(vec<df>(p, p->s, VOP_MAP_OUT, SC_NONE, false));
-  }
+}  // extern "C"
+
+namespace {
+// Whether a caller's map can be read and written in pixel pairs in place.
+template <typename T>
+bool pair_aligned(const void* map) {
+  return reinterpret_cast<uintptr_t>(map) % (2 * sizeof(typename MapOf<T>::type)) == 0;
+}
+
+// y = F^-1[sqrt(P) F xi] straight into the caller's maps (through y and a copy
+// if they are not aligned to pixel pairs; every pass reads descriptors only,
+// so the CG states are left as they are).
+template <typename T>
+fill_status draw_t(fill_plan* p, const uint64_t* seeds, void* out) {
+  constexpr bool same = std::is_same<T, typename MapOf<T>::type>::value;
+  const bool direct = !same || pair_aligned<T>(out);
+  fill_desc<T>(p, nullptr, 0, seeds, out, nullptr);
+  CK(upload_desc<T>(p));
+  CK(row<T>(p, p->s, OP_XI, SC_NONE, false, true, SKIP_NEVER));
+  CK(col<T>(p, p->s, 1, SKIP_NEVER));
+  CK(row<T>(p, p->s, direct ? OP_STORE_OUT : OP_STORE_Y, SC_NONE, true, false, SKIP_NEVER));
+  if (!direct)
+    CK(cudaMemcpyAsync(out, prec<T>(p).y, p->batch * size_t(p->npix) * sizeof(T),
+                       cudaMemcpyDeviceToDevice, p->s));
   CK(cudaStreamSynchronize(p->s));
   return FILL_OK;
 }
 
-}  // extern "C"
-
-namespace {
+// One operator application, from and to the caller's maps (through w and y if
+// they are not aligned to pixel pairs).
 template <typename T>
 fill_status apply_t(fill_plan* p, int which, const void* in, void* out) {
   Precision<T>& P = prec<T>(p);
   const size_t n = p->npix;
   constexpr bool same = std::is_same<T, typename MapOf<T>::type>::value;
-  fill_desc<T>(p, in, 0, nullptr, out, nullptr);
-  CK(upload_desc<T>(p));
-  CK(init_states<T>(p, 0.0));
-  if (same)
-    CK(cudaMemcpyAsync(P.w, in, n * sizeof(T), cudaMemcpyDeviceToDevice, p->s));
-  else
-    CK(vec<T>(ctx<T>(p, 1), p->s, VOP_MAP_IN, SC_NONE, false));
+  const bool direct = !same || (pair_aligned<T>(in) && pair_aligned<T>(out));
   const bool masked = which >= 2;
   const int table = (which == 0 || which == 2) ? 0 : 1;
-  CK(row<T>(p, p->s, masked ? OP_LOAD_W_MASK : OP_LOAD_W, SC_NONE, false, true, false, 1));
-  CK(col<T>(p, p->s, table, false, 1));
-  CK(row<T>(p, p->s, masked ? OP_STORE_Y_MASK : OP_STORE_Y, SC_NONE, true, false, false, 1));
-  if (same)
+  fill_desc<T>(p, in, 0, nullptr, out, nullptr);
+  CK(upload_desc<T>(p));
+  if (!direct)
+    CK(cudaMemcpyAsync(P.w, in, n * sizeof(T), cudaMemcpyDeviceToDevice, p->s));
+  const int src = direct ? (masked ? OP_LOAD_D_M : OP_LOAD_D) : masked ? OP_LOAD_W_MASK : OP_LOAD_W;
+  const int dst = direct ? (masked ? OP_STORE_OUT_MASK : OP_STORE_OUT)
+                         : masked ? OP_STORE_Y_MASK : OP_STORE_Y;
+  CK(row<T>(p, p->s, src, SC_NONE, false, true, SKIP_NEVER, 1));
+  CK(col<T>(p, p->s, table, SKIP_NEVER, 1));
+  CK(row<T>(p, p->s, dst, SC_NONE, true, false, SKIP_NEVER, 1));
+  if (!direct)
     CK(cudaMemcpyAsync(out, P.y, n * sizeof(T), cudaMemcpyDeviceToDevice, p->s));
-  else
-    CK(vec<T>(ctx<T>(p, 1), p->s, VOP_MAP_OUT, SC_NONE, false));
   CK(cudaStreamSynchronize(p->s));
   return FILL_OK;
 }
 }  // namespace
 
 extern "C" {
+
+fill_status fill_draw(fill_plan* p, const uint64_t* seeds, void* out) {
+  if (!p || !seeds || !out) return FILL_EINVAL;
+  return p->o.mode == FILL_MODE_FP32   ? draw_t<float>(p, seeds, out)
+         : p->o.mode == FILL_MODE_FP64 ? draw_t<double>(p, seeds, out)
+                                       : draw_t<df>(p, seeds, out);
+}
 
 fill_status fill_apply(fill_plan* p, int which, const void* in, void* out) {
   if (!p || !in || !out || which < 0 || which > 3 || in == out) return FILL_EINVAL;
