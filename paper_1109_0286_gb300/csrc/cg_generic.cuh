@@ -738,7 +738,7 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
       const int rowpix = (y0 + (v < nv ? v : 0)) * a.nx;
       for (int j = t; j < L; j += nt) {
         double x0 = 0.0, x1 = 0.0;
-        if (v < nv) normal_pair(I.seed, (uint32_t)((rowpix >> 1) + j), x0, x1);
+        if (v < nv) normal_pair(I.noise, I.seed, (uint32_t)((rowpix >> 1) + j), x0, x1);
         Z[j * V + v] = cx<T>{(T)x0, (T)x1};
       }
     }

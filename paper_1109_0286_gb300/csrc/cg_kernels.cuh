@@ -490,7 +490,7 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       double x0, x1;
-      normal_pair(I.seed, (uint32_t)((rowpix >> 1) + tid + e * TT), x0, x1);
+      normal_pair(I.noise, I.seed, (uint32_t)((rowpix >> 1) + tid + e * TT), x0, x1);
       v[e] = cx<T>{(T)x0, (T)x1};
     }
   } else {

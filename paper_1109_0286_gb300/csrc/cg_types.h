@@ -109,6 +109,7 @@ struct InstDesc {
   const T* kt;             // kernel tables [j][kx][ky] of the Sect. 6.3 solver, or null
   T* speck;                // spectra of that solver's kernels that run together, or null
   const uint8_t* cls;      // kernel class of every pixel (Sect. 6.3 solver), or null
+  const double* noise;     // tables of the white-noise source
   long long nvec;          // CG-vector length: 32 per word with a masked pixel
   unsigned long long seed;
 };
@@ -291,6 +292,12 @@ CGF_HD constexpr int stw_base(int le, int log) {
 }
 constexpr int kStwEntries = stw_base(4, 14);   // all lengths 2^4 .. 2^13, le = 2, 3, 4
 constexpr int kTwEntries = kLmax + kStwEntries;   // complex entries of a twiddle buffer
+
+// Tables of the white-noise source (normal_pair in cg_common.cuh), doubles:
+// 256 pairs (-2/c, 2 log(1/c)), c the centre of [1 + i/256, 1 + (i+1)/256), halved
+// from 3/2 on, 1 for the intervals next to 1; 256 times cos, sin of 2 pi i/256 and
+// their low parts; 2 k log 2, k < 54.
+constexpr int kNoiseLog = 0, kNoiseArc = 512, kNoiseExp = 1536, kNoiseEntries = 1536 + 54;
 constexpr int kMaxPartials = 4096; // CTAs per instance per reducing pass
 constexpr int kMaxBands = 64;      // band-power gradient bins
 constexpr int kDotCtas = 256;      // CTAs per instance of the band-binned product

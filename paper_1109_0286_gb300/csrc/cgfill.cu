@@ -117,6 +117,37 @@ const std::vector<double>& twiddles_host() {
   return tw;
 }
 
+// The white-noise source's tables (kNoise*), each entry rounded once from
+// extended precision.
+std::vector<double> noise_build() {
+  std::vector<double> t(kNoiseEntries);
+  for (int i = 0; i < 256; ++i) {
+    long double c = 1.0L + (i + 0.5L) / 256.0L;
+    if (i >= 128) c /= 2.0L;
+    const double inv = i == 0 || i == 255 ? 1.0 : (double)(1.0L / c);
+    t[kNoiseLog + 2 * i] = -2.0 * inv;
+    t[kNoiseLog + 2 * i + 1] = (double)(2.0L * std::log((long double)inv));
+    // cos, sin by octants (exact 0, 1 and equal magnitudes on the symmetries)
+    const int o = i / 32, f = i % 32;
+    const long double th = 3.14159265358979323846264338327950288L / 128.0L * (o & 1 ? 32 - f : f);
+    const long double u = std::cos(th), v = std::sin(th);
+    const bool swap = ((o + 1) / 2) % 2;   // octants 1, 2, 5, 6
+    const long double c8 = (o >= 2 && o < 6 ? -1.0L : 1.0L) * (swap ? v : u);
+    const long double s8 = (o >= 4 ? -1.0L : 1.0L) * (swap ? u : v);
+    double* arc = &t[kNoiseArc + 4 * i];
+    arc[0] = (double)c8;
+    arc[1] = (double)s8;
+    arc[2] = (double)(c8 - (long double)arc[0]);
+    arc[3] = (double)(s8 - (long double)arc[1]);
+  }
+  for (int k = 0; k < 54; ++k) t[kNoiseExp + k] = (double)(2.0L * k * std::log(2.0L));
+  return t;
+}
+const std::vector<double>& noise_host() {
+  static const std::vector<double> t = noise_build();
+  return t;
+}
+
 template <typename T>
 struct Precision {
   // device buffers (instance-major slabs of batch * npix)
@@ -166,6 +197,7 @@ struct fill_plan {
   uint2* mw = nullptr;           // mask words: observed bits, CG-vector offset
   long long nvec = 0;            // CG-vector length: 32 per mask word with a masked pixel
   long long nv = 0;              // CG-vector stride per instance (>= nvec)
+  double* noise = nullptr;       // device: tables of the white-noise source
   std::vector<double> P_half;    // host copy of the spectrum
   double* P_dev = nullptr;       // device copy (fill_set_spectrum builds the tables from it)
   double* sig_dev = nullptr;     // device copy of the band templates' S(k) (fill_set_bands)
@@ -1350,6 +1382,7 @@ fill_status setup_precision(fill_plan* p, const std::vector<double>& tinv,
   for (size_t i = 0; i < B; ++i) {
     InstDesc<T> D{};
     D.mw = p->mw;
+    D.noise = p->noise;
     D.nvec = p->nvec;
     D.t_inv = P.t_inv;
     D.t_sqrt = P.t_sqrt;
@@ -1541,6 +1574,9 @@ fill_status fill_init(fill_plan** out, int ny, int nx, const double* P_half,
   }
   if (e != cudaSuccess) return fail(cuda_fail(e, "cudaStreamCreate"));
   if (p->dalloc(&p->mw, words.size()) != cudaSuccess) return fail(FILL_ENOMEM);
+  if (p->dalloc(&p->noise, kNoiseEntries) != cudaSuccess) return fail(FILL_ENOMEM);
+  e = cudaMemcpy(p->noise, noise_host().data(), kNoiseEntries * sizeof(double), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return fail(cuda_fail(e, "upload tables"));
   if (p->dalloc(&p->P_dev, (size_t)ny * nkx) != cudaSuccess) return fail(FILL_ENOMEM);
   e = cudaMemcpy(p->P_dev, P_half, (size_t)ny * nkx * sizeof(double), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return fail(cuda_fail(e, "upload spectrum"));
