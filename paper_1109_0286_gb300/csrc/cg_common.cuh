@@ -73,6 +73,28 @@ __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// a b + c d with one renormalisation: both high products exact (FMA), their
+// TwoSum, and all low-order terms in one FP32 sum (20 FP32 instructions against
+// 25 for two products and an addition, and one rounding to a pair instead of
+// three).
+__device__ __forceinline__ df dot2(df a, df b, df c, df d) {
+  const float p = a.hi * b.hi, q = c.hi * d.hi;
+  const float ep = fmaf(a.hi, b.hi, -p), eq = fmaf(c.hi, d.hi, -q);
+  const float s = p + q, v = s - p;
+  const float e = ((p - (s - v)) + (q - v)) + (ep + eq);
+  const float l = e + fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(c.hi, d.lo, c.lo * d.hi)));
+  const float h = s + l;
+  return df(h, l - (h - s));
+}
+template <>
+__device__ __forceinline__ cx<df> cmul(cx<df> a, cx<df> b) {
+  return {dot2(a.r, b.r, -a.i, b.i), dot2(a.r, b.i, a.i, b.r)};
+}
+template <>
+__device__ __forceinline__ cx<df> cmulc(cx<df> a, cx<df> b) {
+  return {dot2(a.r, b.r, a.i, b.i), dot2(a.i, b.r, -a.r, b.i)};
+}
+
 // Vector types for 8- / 16-byte global accesses.
 template <typename T> struct V2;
 template <> struct V2<float> { using t = float2; };
