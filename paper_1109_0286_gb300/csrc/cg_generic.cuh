@@ -775,8 +775,10 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
   }
 
   if constexpr (!OUT_SPEC) pdl_trigger();
-  if (a.sop != SC_NONE)
-    grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, nt);
+  if constexpr (!AUX) {
+    if (a.sop != SC_NONE)
+      grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, nt);
+  }
 }
 
 // ----------------------------------------------------------------- column pass

@@ -566,9 +566,11 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
   }
 
   if constexpr (!OUT_SPEC) pdl_trigger();
-  if (a.sop != SC_NONE)
-    grid_reduce(acc.total(), red, I.partial, st, a.sop, gridDim.x, blockIdx.x,
-                min(rows, kRedRows) * TT);
+  if constexpr (!AUX) {
+    if (a.sop != SC_NONE)
+      grid_reduce(acc.total(), red, I.partial, st, a.sop, gridDim.x, blockIdx.x,
+                  min(rows, kRedRows) * TT);
+  }
 }
 
 // ----------------------------------------------------------------- column pass

@@ -31,13 +31,18 @@ inline int default_rows(int log_l, int ny) {
 
 // Column FFTs per CTA: about 256 threads (FP64: 64, as above; 256^2, one
 // map, 8 columns 269, 2 columns 203 us per iteration), within the thread and
-// shared-memory limits.
+// shared-memory limits, and in FP32 no more than leaves two CTAs per SM (1024^2,
+// one map, 4 columns 70.5, 1 column 66.0 us per iteration; 16 maps 300 and 348;
+// double-float relaxation of 1024^2 1174 and 1257 us, so not there).  ninst
+// maps share a launch; the results do not depend on the choice.
 template <typename T>
-inline int default_ffts(int log_n, int nkx) {
+inline int default_ffts(int log_n, int nkx, int ninst) {
   const int TT = (1 << log_n) >> col_le<T>(log_n);
   int f = std::max(1, (std::is_same<T, double>::value ? 64 : 256) / TT);
   f = std::min(f, std::max(1, Launch<T>::max_threads() / TT));
-  while (f > 1 && Launch<T>::col_smem(log_n, f) > 100 * 1024) f /= 2;
+  while (f > 1 && (Launch<T>::col_smem(log_n, f) > 100 * 1024 ||
+                   (std::is_same<T, float>::value && (long long)nkx * ninst < 2LL * 152 * f)))
+    f /= 2;
   return std::min(f, nkx);
 }
 

@@ -166,7 +166,7 @@ extern "C" fill_status fill_apply_static(int ny, int nx, const double* P_half,
   if (L.total > kStaticScratchBytes)
     return reject("grid too large for the 8 MiB static scratch (at most about 1024 x 1024 pixels)");
   // the launch schedule of a plan with default options on this grid
-  const int rows = default_rows<float>(log_l, ny), ffts = default_ffts<float>(log_n, nx / 2 + 1);
+  const int rows = default_rows<float>(log_l, ny), ffts = default_ffts<float>(log_n, nx / 2 + 1, 1);
   if (!schedule_valid<float>(log_l, log_n, ny, rows, ffts))
     return reject("no valid launch schedule for this grid");
   // an error left pending by earlier, unrelated work would otherwise be

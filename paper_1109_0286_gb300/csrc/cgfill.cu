@@ -170,6 +170,7 @@ struct Precision {
   InstDesc<T>* desc = nullptr;  // device, batch
   InstDesc<T>* hdesc = nullptr; // pinned
   int rows = 0, ffts = 0;
+  bool ffts_auto = false;       // ffts is the default for the plan's batch
   int col_variant = 0;          // column kernel of the table passes (ColArgs::variant)
   bool used = false;
   cudaGraphExec_t iter_graph = nullptr;   // CG loop graph (conditional WHILE node)
@@ -1374,7 +1375,8 @@ fill_status setup_precision(fill_plan* p, const std::vector<double>& tinv,
     P.rows = user && p->o.rows_per_cta > 0 ? fit_rows<T>(p->log_l, std::min(p->o.rows_per_cta, p->ny))
                                            : default_rows<T>(p->log_l, p->ny);
     P.ffts = user && p->o.ffts_per_cta > 0 ? fit_ffts<T>(p->log_n, p->o.ffts_per_cta)
-                                           : default_ffts<T>(p->log_n, p->nx / 2 + 1);
+                                           : default_ffts<T>(p->log_n, p->nx / 2 + 1, p->batch);
+    P.ffts_auto = !(user && p->o.ffts_per_cta > 0);
     if (!schedule_valid<T>(p->log_l, p->log_n, p->ny, P.rows, P.ffts)) return FILL_EINVAL;
     P.col_variant = std::is_same<T, float>::value ? p->o.col_kernel : 0;
   }
@@ -2452,6 +2454,7 @@ fill_status tune_plan_t(fill_plan* p, const char* path) {
   if (rows != P.rows || nf != P.ffts || nv != P.col_variant) {
     P.rows = rows;
     P.ffts = nf;
+    P.ffts_auto = false;
     P.col_variant = nv;
     if (P.iter_graph) {
       cudaGraphExecDestroy(P.iter_graph);
@@ -2665,7 +2668,8 @@ fill_status group_setup(fill_group* g, int autotune, const char* path) {
     }
     fill_plan* p0 = g->plans[c.plans[0]];
     c.rows = prec<T>(p0).rows;
-    c.ffts = prec<T>(p0).ffts;
+    c.ffts = prec<T>(p0).ffts_auto ? default_ffts<T>(c.log_n, c.nx / 2 + 1, c.ninst)
+                                   : prec<T>(p0).ffts;
     c.col_variant = prec<T>(p0).col_variant;
     CK(cudaMemcpy(c.desc, c.hdesc, nb, cudaMemcpyHostToDevice));
     if (autotune && !p0->gen) {   // mixed-radix classes keep their fixed schedule
@@ -2719,7 +2723,7 @@ fill_status group_setup_hi(fill_group* g) {
     }
     fill_plan* p0 = g->plans[c.plans[0]];
     c.rows_hi = p0->h.rows;
-    c.ffts_hi = p0->h.ffts;
+    c.ffts_hi = p0->h.ffts_auto ? default_ffts<df>(c.log_n, c.nx / 2 + 1, c.ninst) : p0->h.ffts;
     c.col_variant_hi = p0->h.col_variant;
     CK(cudaMemcpy(c.desc_hi, c.hdesc_hi, nb, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c.stp_hi, ptrs.data(), sizeof(CgState*) * ptrs.size(), cudaMemcpyHostToDevice));
