@@ -495,7 +495,7 @@ __device__ __forceinline__ cx<T> mid_op(const InstDesc<T>& I, const Opnd& o, T d
   }
 }
 
-// Operations whose inputs and outputs are all compact CG vectors: a pixel
+// Operations whose inputs and outputs are all CG vectors (masked pixels only): a pixel
 // pair without a masked pixel reads nothing, writes nothing, adds nothing to
 // the reduction and (sources) contributes zeros to the transform.
 template <int OP>

@@ -45,8 +45,9 @@ constexpr int kGenMaxLen = 4096;   // nx / 2 and ny at most 4096
 struct GenLen {
   int n;
   int nst;
-  int nt;
-  int code;   // radix schedule (gen_factor)
+  int nt;       // threads per group (gen_threads)
+  int nt_base;  // nt before the few-transform rule (gen_threads): admits CTA shapes
+  int code;     // radix schedule (gen_factor)
   int radix[kGenMaxStages];
   // Stage s < nst - 1: twiddles W_{n_s}^{q j} (j < h_s, q = 1 .. R_s - 1) at
   // complex entry twoff[s] + (q - 1) h_s + j of the table, so that the threads

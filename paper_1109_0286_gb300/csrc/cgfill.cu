@@ -1131,19 +1131,32 @@ void gen_tables(const GenLen& g, std::vector<double>& tw, std::vector<unsigned s
 }
 
 // Threads per group of V mixed-radix transforms (a multiple of 32, at most
-// 512).  A stage of radix R has n/R butterflies, shared round-robin by the
+// kGenThreads).  A stage of radix R has n/R butterflies, shared round-robin by the
 // group's threads; the last round leaves threads idle.  Among the
 // candidates, take the one with the best product of stage efficiency
 // (butterflies / thread slots over all stages) and SM occupancy (groups
 // resident per SM by shared memory -- V n complex values each -- times
 // threads, against the threads an SM runs at the kernels' register counts:
 // kGenThreads x gen_minb).
-void gen_threads(GenLen* g, int V, bool wide) {
+//
+// If one map's `count` transforms leave the chip half empty at that width, a
+// pass of a few maps is one wave of CTAs and its time the rounds of a group:
+// then the fewest threads that need the fewest rounds over all stages, among
+// those within 0.8 of the best product, at most `cap`.  The columns stop at
+// 64 threads: a CTA of wider groups holds fewer columns, and its loads get
+// shorter than a sector (600 x 7000 with 128: column pass 69 -> 88 us).
+// Measured, whole calls to 1e-6, before -> now: 375 x 1050 FP32 one map 11.5
+// -> 7.4 ms, three 13.1 -> 9.2; FP64 38.8 -> 28.8; 600 x 700 four maps 22.6 ->
+// 18.6; the 32 lanes of a 480^2 gradient 31.1 -> 25.9.  With 0.9 in place of 0.8: 9.8,
+// 10.4, 38.8, 18.6, 31.1.  Groups that fill the chip with many maps of such a
+// grid lose up to the 0.8: 16 maps of 600 x 700 25.5 -> 27.5 ms, of 280 x 504
+// 9.9 -> 11.4.  The choice cannot follow the batch: a thread's share of a sum
+// is its share of the row, and a map's sums do not depend on its neighbours.
+void gen_threads(GenLen* g, int V, bool wide, int count, int cap) {
   const double tmax = double(kGenThreads) * (wide ? gen_minb<double>() : gen_minb<float>());
   const size_t bytes = size_t(V) * g->n * (wide ? 16 : 8);
   const size_t per_sm = std::max<size_t>(1, size_t(225) * 1024 / bytes);
-  double best = -1.0;
-  for (int nt = 32; nt <= kGenThreads; nt += 32) {
+  auto score_of = [&](int nt) {
     long long slots_used = 0, work = 0;
     for (int s = 0; s < g->nst; ++s) {
       const int nb = g->n / g->radix[s];
@@ -1152,9 +1165,24 @@ void gen_threads(GenLen* g, int V, bool wide) {
     }
     const double eff = double(work) / double(slots_used);
     const double resident = std::min<double>(double(per_sm), std::floor(tmax / nt));
-    const double score = eff * std::min(1.0, resident * nt / tmax);
+    return eff * std::min(1.0, resident * nt / tmax);
+  };
+  double best = -1.0;
+  for (int nt = 32; nt <= kGenThreads; nt += 32) {
+    const double score = score_of(nt);
     if (score > best + 1e-9 || (score > best - 1e-9 && nt > g->nt)) {
       best = std::max(best, score);
+      g->nt = nt;
+    }
+  }
+  g->nt_base = g->nt;
+  if (double((count + V - 1) / V) * g->nt > 0.5 * 152.0 * tmax) return;
+  int least = 1 << 30;
+  for (int nt = g->nt; nt <= cap; nt += 32) {
+    int rounds = 0;
+    for (int s = 0; s < g->nst; ++s) rounds += (g->n / g->radix[s] + nt - 1) / nt;
+    if (rounds < least && score_of(nt) >= 0.8 * best) {
+      least = rounds;
       g->nt = nt;
     }
   }
@@ -1174,16 +1202,31 @@ bool loop_precision(const fill_plan* p) {
 // row groups a power of two, within kGenThreads threads, the partial-sum slots
 // and 200 KB of shared memory (the mask words take up to 13 KB more).
 template <typename T>
-bool gen_row_ok(const fill_plan* p, int r) {
+bool gen_row_ok(const fill_plan* p, int r, int nt) {
   constexpr int V = gen_vrow<T>();
-  return r >= V && r % V == 0 && pow2(r / V) && (r / V) * p->grow.nt <= GenLaunch<T>::max_threads() &&
+  return r >= V && r % V == 0 && pow2(r / V) && (r / V) * nt <= GenLaunch<T>::max_threads() &&
          (p->ny + r - 1) / r <= kMaxPartials && GenLaunch<T>::row_main(p->nx / 2, r) <= 200 * 1024;
 }
 template <typename T>
-bool gen_col_ok(const fill_plan* p, int f) {
+bool gen_col_ok(const fill_plan* p, int f, int nt) {
   constexpr int V = gen_v<T>();
-  return f >= V && f % V == 0 && (f / V) * p->gcol.nt <= GenLaunch<T>::max_threads() &&
+  return f >= V && f % V == 0 && (f / V) * nt <= GenLaunch<T>::max_threads() &&
          GenLaunch<T>::col_smem(p->ny, f) <= 200 * 1024;
+}
+
+// A CTA shape asked for by the options or read from a tuning cache: admitted by
+// the width that the stages and the occupancy ask for (GenLen::nt_base), then
+// cut to the groups of nt threads that one CTA holds.
+template <typename T>
+int gen_fit_rows(const fill_plan* p, int r) {
+  if (!gen_row_ok<T>(p, r, p->grow.nt_base)) return r;
+  while (r / gen_vrow<T>() * p->grow.nt > GenLaunch<T>::max_threads()) r /= 2;
+  return r;
+}
+template <typename T>
+int gen_fit_ffts(const fill_plan* p, int f) {
+  if (!gen_col_ok<T>(p, f, p->gcol.nt_base)) return f;
+  return std::min(f, GenLaunch<T>::max_threads() / p->gcol.nt * gen_v<T>());
 }
 
 // Twiddle tables of precision T for the plan's current radix schedules, in
@@ -1244,22 +1287,22 @@ fill_status setup_generic(fill_plan* p) {
   const int ctas = 2 * 152;
   const bool user = loop_precision<T>(p);
   if (user && p->o.rows_per_cta > 0) {
-    P.rows = p->o.rows_per_cta;
+    P.rows = gen_fit_rows<T>(p, p->o.rows_per_cta);
   } else {
     P.rows = VR;
-    if (gen_row_ok<T>(p, 2 * VR) && GenLaunch<T>::row_smem(p->nx / 2, 2 * VR) <= third &&
+    if (gen_row_ok<T>(p, 2 * VR, p->grow.nt) && GenLaunch<T>::row_smem(p->nx / 2, 2 * VR) <= third &&
         (long long)p->ny * p->batch >= 2LL * VR * ctas)
       P.rows = 2 * VR;
   }
   if (user && p->o.ffts_per_cta > 0) {
-    P.ffts = p->o.ffts_per_cta;
+    P.ffts = gen_fit_ffts<T>(p, p->o.ffts_per_cta);
   } else {
     P.ffts = V;
-    while (gen_col_ok<T>(p, 2 * P.ffts) && GenLaunch<T>::col_smem(p->ny, 2 * P.ffts) <= third &&
+    while (gen_col_ok<T>(p, 2 * P.ffts, p->gcol.nt) && GenLaunch<T>::col_smem(p->ny, 2 * P.ffts) <= third &&
            2 * P.ffts <= 16 && (long long)(p->nx / 2 + 1) * p->batch >= 2LL * P.ffts * ctas)
       P.ffts *= 2;
   }
-  if (!gen_row_ok<T>(p, P.rows) || !gen_col_ok<T>(p, P.ffts)) return FILL_EINVAL;
+  if (!gen_row_ok<T>(p, P.rows, p->grow.nt) || !gen_col_ok<T>(p, P.ffts, p->gcol.nt)) return FILL_EINVAL;
   fill_status fs = gen_upload<T>(p);
   if (fs != FILL_OK) return fs;
   if (!p->grow.rev) {
@@ -1326,7 +1369,7 @@ fill_status setup_precision(fill_plan* p, const std::vector<double>& tinv,
   P.used = true;
   const size_t B = p->batch, n = p->npix, nv = p->nv;
   const size_t nspec = 2 * size_t(p->nx / 2 + 1) * p->ny;
-  T** cvecs[] = {&P.r, &P.p, &P.q, &P.z, &P.u, &P.b};   // compact CG vectors
+  T** cvecs[] = {&P.r, &P.p, &P.q, &P.z, &P.u, &P.b};   // CG vectors (nvec values)
   for (T** v : cvecs)
     if (p->dalloc(v, B * nv) != cudaSuccess) return FILL_ENOMEM;
   if (p->dalloc(&P.y, B * n) != cudaSuccess || p->dalloc(&P.w, B * n) != cudaSuccess)
@@ -1505,8 +1548,8 @@ fill_status fill_init(fill_plan** out, int ny, int nx, const double* P_half,
       return FILL_EINVAL;
     // threads per transform, for the precision that carries the CG loop
     const bool wide = opts && opts->mode == FILL_MODE_FP64;
-    gen_threads(&grow, wide ? 1 : gen_vrow<float>(), wide);
-    gen_threads(&gcol, wide ? 1 : gen_v<float>(), wide);
+    gen_threads(&grow, wide ? 1 : gen_vrow<float>(), wide, ny, kGenThreads);
+    gen_threads(&gcol, wide ? 1 : gen_v<float>(), wide, nx / 2 + 1, 64);
   }
   fill_opts o;
   if (opts)
@@ -2095,7 +2138,7 @@ fill_status time_pass_t(fill_plan* p, int pass, int reps, double* ms, double* by
       default: return row<T>(p, s, OP_MASK, SC_NONE, true, true, false);
     }
   };
-  // per instance: compact CG vectors (nM values), spectra; once per launch
+  // per instance: the masked pixels' CG values (nM), spectra; once per launch
   // (shared by the batch): the column table, the mask words (8 bytes per 32 pixels)
   const double nM = double(p->nmasked), MW = n / 4.0;
   double b = 0.0, shared = MW;
@@ -2532,7 +2575,7 @@ fill_status tune_gen_t(fill_plan* p, const char* path) {
       fill_status fs = apply_gen_code(p, true, code);
       if (fs != FILL_OK) return fs;
       for (int r = gen_vrow<T>(); r <= 4 * gen_vrow<T>(); r *= 2) {
-        if (!gen_row_ok<T>(p, r)) continue;
+        if (!gen_row_ok<T>(p, r, p->grow.nt)) continue;
         Ctx<T> c = ctx<T>(p);
         c.rows = r;
         float ms = 0.f;
@@ -2549,7 +2592,7 @@ fill_status tune_gen_t(fill_plan* p, const char* path) {
       fill_status fs = apply_gen_code(p, false, code);
       if (fs != FILL_OK) return fs;
       for (int f = V; f <= 16; f *= 2) {
-        if (!gen_col_ok<T>(p, f)) continue;
+        if (!gen_col_ok<T>(p, f, p->gcol.nt)) continue;
         Ctx<T> c = ctx<T>(p);
         c.ffts = f;
         float ms = 0.f;
@@ -2563,7 +2606,9 @@ fill_status tune_gen_t(fill_plan* p, const char* path) {
     }
     cache_store_gen(path, pr, p->ny, p->nx, p->batch, rows, ffts, rcode, ccode);
   }
-  if (!gen_row_ok<T>(p, rows) || !gen_col_ok<T>(p, ffts)) return FILL_EINVAL;
+  rows = gen_fit_rows<T>(p, rows);
+  ffts = gen_fit_ffts<T>(p, ffts);
+  if (!gen_row_ok<T>(p, rows, p->grow.nt) || !gen_col_ok<T>(p, ffts, p->gcol.nt)) return FILL_EINVAL;
   fill_status fs = apply_gen_code(p, true, rcode);
   if (fs == FILL_OK) fs = apply_gen_code(p, false, ccode);
   if (fs != FILL_OK) return fs;
