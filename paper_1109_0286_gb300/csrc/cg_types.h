@@ -244,6 +244,10 @@ constexpr int kLmax = 8192;        // twiddle master table: W_8192^m
 //   FP32, us per CG iteration: 64^2 62, 44, 38; 256^2 65, 53, 46 (16 maps 71,
 //   66, 71; rows 8 and columns 4: 49 and 67); 512^2 69, 55, 56 (16 maps 128,
 //   137, 186); 1024^2 76, 72, 78 (16 maps 359, 477, 424); 2048^2 149, 183, -.
+//   (256^2 with rows of 8: columns of 4 or 8, one map 2.26, 2.33 ms a call, a
+//   group of 24 maps 4.34, 4.06; 128 x 256^2 + 96 x 512^2 + 32 x 1024^2 in one group
+//   133.8, 131.3, in mixed precision 280.3, 275.8: 8.  That group with 16 everywhere
+//   117, 251, but single maps of 256^2 2.84, of 512^2 3.92 against 3.24: not taken.)
 //   FP64: 64^2 264, -, 82; 512^2 586, -, 165; 1024^2 966, -, 606.  An FP64
 //   instruction holds its scheduler's pipe for 64 cycles, so a short chain
 //   counts most; from 2048 pixels on, 8 and 16 keep the rows of a CTA.
@@ -253,7 +257,7 @@ constexpr int kLmax = 8192;        // twiddle master table: W_8192^m
 template <typename T>
 CGF_HD constexpr int row_le(int log) { return log <= 6 ? 2 : log <= 8 ? 3 : 4; }
 template <typename T>
-CGF_HD constexpr int col_le(int log) { return log <= 8 ? 2 : log <= 9 ? 3 : 4; }
+CGF_HD constexpr int col_le(int log) { return log <= 7 ? 2 : log <= 9 ? 3 : 4; }
 struct df;
 template <>
 CGF_HD constexpr int row_le<df>(int log) { return log <= 8 ? 2 : log <= 11 ? 3 : 4; }
