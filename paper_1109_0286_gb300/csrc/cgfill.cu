@@ -465,7 +465,7 @@ cudaError_t vec(fill_plan* p, cudaStream_t s, int op, int sop, int skip) {
 
 // Unconstrained draw and right-hand side (Sects. 2.3, 2.1):
 //   y = F^-1 sqrt(P) F xi;  b = -P_x F^-1 (1/P) F [(d - y) on U].
-// Iterations per loop body.  A body costs 8 us of its own (the control kernel
+// Iterations per loop body.  A body costs 6 us of its own (the control kernel
 // and the WHILE node) next to iterations of 30-60 us on small grids (64^2
 // FP32 with 1, 2, 4 iterations per body: 36, 34, 32 us per iteration);
 // iterations past the last convergence only cost their kernels' early exits.
