@@ -450,15 +450,11 @@ __device__ __forceinline__ void scalar_update(int sop, CgState* st, const CgStat
       st->rr = sum;
       st->iter = iter;
       record_hist(c, iter, sum);
-      if (!isfinite(sum)) {
-        stop(st, 4);
-        c.peer->upd = 1;   // fold what was gained and report the true residual
-      } else if (sum <= c.delta2 * c.rrmax || sum <= c.tol2 * c.bb) {
-        c.peer->upd = 1;
-      } else if (iter >= c.max_iter) {
-        stop(st, 3);
-        c.peer->upd = 1;
-      }
+      // at the end of the iterations, too: fold what was gained and report the
+      // true residual (which may have converged)
+      const bool fails = !isfinite(sum), end = iter >= c.max_iter;
+      if (fails || end) stop(st, fails ? 4 : 3);
+      if (fails || end || sum <= c.delta2 * c.rrmax || sum <= c.tol2 * c.bb) c.peer->upd = 1;
       break;
     }
     case SC_RES_UPD: {

@@ -463,14 +463,20 @@ cudaError_t vec(fill_plan* p, cudaStream_t s, int op, int sop, int skip) {
     if (e_ != cudaSuccess) return e_;         \
   } while (0)
 
-// Unconstrained draw and right-hand side (Sects. 2.3, 2.1):
-//   y = F^-1 sqrt(P) F xi;  b = -P_x F^-1 (1/P) F [(d - y) on U].
 // Iterations per loop body.  A body costs 6 us of its own (the control kernel
 // and the WHILE node) next to iterations of 30-60 us on small grids (64^2
 // FP32 with 1, 2, 4 iterations per body: 36, 34, 32 us per iteration);
 // iterations past the last convergence only cost their kernels' early exits.
 constexpr int kLoopUnroll = 4;
 
+// Bodies after which a loop ends whatever the states say: the first to reach
+// max_iter + 4 iterations (each instance stops at max_iter by itself).
+int body_limit(int max_iter) {
+  return (int)(((long long)max_iter + 4 + kLoopUnroll - 1) / kLoopUnroll);
+}
+
+// Unconstrained draw and right-hand side (Sects. 2.3, 2.1):
+//   y = F^-1 sqrt(P) F xi;  b = -P_x F^-1 (1/P) F [(d - y) on U].
 template <typename T>
 cudaError_t draw_and_rhs(const Ctx<T>& c, cudaStream_t s, bool plain_cg) {
   CE(row<T>(c, s, OP_XI, SC_NONE, false, true, false));
@@ -708,7 +714,7 @@ fill_status build_iter_graph(fill_plan* p) {
   if (P.iter_graph) return FILL_OK;
   return build_loop_graph(
       p->cap, [&](cudaStream_t s) { return pcg_body<T>(p, s, true); }, P.stp, p->batch,
-      p->loop_counter, p->o.max_iter + 4, &p->launches, &P.iter_graph, &P.iter_graph_kernels);
+      p->loop_counter, body_limit(p->o.max_iter), &p->launches, &P.iter_graph, &P.iter_graph_kernels);
 }
 
 // Runs CG iterations until every instance's state is done: one launch of the
@@ -719,7 +725,7 @@ fill_status run_pcg(fill_plan* p) {
   if (p->o.host_loops)
     return run_loop_host(
         p->s, [&](cudaStream_t s) { return pcg_body<T>(p, s); }, P.stp, p->batch,
-        p->loop_counter, p->hloop, p->o.max_iter + 4, &p->launches);
+        p->loop_counter, p->hloop, body_limit(p->o.max_iter), &p->launches);
   fill_status fs = build_iter_graph<T>(p);
   if (fs != FILL_OK) return fs;
   return run_loop_graph(p, P.iter_graph, P.iter_graph_kernels);
@@ -936,7 +942,7 @@ fill_status build_mixed_graph(fill_plan* p) {
   if (p->mixed_graph) return FILL_OK;
   return build_loop_graph(
       p->cap, [&](cudaStream_t s) { return mixed_body(p, s, true); }, p->f.stp, p->batch,
-      p->loop_counter, p->o.max_iter + 4, &p->launches, &p->mixed_graph, &p->mixed_graph_kernels);
+      p->loop_counter, body_limit(p->o.max_iter), &p->launches, &p->mixed_graph, &p->mixed_graph_kernels);
 }
 
 // Mixed-precision solve with reliable updates (b, r, r32 and the high-precision state
@@ -947,7 +953,7 @@ fill_status mixed_reliable(fill_plan* p, double tol) {
   if (p->o.host_loops) {
     fs = run_loop_host(
         p->s, [&](cudaStream_t s) { return mixed_body(p, s, false); }, p->f.stp, p->batch,
-        p->loop_counter, p->hloop, p->o.max_iter + 4, &p->launches);
+        p->loop_counter, p->hloop, body_limit(p->o.max_iter), &p->launches);
   } else {
     fs = build_mixed_graph(p);
     if (fs != FILL_OK) return fs;
@@ -2810,7 +2816,7 @@ fill_status group_build_graph(fill_group* g) {
         }
         return cudaSuccess;
       },
-      g->stp, g->ntot, g->counter, g->max_iter + 4, &g->launches, &g->graph, &g->graph_kernels);
+      g->stp, g->ntot, g->counter, body_limit(g->max_iter), &g->launches, &g->graph, &g->graph_kernels);
 }
 
 // The same for a mixed group: each class's body is the reliable-update
@@ -2819,7 +2825,7 @@ fill_status group_build_mixed_graph(fill_group* g) {
   if (g->graph) return FILL_OK;
   return build_loop_graph(
       g->cap, [&](cudaStream_t cap) { return group_mixed_body(g, cap, g->fork_cap, false); },
-      g->stp, g->ntot, g->counter, g->max_iter + 4, &g->launches, &g->graph, &g->graph_kernels);
+      g->stp, g->ntot, g->counter, body_limit(g->max_iter), &g->launches, &g->graph, &g->graph_kernels);
 }
 
 // Starts every class on its own stream after `s` reaches this point, and
@@ -2878,7 +2884,7 @@ fill_status group_realize_t(fill_group* g, const void* const* d, const uint64_t*
           }
           return cudaSuccess;
         },
-        g->stp, g->ntot, g->counter, g->hloop, g->max_iter + 4, &g->launches);
+        g->stp, g->ntot, g->counter, g->hloop, body_limit(g->max_iter), &g->launches);
     if (fs != FILL_OK) return fs;
   } else {
     fs = group_build_graph<T>(g);
@@ -2965,7 +2971,7 @@ fill_status group_realize_mixed(fill_group* g, const void* const* d, const uint6
   if (g->host_loops) {
     fs = run_loop_host(
         g->s, [&](cudaStream_t s) { return group_mixed_body(g, s, g->fork, true); }, g->stp,
-        g->ntot, g->counter, g->hloop, g->max_iter + 4, &g->launches);
+        g->ntot, g->counter, g->hloop, body_limit(g->max_iter), &g->launches);
     if (fs != FILL_OK) return fs;
   } else {
     fs = group_build_mixed_graph(g);
