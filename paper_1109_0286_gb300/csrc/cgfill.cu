@@ -678,10 +678,10 @@ fill_status run_loop_graph(fill_plan* p, cudaGraphExec_t exec, long long body_ke
 
 // Host-driven form of a loop graph (opts.host_loops = 1): the body's kernels
 // are launched from the host and the instances' done flags are read back
-// every kHostCheck bodies; bodies past the last convergence cost only the
-// kernels' early exits.  For profilers that cannot see kernels inside
-// conditional graph nodes.
-constexpr int kHostCheck = 8;
+// every kHostCheck bodies (8 iterations); iterations past the last convergence
+// cost only the kernels' early exits.  For profilers that cannot see kernels
+// inside conditional graph nodes.
+constexpr int kHostCheck = 8 / kLoopUnroll;
 
 __global__ void k_any_running(CgState* const* sts, int n, int* flag) {
   __shared__ int running;

@@ -48,3 +48,21 @@ def test_updates_every_iteration_stop_at_max_iter(ny, nx, precond, max_iter):
     plan = cg.Plan(P, obs, precond=precond, update_delta=0.9, max_iter=need)
     _, st = plan.ml(dg, 1e-12)
     assert (st[0]["iters"], st[0]["status"]) == (need, OK)
+
+
+@pytest.mark.parametrize("precond", [True, False])
+@pytest.mark.parametrize("iters", [1, 8, 33])
+def test_host_loop_checks_every_8_iterations(precond, iters):
+    """Kernels of a host-driven solve of `iters` iterations: those of the graph
+    form, up to 8 iterations more, and one check per 8 iterations."""
+    _, obs, d = flat_case(64, 64)
+    P = synth.spectrum_cmb_like(64, 64, 2 * np.pi / 64)   # some 50 iterations to 1e-6
+    dg = torch.from_numpy(d).float().cuda()
+    n = []
+    for host in (False, True):
+        plan = cg.Plan(P, obs, mode="fp32", precond=precond, max_iter=iters, host_loops=host)
+        _, st = plan.ml(dg, 0.0, check=False)
+        assert (st[0]["iters"], st[0]["status"]) == (iters, ENOTCONV)
+        n.append(st[0]["launches"])
+    passes = 8 if precond else 4
+    assert n[1] - n[0] <= 8 * passes + iters // 8 + 1
