@@ -248,6 +248,18 @@ struct fill_plan {
     }
     return e;
   }
+  // A larger buffer in place of *p, whose contents are dropped; on failure *p
+  // stays as it is.  (For buffers that no captured graph holds.)
+  template <typename X>
+  cudaError_t dgrow(X** p, size_t count) {
+    X* const old = *p;
+    cudaError_t e = dalloc(p, count);
+    if (e == cudaSuccess && old) {
+      dev.erase(std::find(dev.begin(), dev.end(), (void*)old));
+      e = cudaFree(old);
+    }
+    return e;
+  }
   template <typename X>
   cudaError_t halloc(X** p, size_t count) {
     void* v = nullptr;
@@ -1836,24 +1848,29 @@ long long annulus_count(double r_in, double r_out) {
   return c;
 }
 
+// Room for the spectra of the kernels that run together (Sect. 6.3 solver).
+constexpr size_t kAnnuliBytes = size_t(512) << 20;
+
 // Kernel tables 1/(count n) Re F(annulus_j) of the Sect. 6.3 solver, from the
 // annulus images by the plan's own forward transforms (instance 0's buffers).
 template <typename T>
 fill_status set_annuli_t(fill_plan* p, int nk, const double* r_in, const double* r_out) {
   Precision<T>& P = prec<T>(p);
-  if (!P.used) return FILL_OK;
   const size_t ntab = size_t(p->nx / 2 + 1) * p->ny;
   if (nk > P.nk_cap) {
-    if (p->dalloc(&P.kt, size_t(nk) * ntab) != cudaSuccess) return FILL_ENOMEM;
+    if (p->dgrow(&P.kt, size_t(nk) * ntab) != cudaSuccess) return FILL_ENOMEM;
     P.nk_cap = nk;
+    P.nk = 0;   // no annuli until the tables are filled
   }
   const size_t nspec = 2 * ntab;
-  // spectra for all kernels at once (within 4 GB, or as many as there is room
-  // for: the solver then takes the kernels in turns of kz)
+  // spectra for all kernels at once, within kAnnuliBytes or as many as there is
+  // room for, at least one: the solver then takes the kernels in turns of kz.
+  // (What a launch for several kernels saves is the gaps between small
+  // launches; one kernel's spectra of this size fill the chip by themselves.)
   if (P.kz < nk) {
     const size_t one = size_t(p->batch) * nspec * sizeof(T);
-    int kz = (int)std::max<size_t>(1, std::min<size_t>(nk, (size_t(4) << 30) / one));
-    while (kz > P.kz && p->dalloc(&P.speck, size_t(kz) * p->batch * nspec) != cudaSuccess) {
+    int kz = (int)std::max<size_t>(1, std::min<size_t>(nk, kAnnuliBytes / one));
+    while (kz > P.kz && p->dgrow(&P.speck, size_t(kz) * p->batch * nspec) != cudaSuccess) {
       cudaGetLastError();
       if (kz == 1) return FILL_ENOMEM;
       kz /= 2;
@@ -1947,10 +1964,9 @@ fill_status fill_set_annuli(fill_plan* p, int nk, const double* r_in, const doub
     if (!(r_in[j] >= 0.0) || !(r_out[j] > r_in[j]) || 2.0 * r_out[j] >= double(p->nx) ||
         2.0 * r_out[j] >= double(p->ny) || annulus_count(r_in[j], r_out[j]) == 0)
       return FILL_EINVAL;
-  fill_status fs = set_annuli_t<float>(p, nk, r_in, r_out);
-  if (fs == FILL_OK) fs = set_annuli_t<double>(p, nk, r_in, r_out);
-  if (fs == FILL_OK) fs = set_annuli_t<df>(p, nk, r_in, r_out);
-  return fs;
+  return p->o.mode == FILL_MODE_FP32   ? set_annuli_t<float>(p, nk, r_in, r_out)
+         : p->o.mode == FILL_MODE_FP64 ? set_annuli_t<double>(p, nk, r_in, r_out)
+                                       : set_annuli_t<df>(p, nk, r_in, r_out);
 }
 
 fill_status fill_laplace_ms(fill_plan* p, const void* d, long long d_stride, int iters,
