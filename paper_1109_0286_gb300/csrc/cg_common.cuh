@@ -302,6 +302,24 @@ __device__ __forceinline__ void normal_pair(const double* __restrict__ tab,
 // ---------------------------------------------------------------------------
 template <typename T> struct Acc;
 
+// A sum in three FP32 parts.  The additions are exact but for the last parts'
+// (2^-24 of what the first two, 48 bits, leave): closer than FP64.
+struct Sum3 {
+  float h, m, l;
+};
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = a + b, v = s - a;
+  e = (a - (s - v)) + (b - v);
+  return s;
+}
+__device__ __forceinline__ Sum3 operator+(Sum3 a, Sum3 b) {
+  float e, f, g;
+  const float h = two_sum(a.h, b.h, e);
+  const float t = two_sum(a.m, b.m, f);
+  const float m = two_sum(e, t, g);
+  return {h, m, (a.l + b.l) + (f + g)};
+}
+
 template <>
 struct Acc<float> {
   float hi = 0.f, lo = 0.f;
@@ -314,17 +332,14 @@ struct Acc<float> {
     lo += e + e2;
     hi = t;
   }
-  __device__ __forceinline__ df total() const {   // renormalised pair
-    const float h = hi + lo;
-    return df(h, lo - (h - hi));
-  }
+  __device__ __forceinline__ Sum3 total() const { return {hi, lo, 0.f}; }
 };
 
 template <>
 struct Acc<df> {
   df s = df(0.f, 0.f);
   __device__ __forceinline__ void add_prod(df a, df b) { s = s + a * b; }
-  __device__ __forceinline__ df total() const { return s; }
+  __device__ __forceinline__ Sum3 total() const { return {s.hi, s.lo, 0.f}; }
 };
 
 template <>
@@ -335,18 +350,21 @@ struct Acc<double> {
 };
 
 // Partial sums in transit between threads: FP32 and double-float passes carry
-// pairs (hi, lo), FP64 passes doubles.
-__device__ __forceinline__ df shfl_down_sum(unsigned mask, df v, int o) {
-  return df(__shfl_down_sync(mask, v.hi, o), __shfl_down_sync(mask, v.lo, o));
+// three FP32 parts, FP64 passes doubles.
+__device__ __forceinline__ Sum3 shfl_down_sum(unsigned mask, Sum3 v, int o) {
+  return {__shfl_down_sync(mask, v.h, o), __shfl_down_sync(mask, v.m, o),
+          __shfl_down_sync(mask, v.l, o)};
 }
 __device__ __forceinline__ double shfl_down_sum(unsigned mask, double v, int o) {
   return __shfl_down_sync(mask, v, o);
 }
-__device__ __forceinline__ double sum_value(df v) { return (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ double sum_value(Sum3 v) {
+  return (double)v.h + ((double)v.m + (double)v.l);
+}
 __device__ __forceinline__ double sum_value(double v) { return v; }
-// A pair whose high part is this large could overflow FP32 in the sum of a
+// A sum whose first part is this large could overflow FP32 in the sum of a
 // CTA (at most 1024 threads); such sums go through FP64.
-__device__ __forceinline__ bool sum_large(df v) { return !(fabsf(v.hi) < 1e34f); }
+__device__ __forceinline__ bool sum_large(Sum3 v) { return !(fabsf(v.h) < 1e34f); }
 __device__ __forceinline__ bool sum_large(double) { return false; }
 
 // Sum over the segments of `len` consecutive lanes of a warp (len <= 32, any
@@ -522,10 +540,11 @@ __device__ __forceinline__ float cg_beta<float>(const CgState* st) { return st->
 // Every order is fixed and, for a given seg, independent of how many segments
 // a CTA holds, so results are reproducible and do not depend on the CTA shape.
 // What bounds it is the FP64 pipe (64 cycles per dependent instruction): the
-// sums inside a CTA are pairs of FP32 values added with TwoSum (about 2^-47
-// of the sum per addition, below the 2^-44 of a thread's own compensated
-// sum), only a segment's total becomes a double, and the last CTA adds the
-// partials on 32 lanes in parallel.  Measured against shuffles and sums in
+// sums inside a CTA are carried in three FP32 parts (Sum3: no further from
+// the exact sum than FP64 additions; in two parts, 2^-47 per addition, sums
+// with cancellation came out 1.8 times as far; the third part costs 1% of an
+// iteration, 679 -> 686 ms a call at 8 x 4096^2), only a segment's total becomes
+// a double, and the last CTA adds the partials in FP64 on 32 lanes in parallel.  Measured against shuffles and sums in
 // FP64 with one thread adding the partials (1024 of them at 4096^2, 32 us):
 // 4096^2, one map, sink 104 -> 59 us, r-update 124 -> 76 us; an iteration of
 // 1024^2 94.5 -> 84 us; 600 x 7000 x 4, r-update 106 -> 93 us.
@@ -551,7 +570,7 @@ __device__ __forceinline__ void grid_reduce(V v, double* sh, double* partial, Cg
     if (__any_sync(mask, sum_large(w))) s = segment_sum(sum_value(v), mask, lane, nl, seg);
     if (lane % seg == 0) out[tid / seg] = s;
   } else {
-    V* shv = reinterpret_cast<V*>(sh);
+    __shared__ V shv[32];
     __shared__ int large;
     if (tid == 0) large = 0;
     V w = segment_sum(v, mask, lane, nl, 32);
@@ -572,7 +591,7 @@ __device__ __forceinline__ void grid_reduce(V v, double* sh, double* partial, Cg
         if (lane < nw && lane % wps == 0) out[lane / wps] = t;
       }
     } else if (wid == 0) {
-      const V t = segment_sum(lane < nw ? shv[lane] : V(0.0), mask, lane, min(nw, nl), wps);
+      const V t = segment_sum(lane < nw ? shv[lane] : V{}, mask, lane, min(nw, nl), wps);
       if (lane < nw && lane % wps == 0) out[lane / wps] = sum_value(t);
     }
   }

@@ -1,0 +1,71 @@
+"""GPU: device functions by themselves (device_probe.cu, built here with nvcc)."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1109_0286_gb300 import _build  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("probe") / "probe.so")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "device_probe.cu")
+    subprocess.run([_build._nvcc(), *_build.ARCH, *_build.FLAGS, "-shared", "-o", so, src], check=True)
+    lib = ctypes.CDLL(so)
+    lib.probe_reduce.argtypes = [ctypes.c_int] * 4 + [ctypes.c_void_p] * 5
+    return lib
+
+
+TYPES = {"fp32": 0, "mixed": 1, "fp64": 2}
+
+
+@pytest.mark.parametrize("power", [0, 99, (0, 99)])
+@pytest.mark.parametrize("ncta,nthr,seg", [(1, 8, 8), (5, 24, 8), (16, 32, 16), (16, 32, 32),
+                                           (3, 96, 96), (2, 256, 64), (2, 256, 256), (1, 512, 128),
+                                           (1, 512, 512)])
+@pytest.mark.parametrize("mode", ["fp32", "mixed", "fp64"])
+def test_sums_are_as_close_as_in_64_bits(probe, mode, ncta, nthr, seg, power):
+    """Thread sums of 44 bits whose totals fit 53 bits: FP64 additions give the
+    exact sum in every order, and so must the reduction.  With a power, 28 bits
+    times 2^99, in all warps or every other one: no thread sum exceeds FP32's
+    range, but the partials of a CTA do."""
+    n = ncta * nthr
+    rng = np.random.default_rng(nthr + seg)
+    v = rng.integers(2 ** 43, 2 ** 44, n)
+    if power == (0, 99):
+        big = (np.arange(n) // 32) % 2 == 1
+        if not big.any():
+            pytest.skip("one warp")
+        v, e = np.where(big, v >> 16, 0), np.where(big, 99, 0)
+    else:
+        v, e = (v if power == 0 else v >> 16), np.full(n, power)
+    if mode == "fp64":
+        e = np.zeros(n, int)
+    v = v * np.where(rng.random(n) < 0.25, -1, 1)
+    hi = v.astype(np.float32)
+    lo = (v - hi.astype(np.int64)).astype(np.float64)
+    exact = sum(int(a) << int(b) for a, b in zip(v, e))
+    assert abs(exact) < 2 ** (53 + int(e.max()))
+    total = np.abs(np.ldexp(v.astype(np.float64), e)).sum()
+    dev = lambda a: torch.from_numpy(np.ldexp(a.astype(np.float64), e)).cuda()   # noqa: E731
+    h, l = dev(hi), dev(lo)
+    assert float(h.abs().max()) < 3.4e38
+    assert power == 0 or mode == "fp64" or n < 64 or total > 3.4e38
+    partial = torch.zeros(n // seg + 32, dtype=torch.float64, device="cuda")
+    state = torch.zeros(probe.probe_state_bytes(), dtype=torch.uint8, device="cuda")
+    for _ in range(2):   # the second run finds the ticket reset
+        assert probe.probe_reduce(TYPES[mode], ncta, nthr, seg, h.data_ptr(), l.data_ptr(),
+                                  partial.data_ptr(), state.data_ptr(),
+                                  torch.cuda.current_stream().cuda_stream) == 0
+        o = probe.probe_bb_offset()
+        bb = state.cpu()[o:o + 8].view(torch.float64).item()
+        assert bb == float(exact)
