@@ -448,9 +448,9 @@ __device__ __forceinline__ void sink_op(const InstDesc<T>& I, const Opnd& o, con
   } else if constexpr (OP == OP_B) {
     a0 = m0 ? -a0 : (T)0;
     a1 = m1 ? -a1 : (T)0;
-    stc_act(I.r, q, a0, a1);
-    if (I.b) stc_act(I.b, q, a0, a1);
-    if (I.r32) stc_act(I.r32, q, a0, a1);
+    stc(I.r, q, a0, a1);
+    if (I.b) stc(I.b, q, a0, a1);
+    if (I.r32) stc(I.r32, q, a0, a1);
     acc.add_prod(a0, a0);
     acc.add_prod(a1, a1);
   } else if constexpr (OP == OP_RES) {
@@ -612,7 +612,7 @@ __device__ __forceinline__ void sink_rows(const InstDesc<T>& I, const uint2* mws
     for (int c = 0; c < CH; ++c)
 #pragma unroll
       for (int v = 0; v < V; ++v)
-        if (C) o[c][v].ok = o[c][v].ok && (OP == OP_B ? o[c][v].q.act : o[c][v].q.any());
+        if (C) o[c][v].ok = o[c][v].ok && o[c][v].q.any();
     T x[CH][V][2];
 #pragma unroll
     for (int c = 0; c < CH; ++c)

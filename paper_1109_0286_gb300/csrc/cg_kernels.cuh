@@ -33,17 +33,24 @@ template <> struct KCfg<double> { static constexpr int kMaxThreads = 512; };
 template <> struct KCfg<df> { static constexpr int kMaxThreads = 512; };
 
 // Masked flags and CG-vector index of the pixel pair (pix, pix+1), pix even,
-// from the pair's mask word.  The CG vectors hold 32 values for every mask word
-// with a masked pixel, zero on its observed pixels, so a pair is one aligned
-// vector access at the word's offset plus the pair's place in the word.
-// (One value per masked pixel packed the vectors more tightly, but took a
-// popcount and two predicated 4-byte accesses per pair and vector.)
+// from the pair's mask word.  The CG vectors hold two values for every pair with
+// a masked pixel, zero on an observed one, so a pair is one aligned vector
+// access, at the word's offset plus two values for every such pair below it in
+// the word.  (32 values for every word with a masked pixel save the popcount,
+// but make the vectors of scattered single pixels up to 32 times as long: 5% of
+// 2048^2 x 2, FP32, plan 298 -> 166 MB, PCG 28.2 -> 25.2 ms; band-and-disc masks
+// of 256^2 to 2048^2 0 to 2% faster with them, 8 x 4096^2 the same.)
 struct PairIdx {
   bool m0, m1;   // pixel masked (to fill)
-  bool act;      // the word has a masked pixel: the vectors hold the pair
-  int i;         // index of the pair's first value (valid where act)
+  int i;         // index of the pair's first value (valid where any())
   __device__ __forceinline__ bool any() const { return m0 || m1; }
 };
+
+// Bit 2k is set where pair k of a mask word has a masked pixel.
+__device__ __forceinline__ uint32_t masked_pairs(uint32_t observed) {
+  const uint32_t m = ~observed;
+  return (m | (m >> 1)) & 0x55555555u;
+}
 
 __device__ __forceinline__ PairIdx pair_from_word(uint2 w, int pix) {
   const int b = pix & 31;
@@ -51,8 +58,7 @@ __device__ __forceinline__ PairIdx pair_from_word(uint2 w, int pix) {
   PairIdx q;
   q.m0 = t & 1u;
   q.m1 = t & 2u;
-  q.act = ~w.x != 0u;
-  q.i = (int)w.y + b;
+  q.i = (int)w.y + 2 * __popc(masked_pairs(w.x) & ((1u << b) - 1u));
   return q;
 }
 
@@ -74,7 +80,7 @@ __device__ __forceinline__ void observed_at(const uint2* mwr, int j, bool& o0, b
 
 // CG-vector loads / stores of a pixel pair (nothing for a pair without a
 // masked pixel, whose values are zero).  stc expects zeros on observed
-// pixels; stc_act also writes the zeros of an active word's other pairs.
+// pixels.
 template <typename T, typename S>
 __device__ __forceinline__ void ldc(const S* v, const PairIdx& q, T& a0, T& a1) {
   a0 = (T)0;
@@ -90,14 +96,10 @@ template <typename T, typename S>
 __device__ __forceinline__ void stc(S* v, const PairIdx& q, T a0, T a1) {
   if (q.any()) st_pair(v + q.i, (S)a0, (S)a1);
 }
-template <typename T, typename S>
-__device__ __forceinline__ void stc_act(S* v, const PairIdx& q, T a0, T a1) {
-  if (q.act) st_pair(v + q.i, (S)a0, (S)a1);
-}
 
 // The CG-vector elements of a CTA's rows form one contiguous range [c0, c1)
-// (the words with masked pixels in row-major order): its first word's offset,
-// and the last word's offset plus its 32 values if it has a masked pixel.
+// (the pairs with masked pixels in row-major order): its first word's offset,
+// and the last word's offset plus its values.
 // One thread asks the copy engine to bring the ranges the op will read into
 // L2, so that the per-pixel-pair gathers later in the pass hit L2 instead of
 // waiting on HBM one chunk after another.
@@ -105,7 +107,7 @@ template <typename T>
 __device__ __forceinline__ void prefetch_compact(const InstDesc<T>& I, int op, const uint2* mws,
                                                  int nwords) {
   const uint2 w0 = mws[0], w1 = mws[nwords - 1];
-  const long long c0 = w0.y, c1 = (long long)w1.y + (~w1.x ? 32 : 0);
+  const long long c0 = w0.y, c1 = (long long)w1.y + 2 * __popc(masked_pairs(w1.x));
   switch (op) {
     case OP_R_UPD:
       prefetch_l2(I.r, c0, c1);
@@ -252,9 +254,9 @@ __device__ __forceinline__ void sink_fill(const InstDesc<T>& I, const uint2* mwr
       const int j = tid + (h + e) * TT;
       const bool m0 = q[e].m0, m1 = q[e].m1;   // masked = not observed
       // CG-vector ops: nothing to store or add (exactly) for a pair without a
-      // masked pixel (the right-hand side also sets the zeros of its words)
+      // masked pixel
       constexpr bool C = OP == OP_Q || OP == OP_Z || OP == OP_B || OP == OP_RES || OP == OP_KSEL;
-      if (C && !(OP == OP_B ? q[e].act : q[e].any())) continue;
+      if (C && !q[e].any()) continue;
       T a0 = v[h + e].r, a1 = v[h + e].i;
       if constexpr (OP == OP_Q || OP == OP_Z) {
         a0 = m0 ? a0 : (T)0;
@@ -265,9 +267,9 @@ __device__ __forceinline__ void sink_fill(const InstDesc<T>& I, const uint2* mwr
       } else if constexpr (OP == OP_B) {
         a0 = m0 ? -a0 : (T)0;
         a1 = m1 ? -a1 : (T)0;
-        stc_act(I.r, q[e], a0, a1);
-        if (I.b) stc_act(I.b, q[e], a0, a1);
-        if (I.r32) stc_act(I.r32, q[e], a0, a1);
+        stc(I.r, q[e], a0, a1);
+        if (I.b) stc(I.b, q[e], a0, a1);
+        if (I.r32) stc(I.r32, q[e], a0, a1);
         acc.add_prod(a0, a0);
         acc.add_prod(a1, a1);
       } else if constexpr (OP == OP_RES) {
@@ -875,9 +877,9 @@ k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
           ld_map_pair<T>(I.gx + pix, g0, g1);
           g0 = q.m0 ? g0 : (T)0;
           g1 = q.m1 ? g1 : (T)0;
-          stc_act(I.r, q, g0, g1);
-          stc_act(I.b, q, g0, g1);
-          if (I.r32) stc_act(I.r32, q, g0, g1);
+          stc(I.r, q, g0, g1);
+          stc(I.b, q, g0, g1);
+          if (I.r32) stc(I.r32, q, g0, g1);
           acc.add_prod(g0, g0);
           acc.add_prod(g1, g1);
           break;

@@ -2,17 +2,17 @@
 //
 // Layout on the device, per realization ("instance"):
 //   * full maps (d, y, w, out, gx): row-major ny x nx;
-//   * CG vectors (r, p, q, z, u, b and the mixed-mode r32 / dlt): COMPACT, 32
-//     values for every mask word with a masked pixel, in row-major order of
-//     the words, zero on the word's observed pixels (the masked system of
-//     Sect. 2.4 lives on M only; the vectors are zero on U);
+//   * CG vectors (r, p, q, z, u, b and the mixed-mode r32 / dlt): COMPACT, two
+//     values for every pixel pair (2j, 2j + 1) with a masked pixel, in row-major
+//     order, zero on its observed pixel (the masked system of Sect. 2.4 lives
+//     on M only; the vectors are zero on U);
 //   * half spectrum "spec": transposed, (nx/2+1) rows of ny complex values,
 //     spec[kx * ny + y]; the column pass runs along contiguous rows;
 //   * spectral tables [kx][ky] (same transposed layout), real, with the
 //     1/n of the inverse DFT folded in;
 //   * mask words: for each 32 pixels, the observed bits (1 = constraint, also
-//     beyond the last pixel) and the index of the word's values in the CG
-//     vectors (the values of all words before it).
+//     beyond the last pixel) and the index of the word's first value in the CG
+//     vectors (the number of values of all words before it).
 #pragma once
 #include <cstdint>
 
@@ -110,7 +110,7 @@ struct InstDesc {
   T* speck;                // spectra of that solver's kernels that run together, or null
   const uint8_t* cls;      // kernel class of every pixel (Sect. 6.3 solver), or null
   const double* noise;     // tables of the white-noise source
-  long long nvec;          // CG-vector length: 32 per word with a masked pixel
+  long long nvec;          // CG-vector length: 2 per pixel pair with a masked pixel
   unsigned long long seed;
 };
 

@@ -11,6 +11,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <bitset>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -196,7 +197,7 @@ struct fill_plan {
   cudaEvent_t lane_join[kMaxLanes] = {};
   cudaEvent_t lane_fork = nullptr, lane_fork_cap = nullptr;
   uint2* mw = nullptr;           // mask words: observed bits, CG-vector offset
-  long long nvec = 0;            // CG-vector length: 32 per mask word with a masked pixel
+  long long nvec = 0;            // CG-vector length: 2 per pixel pair with a masked pixel
   long long nv = 0;              // CG-vector stride per instance (>= nvec)
   double* noise = nullptr;       // device: tables of the white-noise source
   std::vector<double> P_half;    // host copy of the spectrum
@@ -1586,7 +1587,7 @@ fill_status fill_init(fill_plan** out, int ny, int nx, const double* P_half,
   long long nmasked = 0, nvec = 0;
   std::vector<uint2> words((npix + 31) / 32, make_uint2(0u, 0u));
   for (long long w = 0; w < (long long)words.size(); ++w) {
-    words[w].y = (unsigned int)nvec;   // index of the word's values in the CG vectors
+    words[w].y = (unsigned int)nvec;   // index of the word's first value in the CG vectors
     for (int b = 0; b < 32; ++b) {
       const long long i = w * 32 + b;
       if (i < npix && observed[i] > 1) return FILL_EINVAL;
@@ -1595,7 +1596,8 @@ fill_status fill_init(fill_plan** out, int ny, int nx, const double* P_half,
       else
         ++nmasked;
     }
-    if (~words[w].x) nvec += 32;
+    const uint32_t m = ~words[w].x;
+    nvec += 2 * (long long)std::bitset<32>((m | (m >> 1)) & 0x55555555u).count();
   }
   fill_plan* p = new (std::nothrow) fill_plan();
   if (!p) return FILL_ENOMEM;
