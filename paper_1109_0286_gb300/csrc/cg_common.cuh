@@ -322,6 +322,7 @@ __device__ __forceinline__ Sum3 operator+(Sum3 a, Sum3 b) {
 
 template <>
 struct Acc<float> {
+  using total_t = Sum3;
   float hi = 0.f, lo = 0.f;
   __device__ __forceinline__ void add_prod(float a, float b) {
     float p = a * b;
@@ -337,6 +338,7 @@ struct Acc<float> {
 
 template <>
 struct Acc<df> {
+  using total_t = Sum3;
   df s = df(0.f, 0.f);
   __device__ __forceinline__ void add_prod(df a, df b) { s = s + a * b; }
   __device__ __forceinline__ Sum3 total() const { return {s.hi, s.lo, 0.f}; }
@@ -344,6 +346,7 @@ struct Acc<df> {
 
 template <>
 struct Acc<double> {
+  using total_t = double;
   double s = 0.0;
   __device__ __forceinline__ void add_prod(double a, double b) { s = fma(a, b, s); }
   __device__ __forceinline__ double total() const { return s; }
@@ -366,6 +369,9 @@ __device__ __forceinline__ double sum_value(double v) { return v; }
 // CTA (at most 1024 threads); such sums go through FP64.
 __device__ __forceinline__ bool sum_large(Sum3 v) { return !(fabsf(v.h) < 1e34f); }
 __device__ __forceinline__ bool sum_large(double) { return false; }
+// Beyond FP32 altogether.
+__device__ __forceinline__ bool sum_lost(Sum3 v) { return !(fabsf(v.h) < 3.4e38f); }
+__device__ __forceinline__ bool sum_lost(double) { return false; }
 
 // Sum over the segments of `len` consecutive lanes of a warp (len <= 32, any
 // value; nl lanes present): the first lane of each segment gets its segment's
@@ -532,30 +538,87 @@ __device__ __forceinline__ T cg_beta(const CgState* st) { return (T)st->beta; }
 template <>
 __device__ __forceinline__ float cg_beta<float>(const CgState* st) { return st->beta_f; }
 
+// Partial sums of a CTA: one of every `seg` consecutive threads' v (seg divides
+// the CTA; fewer than 32 threads or whole warps).  A segment of several warps
+// is added warp on warp by its first one, lane by lane, then across the lanes:
+// the other warps only store their values (buf: one per thread of the CTA, free to
+// write), where shuffles in every warp took five additions of each.  K: the
+// segment's warps hold K shares of what B = seg / (32 K) warps would hold, share
+// by share; the shares are added first.
+template <typename V>
+__device__ __forceinline__ void segment_partials(V v, V* buf, double* out, int seg, int K = 1) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (seg <= 32) {
+    const int nl = min(32, (int)blockDim.x - (wid << 5));   // lanes of this warp
+    const unsigned mask = nl == 32 ? 0xffffffffu : ((1u << nl) - 1u);
+    const V w = segment_sum(v, mask, lane, nl, seg);
+    double s = sum_value(w);
+    if (__any_sync(mask, sum_large(w))) {   // out of the FP32 range: in FP64
+      const double d = segment_sum(sum_value(v), mask, lane, nl, seg);
+      if (sum_large(w)) s = d;
+    }
+    if (lane % seg == 0) out[tid / seg] = s;
+    return;
+  }
+  const int wps = seg >> 5, sg = wid / wps;
+  if (wid != sg * wps) buf[tid] = v;
+  __syncthreads();
+  if (wid != sg * wps) return;
+  const V* b = buf + tid;
+  const int B = wps / K;
+  auto warp = [&](int w) {
+    V x = w ? b[32 * w] : v;
+    for (int k = 1; k < K; ++k) x = x + b[32 * (k * B + w)];
+    return x;
+  };
+  V t = warp(0);
+  int w = 1;
+  for (; w + 4 <= B; w += 4) t = t + ((warp(w) + warp(w + 1)) + (warp(w + 2) + warp(w + 3)));
+  for (; w < B; ++w) t = t + warp(w);
+  t = segment_sum(t, ~0u, lane, 32, 32);
+  double s = sum_value(t);
+  if (__any_sync(~0u, lane == 0 && sum_large(t))) {   // out of the FP32 range: in FP64
+    s = 0.0;
+    for (w = 0; w < B; ++w) {
+      const V x = warp(w);
+      double d = sum_value(x);
+      if (sum_lost(x)) {
+        d = w ? sum_value(b[32 * w]) : sum_value(v);
+        for (int k = 1; k < K; ++k) d += sum_value(b[32 * (k * B + w)]);
+      }
+      s += d;
+    }
+    s = segment_sum(s, ~0u, lane, 32, 32);
+  }
+  if (lane == 0) out[sg] = s;
+}
+
 // Reduction of a pass: every `seg` consecutive threads of a CTA give one
-// partial sum (seg divides the CTA; fewer than 32 threads or whole warps), and
-// the last CTA of the instance adds all partials and runs the scalar update.
-// Called by all threads of the CTA.
+// partial sum, and the last CTA of the instance adds all partials and runs the
+// scalar update.  Called by all threads of the CTA.  partials(out) writes the
+// CTA's nseg partial sums (before the barrier that follows it).
 //
 // Every order is fixed and, for a given seg, independent of how many segments
-// a CTA holds, so results are reproducible and do not depend on the CTA shape.
+// a CTA holds, so results are reproducible and the same for every CTA height of
+// at least kRedRows rows (cg_kernels.cuh).
 // What bounds it is the FP64 pipe (64 cycles per dependent instruction): the
 // sums inside a CTA are carried in three FP32 parts (Sum3: no further from
 // the exact sum than FP64 additions; in two parts, 2^-47 per addition, sums
-// with cancellation came out 1.8 times as far; the third part costs 1% of an
-// iteration, 679 -> 686 ms a call at 8 x 4096^2), only a segment's total becomes
-// a double, and the last CTA adds the partials in FP64 on 32 lanes in parallel.  Measured against shuffles and sums in
-// FP64 with one thread adding the partials (1024 of them at 4096^2, 32 us):
-// 4096^2, one map, sink 104 -> 59 us, r-update 124 -> 76 us; an iteration of
-// 1024^2 94.5 -> 84 us; 600 x 7000 x 4, r-update 106 -> 93 us.
-template <typename V>
-__device__ __forceinline__ void grid_reduce(V v, double* sh, double* partial, CgState* st,
-                                            int sop, int ncta, int cta, int seg) {
+// with cancellation came out 1.8 times as far), only a segment's total becomes
+// a double, and the last CTA adds the partials in FP64 on 32 lanes in parallel.
+// Measured against shuffles and sums in FP64 with one thread adding the partials
+// (1024 of them at 4096^2, 32 us): 4096^2, one map, sink 104 -> 59 us, r-update
+// 124 -> 76 us; an iteration of 1024^2 94.5 -> 84 us; 600 x 7000 x 4, r-update
+// 106 -> 93 us.  Two parts and three with shuffles in every warp, three with the
+// warps added first (segment_partials): 8 x 4096^2 FP32 679, 686 and 677 ms a call,
+// 16 x 1024^2 28.2, 28.8 and 28.7, one map 6.0, 6.1 and 6.1.
+template <typename F>
+__device__ __forceinline__ void grid_reduce(double* sh, double* partial, CgState* st, int sop,
+                                            int ncta, int cta, int nseg, F partials) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int nthr = blockDim.x, nseg = nthr / seg, nw = (nthr + 31) >> 5;
+  const int nthr = blockDim.x;
   const int nl = min(32, nthr - (wid << 5));   // lanes of this warp
   const unsigned mask = nl == 32 ? 0xffffffffu : ((1u << nl) - 1u);
-  double* out = partial + (long long)cta * nseg;
   __shared__ bool last;
   __shared__ alignas(8) unsigned char shst[sizeof(CgState)];   // for scalar_update
   static_assert(sizeof(CgState) % 8 == 0, "copied in 8-byte words");
@@ -564,37 +627,7 @@ __device__ __forceinline__ void grid_reduce(V v, double* sh, double* partial, Cg
     for (int i = lane; i < (int)(sizeof(CgState) / 8); i += nl)
       reinterpret_cast<unsigned long long*>(shst)[i] = ld_l2(src + i);
   }
-  if (seg <= 32) {
-    V w = segment_sum(v, mask, lane, nl, seg);
-    double s = sum_value(w);
-    if (__any_sync(mask, sum_large(w))) s = segment_sum(sum_value(v), mask, lane, nl, seg);
-    if (lane % seg == 0) out[tid / seg] = s;
-  } else {
-    __shared__ V shv[32];
-    __shared__ int large;
-    if (tid == 0) large = 0;
-    V w = segment_sum(v, mask, lane, nl, 32);
-    __syncthreads();   // (sh may still be read by the previous use)
-    if (lane == 0) {
-      shv[wid] = w;
-      if (sum_large(w)) large = 1;
-    }
-    __syncthreads();
-    const int wps = seg >> 5;   // warps per segment
-    if (large) {                // uniform over the CTA; out of the FP32 range: in FP64
-      const double d = segment_sum(sum_value(v), mask, lane, nl, 32);
-      __syncthreads();
-      if (lane == 0) sh[wid] = d;
-      __syncthreads();
-      if (wid == 0) {
-        const double t = segment_sum(lane < nw ? sh[lane] : 0.0, mask, lane, min(nw, nl), wps);
-        if (lane < nw && lane % wps == 0) out[lane / wps] = t;
-      }
-    } else if (wid == 0) {
-      const V t = segment_sum(lane < nw ? shv[lane] : V{}, mask, lane, min(nw, nl), wps);
-      if (lane < nw && lane % wps == 0) out[lane / wps] = sum_value(t);
-    }
-  }
+  partials(partial + (long long)cta * nseg);
   __syncthreads();
   if (tid == 0) {
     // releases the CTA's partials (ordered before it by the barrier); the last

@@ -663,18 +663,24 @@ __device__ __forceinline__ void mid_rows(const InstDesc<T>& I, const uint2* mws,
 
 }  // namespace gen
 
-// Shared memory of the values of a CTA's rows (the mask words follow).
+// Shared memory of the values of a CTA's rows, and with the mask words.
 template <typename T>
 __host__ __device__ __forceinline__ size_t gen_row_main(int L, int rows) {
   return (size_t(rows) * L * sizeof(cx<T>) + 15) & ~size_t(15);
+}
+template <typename T>
+__host__ __device__ __forceinline__ size_t gen_row_smem(int L, int rows) {
+  return gen_row_main<T>(L, rows) + size_t(rows) * gen::row_words(2 * L) * sizeof(uint2);
 }
 
 // ----------------------------------------------------------------- row pass
 // CTA = a.rows consecutive grid rows in groups of V (one group per g.nt
 // threads; blockIdx.y is the instance), rows at or beyond ny (odd ny) idle.
 // Shared memory: L complex values per row, interleaved [position][V] within a
-// group, then the rows' mask words.
-template <typename T, int V, bool IN_SPEC, bool OUT_SPEC, bool AUX = false>
+// group, then the rows' mask words, then (groups of several warps, reducing
+// passes) a value per thread for the sums.
+// MULTI: groups of nt_base threads form the sums that wide ones would.
+template <typename T, int V, bool IN_SPEC, bool OUT_SPEC, bool AUX = false, bool MULTI = false>
 __global__ void __launch_bounds__(kGenThreads, gen_minb<T>())
 k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* __restrict__ wl,
           const T* __restrict__ wx) {
@@ -688,7 +694,19 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
   cx<T>* Z = reinterpret_cast<cx<T>*>(smem_raw) + grp * L * V;
   uint2* mws = reinterpret_cast<uint2*>(smem_raw + gen_row_main<T>(L, a.rows)) +
                grp * V * gen::row_words(a.nx);
+  // Sums are taken over g.shares shares, of the threads t, t + nt_base and so on of
+  // wide groups, so they do not depend on nt: groups of nt_base threads go
+  // through the m = g.shares shares one after another.
+  using V3 = typename Acc<T>::total_t;
+  const int m = MULTI ? g.shares : 1;
   Acc<T> acc;
+  V3 tot{};
+  auto end_share = [&](int s) {
+    if constexpr (MULTI) {
+      tot = s ? tot + acc.total() : acc.total();
+      acc = Acc<T>();
+    }
+  };
 
   const int pix0 = y0 * a.nx;
   constexpr bool XI = AUX && !IN_SPEC, KS = AUX && IN_SPEC;   // (as in k_row)
@@ -708,28 +726,32 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
     __syncthreads();
     gen::dit<T, V>(Z, g, wl, t, g.nst);   // Z[j] = x[2j] + i x[2j+1] (scaled)
 #define CGF_SINK(OPC, PARAM) \
-  gen::sink_rows<T, OPC, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt, acc, PARAM)
+  gen::sink_rows<T, OPC, V>(I, mws, pix0, a.nx, nv, Z, L, t + s * nt, m * nt, acc, PARAM)
     if constexpr (OUT_SPEC) {
       if (a.op == OP_Y_W)
         gen::mid_rows<T, OP_Y_W, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt);
       else
         gen::mid_rows<T, OP_MASK, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt);
     } else if constexpr (KS) {
+      const int s = 0;
       CGF_SINK(OP_KSEL, a.param + blockIdx.z);
     } else {
-      switch (a.op) {
-        case OP_Q: CGF_SINK(OP_Q, 0); break;
-        case OP_Z: CGF_SINK(OP_Z, 0); break;
-        case OP_B: CGF_SINK(OP_B, 0); break;
-        case OP_RES: CGF_SINK(OP_RES, 0); break;
-        case OP_GRAD: CGF_SINK(OP_GRAD, 0); break;
-        case OP_RELAX: CGF_SINK(OP_RELAX, 0); break;
-        case OP_STORE_Y: CGF_SINK(OP_STORE_Y, 0); break;
-        case OP_STORE_Y_MASK: CGF_SINK(OP_STORE_Y_MASK, 0); break;
-        case OP_STORE_OUT: CGF_SINK(OP_STORE_OUT, 0); break;
-        case OP_STORE_OUT_MASK: CGF_SINK(OP_STORE_OUT_MASK, 0); break;
-        default: break;
-      }
+      for (int s = 0; s < m; ++s) {
+        switch (a.op) {
+          case OP_Q: CGF_SINK(OP_Q, 0); break;
+          case OP_Z: CGF_SINK(OP_Z, 0); break;
+          case OP_B: CGF_SINK(OP_B, 0); break;
+          case OP_RES: CGF_SINK(OP_RES, 0); break;
+          case OP_GRAD: CGF_SINK(OP_GRAD, 0); break;
+          case OP_RELAX: CGF_SINK(OP_RELAX, 0); break;
+          case OP_STORE_Y: CGF_SINK(OP_STORE_Y, 0); break;
+          case OP_STORE_Y_MASK: CGF_SINK(OP_STORE_Y_MASK, 0); break;
+          case OP_STORE_OUT: CGF_SINK(OP_STORE_OUT, 0); break;
+          case OP_STORE_OUT_MASK: CGF_SINK(OP_STORE_OUT_MASK, 0); break;
+          default: break;
+        }
+        end_share(s);
+        }
     }
 #undef CGF_SINK
   } else if constexpr (XI) {
@@ -746,12 +768,25 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
     __syncthreads();   // mask words
     const T alpha = a.op == OP_R_UPD ? cg_alpha<T>(I.st) : (T)0;
     const T beta = a.op == OP_P_UPD_Z || a.op == OP_P_UPD_R ? cg_beta<T>(I.st) : (T)0;
-#define CGF_SRC(OPC) gen::src_rows<T, OPC, V>(I, mws, pix0, a.nx, nv, Z, L, t, nt, alpha, beta, acc)
+#define CGF_SRC(OPC) \
+  gen::src_rows<T, OPC, V>(I, mws, pix0, a.nx, nv, Z, L, t + s * nt, m * nt, alpha, beta, acc)
+    int s = 0;
     switch (a.op) {
-      case OP_R_UPD: CGF_SRC(OP_R_UPD); break;
+      case OP_R_UPD:
+        for (; s < m; ++s) {
+          CGF_SRC(OP_R_UPD);
+          end_share(s);
+        }
+        break;
+      case OP_LOAD_R:
+        for (; s < m; ++s) {
+          CGF_SRC(OP_LOAD_R);
+          end_share(s);
+        }
+        break;
+      // (the others sum nothing: m = 1)
       case OP_P_UPD_Z: CGF_SRC(OP_P_UPD_Z); break;
       case OP_P_UPD_R: CGF_SRC(OP_P_UPD_R); break;
-      case OP_LOAD_R: CGF_SRC(OP_LOAD_R); break;
       case OP_LOAD_U: CGF_SRC(OP_LOAD_U); break;
       case OP_LOAD_Y: CGF_SRC(OP_LOAD_Y); break;
       case OP_LOAD_W: CGF_SRC(OP_LOAD_W); break;
@@ -777,7 +812,14 @@ k_row_gen(const InstDesc<T>* __restrict__ insts, RowArgs a, GenLen g, const T* _
   if constexpr (!OUT_SPEC) pdl_trigger();
   if constexpr (!AUX) {
     if (a.sop != SC_NONE)
-      grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, nt);
+      grid_reduce(red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, (int)blockDim.x / nt,
+                  [&](double* out) {
+                    V3* const buf = reinterpret_cast<V3*>(smem_raw + gen_row_smem<T>(L, a.rows));
+                    if constexpr (MULTI)
+                      segment_partials(tot, buf, out, nt);
+                    else
+                      segment_partials(acc.total(), buf, out, nt, g.shares);
+                  });
   }
 }
 
@@ -917,9 +959,7 @@ template <typename T>
 size_t GenLaunch<T>::row_main(int L, int rows) { return gen_row_main<T>(L, rows); }
 
 template <typename T>
-size_t GenLaunch<T>::row_smem(int L, int rows) {
-  return gen_row_main<T>(L, rows) + size_t(rows) * gen::row_words(2 * L) * sizeof(uint2);
-}
+size_t GenLaunch<T>::row_smem(int L, int rows) { return gen_row_smem<T>(L, rows); }
 
 template <typename T>
 size_t GenLaunch<T>::col_smem(int ny, int ffts) {
@@ -936,12 +976,15 @@ cudaError_t GenLaunch<T>::row(bool in_spec, bool out_spec, const InstDesc<T>* d,
   constexpr int V = gen_vrow<T>();
   const dim3 grid((a.ny + a.rows - 1) / a.rows, ninst, a.nz > 0 ? a.nz : 1);
   const dim3 block(a.rows / V * g.nt);
-  const size_t sm = row_smem(g.n, a.rows);
-  const Launcher l{grid, block, sm, s, a.pdl != 0};
+  const size_t sums = a.sop != SC_NONE && g.nt > 32 ? block.x * sizeof(typename Acc<T>::total_t) : 0;
+  const Launcher l{grid, block, row_smem(g.n, a.rows) + sums, s, a.pdl != 0};
+  const bool multi = a.sop != SC_NONE && g.nt == g.nt_base && g.shares > 1;
   if (in_spec && out_spec) return l(k_row_gen<T, V, true, true>, d, a, g, wl, wx);
   if (in_spec && a.op == OP_KSEL) return l(k_row_gen<T, V, true, false, true>, d, a, g, wl, wx);
+  if (in_spec && multi) return l(k_row_gen<T, V, true, false, false, true>, d, a, g, wl, wx);
   if (in_spec) return l(k_row_gen<T, V, true, false>, d, a, g, wl, wx);
   if (a.op == OP_XI) return l(k_row_gen<T, V, false, true, true>, d, a, g, wl, wx);
+  if (multi) return l(k_row_gen<T, V, false, true, false, true>, d, a, g, wl, wx);
   return l(k_row_gen<T, V, false, true>, d, a, g, wl, wx);
 }
 
@@ -963,6 +1006,8 @@ cudaError_t GenLaunch<T>::prepare() {
   cudaError_t e = detail::allow_smem(k_row_gen<T, VR, true, true>);
   if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, true, false>);
   if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, true, false, true>);
+  if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, true, false, false, true>);
+  if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, false, true, false, true>);
   if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, false, true>);
   if (e == cudaSuccess) e = detail::allow_smem(k_row_gen<T, VR, false, true, true>);
   if (e == cudaSuccess) e = detail::allow_smem(k_col_gen<T, V>);

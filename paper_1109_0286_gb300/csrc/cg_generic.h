@@ -45,8 +45,10 @@ constexpr int kGenMaxLen = 4096;   // nx / 2 and ny at most 4096
 struct GenLen {
   int n;
   int nst;
-  int nt;       // threads per group (gen_threads)
-  int nt_base;  // nt before the few-transform rule (gen_threads): admits CTA shapes
+  int nt;       // threads per group (gen_threads) of a launch of few transforms
+  int nt_base;  // threads per group of a launch that fills the chip; a divisor of nt
+  int shares;   // of a row launch: the sums are taken over this many shares of nt_base
+                // threads (nt / nt_base of the wide groups, whatever nt is)
   int code;     // radix schedule (gen_factor)
   int radix[kGenMaxStages];
   // Stage s < nst - 1: twiddles W_{n_s}^{q j} (j < h_s, q = 1 .. R_s - 1) at

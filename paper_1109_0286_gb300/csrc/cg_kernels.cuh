@@ -23,8 +23,9 @@ template <int E> CGF_HD constexpr int src_chunk() { return 4; }
 template <int E> CGF_HD constexpr int src_chunk_wide() { return E == 16 ? 2 : 4; }
 template <int E> CGF_HD constexpr int sink_chunk() { return 4; }
 
-// Rows per partial sum of a row pass (fewer if the CTA holds fewer), so that
-// the sums do not depend on the CTA height.
+// Rows per partial sum of a row pass, so that the sums do not depend on the CTA
+// height.  A CTA of fewer rows (two by default in FP64 on rows of 1024 pixels
+// and more) sums what it holds: there the partials follow the height.
 constexpr int kRedRows = 4;
 
 template <typename T> struct KCfg;
@@ -570,8 +571,13 @@ k_row(const InstDesc<T>* __restrict__ insts, RowArgs a, const T* __restrict__ tw
   if constexpr (!OUT_SPEC) pdl_trigger();
   if constexpr (!AUX) {
     if (a.sop != SC_NONE)
-      grid_reduce(acc.total(), red, I.partial, st, a.sop, gridDim.x, blockIdx.x,
-                  min(rows, kRedRows) * TT);
+      grid_reduce(red, I.partial, st, a.sop, gridDim.x, blockIdx.x,
+                  rows > kRedRows ? rows / kRedRows : 1, [&](double* out) {
+                    using V = typename Acc<T>::total_t;
+                    const int seg = min(rows, kRedRows) * TT;
+                    if (seg > 32) __syncthreads();   // the exchange areas have been read
+                    segment_partials(acc.total(), reinterpret_cast<V*>(smem_raw), out, seg);
+                  });
   }
 }
 
@@ -891,7 +897,10 @@ k_vec(const InstDesc<T>* __restrict__ insts, VecArgs a) {
   }
   pdl_trigger();
   if (a.sop != SC_NONE)
-    grid_reduce(acc.total(), red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, blockDim.x);
+    grid_reduce(red, I.partial, I.st, a.sop, gridDim.x, blockIdx.x, 1, [&](double* out) {
+      __shared__ typename Acc<T>::total_t buf[256];
+      segment_partials(acc.total(), buf, out, blockDim.x);
+    });
 }
 
 // ----------------------------------------------------------------- band products

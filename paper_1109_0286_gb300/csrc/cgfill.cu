@@ -403,6 +403,25 @@ int use_pdl(long long npix, int ninst, bool gen) {
   return npix * ninst <= most;
 }
 
+// Whether `groups` groups of nt threads leave a chip that runs tmax threads per
+// SM half empty.
+bool few_groups(long long groups, int nt, double tmax) {
+  return double(groups) * nt <= 0.5 * 152.0 * tmax;
+}
+
+// The row transform as one launch over ninst maps runs it, `rows` rows per CTA:
+// groups of g.nt threads where narrow ones leave the chip half empty and the CTA
+// holds them, else of g.nt_base; the sums are the same (gen_threads).
+template <typename T>
+GenLen gen_row_len(GenLen g, int ny, int ninst, int rows) {
+  constexpr int V = gen_vrow<T>();
+  g.shares = g.nt / g.nt_base;
+  if (!few_groups((long long)((ny + V - 1) / V) * ninst, g.nt_base, double(kGenThreads) * gen_minb<T>()) ||
+      rows / V * g.nt > kGenThreads)
+    g.nt = g.nt_base;
+  return g;
+}
+
 template <typename T>
 Ctx<T> no_pdl(Ctx<T> c) {
   c.pdl = 0;
@@ -432,7 +451,8 @@ cudaError_t row(const Ctx<T>& c, cudaStream_t s, int op, int sop, bool in_spec, 
   ++*c.launches;
   RowArgs a{c.ny, c.nx, c.rows, ilog2(c.rows), op, sop, skip, spec_sel, param, c.pdl, nz};
   if (c.grow)
-    return GenLaunch<T>::row(in_spec, out_spec, c.desc, c.ninst, a, *c.grow, c.gwl, c.gwx, s);
+    return GenLaunch<T>::row(in_spec, out_spec, c.desc, c.ninst, a,
+                             gen_row_len<T>(*c.grow, c.ny, c.ninst, c.rows), c.gwl, c.gwx, s);
   return Launch<T>::row(c.log_l, in_spec, out_spec, c.desc, c.ninst, a, c.tw, s);
 }
 
@@ -1158,19 +1178,22 @@ void gen_tables(const GenLen& g, std::vector<double>& tw, std::vector<unsigned s
 // threads, against the threads an SM runs at the kernels' register counts:
 // kGenThreads x gen_minb).
 //
-// If one map's `count` transforms leave the chip half empty at that width, a
-// pass of a few maps is one wave of CTAs and its time the rounds of a group:
-// then the fewest threads that need the fewest rounds over all stages, among
-// those within 0.8 of the best product, at most `cap`.  The columns stop at
+// If the transforms of a launch leave the chip half empty at that width (nt_base),
+// a pass of a few maps is one wave of CTAs and its time the rounds of a group:
+// then the fewest threads, a multiple of nt_base, that need the fewest rounds over
+// all stages, among those within 0.8 of the best product, at most `cap` (nt; what
+// one map's `count` transforms ask for).  The columns stop at
 // 64 threads: a CTA of wider groups holds fewer columns, and its loads get
 // shorter than a sector (600 x 7000 with 128: column pass 69 -> 88 us).
-// Measured, whole calls to 1e-6, before -> now: 375 x 1050 FP32 one map 11.5
-// -> 7.4 ms, three 13.1 -> 9.2; FP64 38.8 -> 28.8; 600 x 700 four maps 22.6 ->
-// 18.6; the 32 lanes of a 480^2 gradient 31.1 -> 25.9.  With 0.9 in place of 0.8: 9.8,
-// 10.4, 38.8, 18.6, 31.1.  Groups that fill the chip with many maps of such a
-// grid lose up to the 0.8: 16 maps of 600 x 700 25.5 -> 27.5 ms, of 280 x 504
-// 9.9 -> 11.4.  The choice cannot follow the batch: a thread's share of a sum
-// is its share of the row, and a map's sums do not depend on its neighbours.
+// The columns are nt wide in every launch; the rows follow the launch
+// (gen_row_len), their sums taken over the shares of nt threads in any case, so
+// that a map's results do not depend on what it is batched with.  Measured, whole
+// FP32 calls to 1e-6 with narrow and with wide rows: 375 x 1050 one map 10.8 and
+// 7.2 ms, four 13.8 and 10.9; 600 x 700 one map 8.5 and 6.5, four 10.7 and 9.5, 16
+// 24.7 and 25.9; 280 x 504 one map 6.1 and 5.0, 16 11.1 and 12.0, 64 28.7 and 35.7;
+// 480 x 480 64 maps 43.5 and 47.9.  The shares cost the narrow rows 4 to 6% (64
+// maps of 280 x 504 27.1, of 480 x 480 41.8 with sums that follow the launch).
+// 0.9 in place of 0.8: 375 x 1050 9.8 ms.
 void gen_threads(GenLen* g, int V, bool wide, int count, int cap) {
   const double tmax = double(kGenThreads) * (wide ? gen_minb<double>() : gen_minb<float>());
   const size_t bytes = size_t(V) * g->n * (wide ? 16 : 8);
@@ -1195,9 +1218,9 @@ void gen_threads(GenLen* g, int V, bool wide, int count, int cap) {
     }
   }
   g->nt_base = g->nt;
-  if (double((count + V - 1) / V) * g->nt > 0.5 * 152.0 * tmax) return;
+  if (!few_groups((count + V - 1) / V, g->nt_base, tmax)) return;
   int least = 1 << 30;
-  for (int nt = g->nt; nt <= cap; nt += 32) {
+  for (int nt = g->nt_base; nt <= cap; nt += g->nt_base) {
     int rounds = 0;
     for (int s = 0; s < g->nst; ++s) rounds += (g->n / g->radix[s] + nt - 1) / nt;
     if (rounds < least && score_of(nt) >= 0.8 * best) {
@@ -1233,15 +1256,10 @@ bool gen_col_ok(const fill_plan* p, int f, int nt) {
          GenLaunch<T>::col_smem(p->ny, f) <= 200 * 1024;
 }
 
-// A CTA shape asked for by the options or read from a tuning cache: admitted by
-// the width that the stages and the occupancy ask for (GenLen::nt_base), then
-// cut to the groups of nt threads that one CTA holds.
-template <typename T>
-int gen_fit_rows(const fill_plan* p, int r) {
-  if (!gen_row_ok<T>(p, r, p->grow.nt_base)) return r;
-  while (r / gen_vrow<T>() * p->grow.nt > GenLaunch<T>::max_threads()) r /= 2;
-  return r;
-}
+// Column FFTs per CTA asked for by the options or read from a tuning cache:
+// admitted by the width that the stages and the occupancy ask for
+// (GenLen::nt_base), then cut to the groups of nt threads that one CTA holds.
+// (Rows per CTA are admitted in the same way and taken as they are: gen_row_len.)
 template <typename T>
 int gen_fit_ffts(const fill_plan* p, int f) {
   if (!gen_col_ok<T>(p, f, p->gcol.nt_base)) return f;
@@ -1295,7 +1313,7 @@ fill_status gen_upload_maps(fill_plan* p) {
 }
 
 // Mixed-radix schedule and twiddle tables of one precision: rows per CTA
-// and column FFTs per CTA (groups of g.nt threads, within 75 KB of shared
+// and column FFTs per CTA (groups of threads, within 75 KB of shared
 // memory so that three CTAs share an SM, and no more than leaves two CTAs per
 // SM), unless the options fix them; the digit-reversal maps once per plan.
 template <typename T>
@@ -1306,10 +1324,11 @@ fill_status setup_generic(fill_plan* p) {
   const int ctas = 2 * 152;
   const bool user = loop_precision<T>(p);
   if (user && p->o.rows_per_cta > 0) {
-    P.rows = gen_fit_rows<T>(p, p->o.rows_per_cta);
+    P.rows = p->o.rows_per_cta;
   } else {
     P.rows = VR;
-    if (gen_row_ok<T>(p, 2 * VR, p->grow.nt) && GenLaunch<T>::row_smem(p->nx / 2, 2 * VR) <= third &&
+    const int nt = gen_row_len<T>(p->grow, p->ny, p->batch, VR).nt;
+    if (gen_row_ok<T>(p, 2 * VR, nt) && GenLaunch<T>::row_smem(p->nx / 2, 2 * VR) <= third &&
         (long long)p->ny * p->batch >= 2LL * VR * ctas)
       P.rows = 2 * VR;
   }
@@ -1321,7 +1340,8 @@ fill_status setup_generic(fill_plan* p) {
            2 * P.ffts <= 16 && (long long)(p->nx / 2 + 1) * p->batch >= 2LL * P.ffts * ctas)
       P.ffts *= 2;
   }
-  if (!gen_row_ok<T>(p, P.rows, p->grow.nt) || !gen_col_ok<T>(p, P.ffts, p->gcol.nt)) return FILL_EINVAL;
+  if (!gen_row_ok<T>(p, P.rows, p->grow.nt_base) || !gen_col_ok<T>(p, P.ffts, p->gcol.nt))
+    return FILL_EINVAL;
   fill_status fs = gen_upload<T>(p);
   if (fs != FILL_OK) return fs;
   if (!p->grow.rev) {
@@ -2599,7 +2619,7 @@ fill_status tune_gen_t(fill_plan* p, const char* path) {
       fill_status fs = apply_gen_code(p, true, code);
       if (fs != FILL_OK) return fs;
       for (int r = gen_vrow<T>(); r <= 4 * gen_vrow<T>(); r *= 2) {
-        if (!gen_row_ok<T>(p, r, p->grow.nt)) continue;
+        if (!gen_row_ok<T>(p, r, p->grow.nt_base)) continue;
         Ctx<T> c = ctx<T>(p);
         c.rows = r;
         float ms = 0.f;
@@ -2630,9 +2650,9 @@ fill_status tune_gen_t(fill_plan* p, const char* path) {
     }
     cache_store_gen(path, pr, p->ny, p->nx, p->batch, rows, ffts, rcode, ccode);
   }
-  rows = gen_fit_rows<T>(p, rows);
   ffts = gen_fit_ffts<T>(p, ffts);
-  if (!gen_row_ok<T>(p, rows, p->grow.nt) || !gen_col_ok<T>(p, ffts, p->gcol.nt)) return FILL_EINVAL;
+  if (!gen_row_ok<T>(p, rows, p->grow.nt_base) || !gen_col_ok<T>(p, ffts, p->gcol.nt))
+    return FILL_EINVAL;
   fill_status fs = apply_gen_code(p, true, rcode);
   if (fs == FILL_OK) fs = apply_gen_code(p, false, ccode);
   if (fs != FILL_OK) return fs;

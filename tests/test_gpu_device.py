@@ -21,7 +21,7 @@ def probe(tmp_path_factory):
     src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "device_probe.cu")
     subprocess.run([_build._nvcc(), *_build.ARCH, *_build.FLAGS, "-shared", "-o", so, src], check=True)
     lib = ctypes.CDLL(so)
-    lib.probe_reduce.argtypes = [ctypes.c_int] * 4 + [ctypes.c_void_p] * 5
+    lib.probe_reduce.argtypes = [ctypes.c_int] * 5 + [ctypes.c_void_p] * 5
     return lib
 
 
@@ -29,11 +29,12 @@ TYPES = {"fp32": 0, "mixed": 1, "fp64": 2}
 
 
 @pytest.mark.parametrize("power", [0, 99, (0, 99)])
-@pytest.mark.parametrize("ncta,nthr,seg", [(1, 8, 8), (5, 24, 8), (16, 32, 16), (16, 32, 32),
-                                           (3, 96, 96), (2, 256, 64), (2, 256, 256), (1, 512, 128),
-                                           (1, 512, 512)])
+@pytest.mark.parametrize("ncta,nthr,seg,shares", [
+    (1, 8, 8, 1), (5, 24, 8, 1), (16, 32, 16, 1), (16, 32, 32, 1), (3, 96, 96, 1), (3, 96, 96, 3),
+    (2, 256, 64, 1), (2, 256, 64, 2), (2, 256, 256, 1), (2, 256, 256, 4), (2, 192, 192, 2),
+    (1, 512, 128, 1), (1, 512, 512, 1), (1, 512, 512, 8)])
 @pytest.mark.parametrize("mode", ["fp32", "mixed", "fp64"])
-def test_sums_are_as_close_as_in_64_bits(probe, mode, ncta, nthr, seg, power):
+def test_sums_are_as_close_as_in_64_bits(probe, mode, ncta, nthr, seg, shares, power):
     """Thread sums of 44 bits whose totals fit 53 bits: FP64 additions give the
     exact sum in every order, and so must the reduction.  With a power, 28 bits
     times 2^99, in all warps or every other one: no thread sum exceeds FP32's
@@ -63,7 +64,7 @@ def test_sums_are_as_close_as_in_64_bits(probe, mode, ncta, nthr, seg, power):
     partial = torch.zeros(n // seg + 32, dtype=torch.float64, device="cuda")
     state = torch.zeros(probe.probe_state_bytes(), dtype=torch.uint8, device="cuda")
     for _ in range(2):   # the second run finds the ticket reset
-        assert probe.probe_reduce(TYPES[mode], ncta, nthr, seg, h.data_ptr(), l.data_ptr(),
+        assert probe.probe_reduce(TYPES[mode], ncta, nthr, seg, shares, h.data_ptr(), l.data_ptr(),
                                   partial.data_ptr(), state.data_ptr(),
                                   torch.cuda.current_stream().cuda_stream) == 0
         o = probe.probe_bb_offset()
