@@ -253,11 +253,8 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 // conversions to double took about 100 (2048^2 x 4, double-float: draw 2040 ->
 // 1421 us; 2048^2 x 2 FP32 915 -> 530 us).  Error of the noise against 64-bit
 // arithmetic as before (with the transforms, 2048^2 FP64: 5.35e-16, now 5.30e-16).
-__device__ __forceinline__ void normal_pair(const double* __restrict__ tab,
-                                            unsigned long long seed, uint32_t j, double& x0,
-                                            double& x1) {
-  const uint4 w = philox4x32_10(make_uint4(j, 0u, 0u, 0u),
-                                make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
+__device__ __forceinline__ void normals_of(const double* __restrict__ tab, uint4 w, double& x0,
+                                           double& x1) {
   // u1 = m 2^-53 (m odd), and z, k
   const unsigned long long m =
       ((((unsigned long long)(w.x >> 6) << 26) | (w.y >> 6)) << 1) | 1ull;
@@ -291,6 +288,14 @@ __device__ __forceinline__ void normal_pair(const double* __restrict__ tab,
   const double cm = q * fma(fma(-1.0 / 720.0, q, 1.0 / 24.0), q, -0.5);   // cos - 1
   x0 = rad * (cs.x + fma(cs.x, cm, fma(-cs.y, sn, lo.x)));
   x1 = rad * (cs.y + fma(cs.y, cm, fma(cs.x, sn, lo.y)));
+}
+__device__ __forceinline__ void normal_pair(const double* __restrict__ tab,
+                                            unsigned long long seed, uint32_t j, double& x0,
+                                            double& x1) {
+  normals_of(tab,
+             philox4x32_10(make_uint4(j, 0u, 0u, 0u),
+                           make_uint2((uint32_t)seed, (uint32_t)(seed >> 32))),
+             x0, x1);
 }
 
 // ---------------------------------------------------------------------------

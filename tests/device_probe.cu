@@ -4,6 +4,7 @@
 #include <type_traits>
 
 #include "cg_common.cuh"
+#include "cg_noise.h"
 
 using namespace cgf;
 
@@ -31,7 +32,23 @@ __global__ void k_reduce(const double* hi, const double* lo, double* partial, Cg
               });
 }
 
+__global__ void k_normals(const double* tab, const uint4* words, int n, double2* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) normals_of(tab, words[i], out[i].x, out[i].y);
+}
+
 }  // namespace
+
+// Normals of n Philox outputs; tab: device room for probe_noise_entries() doubles.
+extern "C" int probe_normals(double* tab, const void* words, int n, void* out, void* stream) {
+  cudaStream_t s = (cudaStream_t)stream;
+  const std::vector<double> t = noise_tables();
+  cudaError_t e = cudaMemcpy(tab, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return (int)e;
+  k_normals<<<(n + 127) / 128, 128, 0, s>>>(tab, (const uint4*)words, n, (double2*)out);
+  return (int)cudaGetLastError();
+}
+extern "C" int probe_noise_entries() { return kNoiseEntries; }
 
 extern "C" int probe_reduce(int type, int ncta, int nthr, int seg, int shares,
                             const double* hi, const double* lo, double* partial, void* state, void* stream) {

@@ -22,6 +22,7 @@ def probe(tmp_path_factory):
     subprocess.run([_build._nvcc(), *_build.ARCH, *_build.FLAGS, "-shared", "-o", so, src], check=True)
     lib = ctypes.CDLL(so)
     lib.probe_reduce.argtypes = [ctypes.c_int] * 5 + [ctypes.c_void_p] * 5
+    lib.probe_normals.argtypes = [ctypes.c_void_p] * 2 + [ctypes.c_int] + [ctypes.c_void_p] * 2
     return lib
 
 
@@ -70,3 +71,43 @@ def test_sums_are_as_close_as_in_64_bits(probe, mode, ncta, nthr, seg, shares, p
         o = probe.probe_bb_offset()
         bb = state.cpu()[o:o + 8].view(torch.float64).item()
         assert bb == float(exact)
+
+
+def test_normals_at_the_edges(probe):
+    """Box-Muller on the tables against extended precision: smallest and largest
+    uniforms, both sides of every power of two, every interval of the logarithm
+    and every sector of the angle, and random words.  Bound: half an ulp each for
+    the argument's two additions and the root (2^-52 of the radius in all, with the
+    halving of the root), 2^-53 for the unit vector and 2^-53 for the product:
+    2^-51 of the radius."""
+    rng = np.random.default_rng(5)
+    u1, u2 = [0, 1, 2, 2 ** 52 - 1, 2 ** 52 - 2], [0, 1, 2 ** 52 - 1]   # u = (k + 1/2) 2^-52
+    for p in range(52):
+        u1 += [2 ** p - 1, 2 ** p, 2 ** p + 1]
+    for i in range(256):
+        for p in (51, 50, 40, 8):   # first value of interval i at that power of two
+            k = 2 ** p + (i << p >> 8)
+            u1 += [k - 1, k, k + 1]
+        k = i << 44
+        u2 += [abs(k - 1), k, k + 1, k + 2 ** 43 - 1, k + 2 ** 43, k + 2 ** 43 + 1]
+    u1, u2 = np.array(u1, np.int64), np.array(u2, np.int64)
+    n = 60000
+    a = np.concatenate([u1, rng.integers(0, 2 ** 52, n)])
+    b = np.concatenate([rng.choice(u2, u1.size), rng.integers(0, 2 ** 52, n)])
+    a = np.concatenate([a, rng.integers(0, 2 ** 52, u2.size)])
+    b = np.concatenate([b, u2])
+    assert a.min() >= 0 and max(a.max(), b.max()) < 2 ** 52
+    low = rng.integers(0, 64, (a.size, 4))   # the six bits of a word that are not used
+    words = np.stack([a >> 26, a & (2 ** 26 - 1), b >> 26, b & (2 ** 26 - 1)], 1) << 6 | low
+    dw = torch.from_numpy(words.astype(np.uint32).view(np.int32)).cuda()
+    tab = torch.empty(probe.probe_noise_entries(), dtype=torch.float64, device="cuda")
+    out = torch.empty((a.size, 2), dtype=torch.float64, device="cuda")
+    assert probe.probe_normals(tab.data_ptr(), dw.data_ptr(), a.size, out.data_ptr(),
+                               torch.cuda.current_stream().cuda_stream) == 0
+    L = np.longdouble
+    assert np.finfo(L).nmant >= 63
+    v = lambda k: (k.astype(L) + L(0.5)) / L(2 ** 52)   # noqa: E731
+    rad = np.sqrt(L(-2) * np.where(a < 2 ** 51, np.log(v(a)), np.log1p(v(a) - L(1))))
+    th = L(2) * np.arccos(L(-1)) * v(b)
+    err = np.abs(out.cpu().numpy().astype(L) - np.stack([rad * np.cos(th), rad * np.sin(th)], 1))
+    assert np.max(err / rad[:, None]) <= 2.0 ** -51
