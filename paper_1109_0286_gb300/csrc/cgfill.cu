@@ -362,8 +362,9 @@ struct Ctx {
   const T* gwx = nullptr;
   const T* gwn = nullptr;
   // programmatic dependent launches: a pass may start while the kernel before
-  // it in the stream still runs.  Off for the first pass after something that
-  // is no kernel of the same stream (an event, a conditional node), and for
+  // it in the stream still runs.  Off for the first pass after an event wait or
+  // a conditional node (a copy, a memset or a graph launch before it in the
+  // stream is waited for as usual), and for
   // FP64 beyond 2^17 pixels: those passes are long against the launch gap, and
   // CTAs that start early share an SM's FP64 pipe unevenly (512^2 165 without,
   // 185 us per iteration with; 64^2 75 and 73; FP32 256^2 x 16 61 and 57;
@@ -930,7 +931,7 @@ cudaError_t mixed_start(const Ctx<float>& lo, const Ctx<df>& hi, cudaStream_t s,
 // After a mixed loop: fold anything left (breakdown / limits), report the
 // true residual, and add the FP32 iterations to the high-precision counts.
 cudaError_t mixed_finish(const Ctx<float>& lo, const Ctx<df>& hi, cudaStream_t s) {
-  CE(row<df>(hi, s, OP_U64_UPD, SC_NONE, false, true, SKIP_DONE));
+  CE(row<df>(no_pdl(hi), s, OP_U64_UPD, SC_NONE, false, true, SKIP_DONE));
   CE(col<df>(hi, s, 0, SKIP_DONE));
   CE(row<df>(hi, s, OP_RES, SC_RES, true, false, SKIP_DONE));
   ++*lo.launches;
@@ -2907,7 +2908,7 @@ fill_status group_realize_t(fill_group* g, const void* const* d, const uint64_t*
   }
   fs = group_fork_join<T>(g, [&](GroupClass& c) -> cudaError_t {
     Ctx<T> cx_ = gctx<T>(g, c);
-    CE(vec<T>(cx_, c.cs, VOP_ASSEMBLE, SC_NONE, false));
+    CE(vec<T>(no_pdl(cx_), c.cs, VOP_ASSEMBLE, SC_NONE, false));
     ++g->launches;
     k_gather_states<T><<<(c.ninst + 127) / 128, 128, 0, c.cs>>>(cx_.desc, c.ninst, c.st);
     CE(cudaGetLastError());
