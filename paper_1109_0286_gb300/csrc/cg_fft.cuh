@@ -13,11 +13,13 @@
 // correctly rounded values (stw_* in cg_types.h), or (E = 16 columns in FP32)
 // from three of the table's entries and complex products (TAB = false).
 //
-// E trades the exchanges against the length of a thread's instruction chain:
-// E = 16 for the large FP32 and double-float grids, which fill the chip and
-// are bound by issue and shared-memory traffic; E = 8 for small ones, where a
-// pass is one wave and its duration is the latency of one thread; E = 4 in
-// FP64, where an instruction occupies the FP64 pipe for 64 cycles per warp.
+// E trades the exchanges against the length of a thread's instruction chain
+// (row_le and col_le in cg_types.h): 16 on long transforms, whose grids fill the
+// chip and are bound by issue and shared-memory traffic; 8 and then 4 on shorter
+// ones, where a pass is one wave and its duration is the latency of one thread,
+// the earlier the longer an instruction takes (FP32: 4 up to 64 points in rows
+// and 128 in columns; double-float 256 and 512; FP64, where an instruction
+// occupies its pipe for 64 cycles per warp, 512 and 1024).
 #pragma once
 #include "cg_common.cuh"
 

@@ -32,7 +32,7 @@ struct Launcher {
 
 template <typename T>
 size_t Launch<T>::row_smem(int log_l, int rows) {
-  // FFT areas / transposed tile, then the mask words (8 bytes per 32 pixels)
+  // exchange areas, then the mask words (8 bytes per 32 pixels)
   const size_t nw = (size_t(1) << log_l) / 16;
   return row_main_bytes<T>(log_l, rows) + size_t(rows) * nw * sizeof(uint2);
 }
