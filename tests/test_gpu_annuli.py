@@ -44,12 +44,12 @@ def test_only_the_present_set_is_held(mode):
 
 @pytest.mark.parametrize("mode", ["fp32", "mixed"])
 def test_kernels_in_turns(mode):
-    """A batch whose spectra exceed 512 MB for all annuli takes them in turns;
+    """A batch whose spectra exceed 1 GB for all annuli takes them in turns;
     every map as in a plan of its own, whose annuli run together."""
     n, nk = 2048, 9
-    batch = 2 if mode == "mixed" else 4
+    batch = 4 if mode == "mixed" else 8
     one = batch * 2 * n * (n // 2 + 1) * ELEM[mode]
-    assert nk * one > 2 ** 29 >= nk * one // batch
+    assert nk * one > 2 ** 30 >= nk * one // batch
     obs, many = make(n, mode, batch)
     _, single = make(n, mode)
     for p in (many, single):
